@@ -210,19 +210,78 @@ cudaError_t launch_plane_copies(const GeomDev &g, const float *vol, const double
 // ---------------------------------------------------------------------------
 // y = A x.
 //
-// One thread walks A_VR rays of one detector column: same view and u,
+// One thread walks VR rays of one detector column: same view and u,
 // consecutive v.  On a flat detector those rays share d_x, d_y and the cross
 // product, hence the dominant axis and the in-plane coordinate f_b(p) of every
 // plane; only z differs, f_z(p, v) = cz + gz(v) (p - c_a - S_a/vox), with
 // gz(v) = v dzv / d_a.  Per plane the thread interpolates along b once per
-// z-row it needs and keeps a two-row window (rows zc, zc+1) that slides up as
-// v increases (z is monotone in v along a column), so most rays cost one new
-// row pair instead of two.  Lanes are consecutive u of one detector row
+// z-row it needs.  Lanes are consecutive u of one detector row
 // segment and walk a warp-uniform plane range, so a warp's loads of one plane
 // fall in a few consecutive sectors.  Samples outside a ray's own range have
 // their row / column clamped into the zero border and add exactly zero.
 // ---------------------------------------------------------------------------
 constexpr int A_BLOCK = 128;
+
+// What the rays iv0 .. iv0 + VR - 1 of one detector column share.
+struct ColumnA {
+    bool xdom;            // planes along x
+    int Na, Nb, p0, p1;   // planes, cells per plane row, warp-uniform inclusive plane range
+    float ca, gb, fbc;    // central plane; in-plane coordinate: slope per plane, value at ca
+    float Sv;             // source coordinate along the axis, in voxels
+    float gz0, gz_step;   // z slope of the first ray, and its change from ray to ray
+    float dxy2, inv_da, dzv;
+};
+
+// All lanes of the warp call it; lanes that are not live do not widen the range.
+template <int VR>
+__device__ __forceinline__ ColumnA column_A(const GeomDev &g, int s, int iv0, int iu, bool live)
+{
+    const float4 *vp = reinterpret_cast<const float4 *>(g.viewA + s);
+    const float4 a = __ldg(vp), b = __ldg(vp + 1);   // (dx0, dxu, dy0, dyu), (dzv, crossu, sx, sy)
+    const float u = (float(iu) - g.cu) * g.du;
+    const float dx = fmaf(u, a.y, a.x);
+    const float dy = fmaf(u, a.w, a.z);
+    const float cross = u * b.y;
+    ColumnA c;
+    c.xdom = fabsf(dx) >= fabsf(dy);
+    const float da = c.xdom ? dx : dy;
+    c.inv_da = 1.0f / da;
+    c.Na = c.xdom ? g.nx : g.ny;
+    c.Nb = c.xdom ? g.ny : g.nx;
+    c.ca = c.xdom ? g.cx : g.cy;
+    c.gb = (c.xdom ? dy : dx) * c.inv_da;
+    const float cterm = cross * c.inv_da * g.inv_vox;
+    c.fbc = c.xdom ? g.cy - cterm : g.cx + cterm;
+    c.Sv = (c.xdom ? b.z : b.w) * g.inv_vox;
+    c.gz_step = g.dv * b.x * c.inv_da;
+    c.gz0 = (float(iv0) - g.cv) * c.gz_step;
+    c.dxy2 = fmaf(dx, dx, dy * dy);
+    c.dzv = b.x;
+
+    // plane range: the b range of the column met with the planes on which
+    // any of its rays is inside the grid in z, then joined over the warp
+    int p0 = 0, p1 = c.Na - 1;
+    clip_planes(c.fbc, c.gb, -1.0f, float(c.Nb), c.ca, c.Na, p0, p1);
+    const float gzl = (float(min(iv0 + VR - 1, g.nv - 1)) - g.cv) * c.gz_step;
+    clip_planes_run(fmaf(-c.Sv, c.gz0, g.cz), c.gz0, fmaf(-c.Sv, gzl, g.cz), gzl, -1.0f, float(g.nz), c.ca, c.Na, p0,
+                    p1);
+    if (!live) {
+        p0 = c.Na;
+        p1 = -1;
+    }
+    c.p0 = __reduce_min_sync(0xffffffffu, p0);
+    // lanes of one warp can differ in axis (views near 45 degrees); each stays
+    // inside its own plane count
+    c.p1 = min(__reduce_max_sync(0xffffffffu, p1), c.Na - 1);
+    return c;
+}
+
+// Step length vox |d| / |d_a| of ray iv of a column.
+__device__ __forceinline__ float step_weight(const GeomDev &g, const ColumnA &c, int iv)
+{
+    const float dz = (float(iv) - g.cv) * g.dv * c.dzv;
+    return g.vox * sqrtf(fmaf(dz, dz, c.dxy2)) * fabsf(c.inv_da);
+}
 
 // b-interpolated value of one plane row: (1 - wb) V[b0] + wb V[b0+1], read as
 // two floats or as one packed bf16 pair
@@ -238,135 +297,222 @@ __device__ __forceinline__ float row_lerp(const float *p, float wb)
     return fmaf(wb, v1 - v0, v0);
 }
 
-// plane-loop unroll (tuning): 2 for FP32 copies, 4 for bf16 pairs (measured
-// at 256^3 with 16 rays per thread and 64 registers: 5.31 and 5.74 ms; unrolling the FP32
-// loop by 1 or 4 took 8.44 and 5.63 ms, the bf16 loop by 2 8.76 ms); the
-// rays per thread, A_VR, are in the shared header
-#ifndef CT_A_PUNROLL
-#define CT_A_PUNROLL 2
-#endif
-#ifndef CT_A_PUNROLL_BF
-#define CT_A_PUNROLL_BF 4
-#endif
-constexpr int kAPlaneUnroll = CT_A_PUNROLL;
-constexpr int kAPlaneUnrollBF = CT_A_PUNROLL_BF;
-// resident blocks per SM that ptxas sizes the registers for (tuning): 5 for
-// FP32 copies (96 registers), 4 for bf16 pairs (128).  At 256^3 these took
-// 5.03 and 5.41 ms, against 5.29 and 5.73 ms with ptxas's own choice of 64
-// registers (8 blocks); 6 or 7 blocks gave 5.07 / 5.04 ms (FP32), 9 blocks
-// (56 registers) 8.5 ms.
-constexpr int kAMinBlocks = 5;
-constexpr int kAMinBlocksBF = 4;
+// One ray's sample on plane p from its plane row: z interpolated between two
+// rows of the copy, or (FLAT: a 2D scan, whose rays stay in its one slice) the
+// row itself.
+template <bool FLAT, bool BF>
+__device__ __forceinline__ float plane_sample(const GeomDev &g, const float *rowp, int zstride, float wb, float fz)
+{
+    if (FLAT) return row_lerp<BF>(rowp, wb);
+    const float z0f = floorf(fz);
+    const float *r = rowp + min(max(int(z0f), -PAD_A), g.nz) * zstride;
+    const float lo = row_lerp<BF>(r, wb), hi = row_lerp<BF>(r + zstride, wb);
+    return fmaf(fz - z0f, hi - lo, lo);
+}
 
-template <int VR, bool WINDOW, bool ZCLAMP, bool BF>
-__global__ void __launch_bounds__(A_BLOCK, BF ? kAMinBlocksBF : kAMinBlocks) joseph_A_kernel(GeomDev g, const float *__restrict__ Xc,
-                                                           const float *__restrict__ Yc,
-                                                           float *__restrict__ y, SinoLayout lay,
+// The walk of detectors with one row (2D scans above all).  A scan has few
+// rays (8550 of them for 64 x 64 pixels and 90 views: two warps an SM), so
+// what bounds it is one ray's chain of loads: `split` (1, 2, 4 or 8) of a
+// block's 8 warps share the planes of a ray and add their sums.  One warp a
+// ray and two interpolated rows took 15.9 us for that scan, this 8.2 us; 256 x
+// 256 with 360 views 69.9 -> 57.7 us, 512 x 512 with 720 views 321 -> 227 us.
+template <bool FLAT, bool BF>
+__global__ void __launch_bounds__(256) joseph_A_row_kernel(GeomDev g, const float *__restrict__ Xc,
+                                                           const float *__restrict__ Yc, float *__restrict__ y,
+                                                           SinoLayout lay, int split,
                                                            const int *__restrict__ stop)
 {
+    if (stop && *stop) return;
+    __shared__ float part[8][32];
+    const int w = threadIdx.y, wp = w % split;   // the warp's share of its rays' planes
+    const int lane_u = (blockIdx.x * (8 / split) + w / split) * 32 + threadIdx.x;
+    const int s = blockIdx.z;
+    const bool live = lane_u < g.nu;
+    const ColumnA c = column_A<1>(g, s, 0, min(lane_u, g.nu - 1), live);
+    const int pitch = c.xdom ? g.pitchX : g.pitchY;
+    const int zstride = c.Na * pitch;
+    // (z = 0, plane 0, b = 0) in the padded copy
+    const float *__restrict__ base = (c.xdom ? Xc : Yc) + PAD_A * zstride + PAD_A;
+    float acc = 0.0f;
+#pragma unroll 4
+    for (int p = c.p0 + wp; p <= c.p1; p += split) {
+        const float pm = float(p) - c.ca;
+        const float fb = fmaf(pm, c.gb, c.fbc);
+        const float b0f = floorf(fb);
+        const int b0 = min(max(int(b0f), -PAD_A), c.Nb);
+        acc += plane_sample<FLAT, BF>(g, base + p * pitch + b0, zstride, fb - b0f, fmaf(c.gz0, pm - c.Sv, g.cz));
+    }
+    part[w][threadIdx.x] = acc;
+    __syncthreads();
+    if (wp > 0 || !live) return;
+    for (int i = 1; i < split; ++i) acc += part[w + i][threadIdx.x];
+    store_sino(y, lay, s, 0, lane_u, acc * step_weight(g, c, 0));
+}
+
+// ---------------------------------------------------------------------------
+// The walk of cone-beam detectors, two neighbouring rays an instruction.
+// What bounds the walk is issue slots (76 % busy) and, for its floors and
+// float-to-int conversions, the XU pipe (66 %: each takes it 8 cycles a
+// warp).  sm_103a's packed FP32 operations (add, sub, fma .f32x2) do the
+// arithmetic of two values in one issue slot, at the same rate a value.  The
+// floor comes from them too: t = z + 1.5 2^23 rounded down holds floor(z) in
+// its low mantissa bits, so a row's address is one wide multiply-add of t's
+// bits (the constant's share is folded into the base pointer) and nothing
+// runs on the XU pipe.
+//
+// WINDOW: every ray of a column moves up at most one z row per detector row
+// (a_window), so the low row of a sample is the low or the high row of the
+// ray before: one new row a ray instead of two.
+//
+// Needs |z| < 2^22: the copies' grid takes 65531 slices at most, and the clamped
+// form bounds z before the floor.  The values and their rounding are those of a
+// walk of one ray at a time.
+// ---------------------------------------------------------------------------
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float &lo, float &hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 add2_down(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("add.rm.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+constexpr float FLOOR_MAGIC = 12582912.0f;   // 1.5 2^23
+constexpr unsigned FLOOR_MAGIC_BITS = 0x4b400000u;
+
+// Registers for 4 resident blocks (128) and a plane loop unrolled by 4: at
+// 256^3 4.32 ms (bf16 copies 4.41 ms); unrolled by 2, 4.38 ms (4.57 ms); 5
+// blocks unrolled by 2, 4.42 ms; 6 and 8 blocks, 4.80 and 5.51 ms (ptxas then
+// keeps fewer row loads in flight); 8 rays a thread, 4.65-4.74 ms.  The plain
+// walk over a two-row window took 5.04 ms (bf16 5.41 ms).  Left after it:
+// 12.1 instructions a sample (16.8 before), the FMA pipe 53 % and issue 56 %
+// busy, the rest latency of the row loads (a third of them miss L1).
+constexpr int kAPlaneUnroll = 4;
+constexpr int kAMinBlocks = 4;
+
+template <int VR, bool WINDOW, bool ZCLAMP, bool BF>
+__global__ void __launch_bounds__(A_BLOCK, kAMinBlocks)
+    joseph_A_pairs_kernel(GeomDev g, const float *__restrict__ Xc, const float *__restrict__ Yc,
+                          float *__restrict__ y, SinoLayout lay, const int *__restrict__ stop)
+{
+    static_assert(VR % 2 == 0, "rays are walked in pairs");
     if (stop && *stop) return;
     const int lane_u = blockIdx.x * 32 + (threadIdx.x & 31);
     const int iv0 = (blockIdx.y * (A_BLOCK / 32) + (threadIdx.x >> 5)) * VR;
     const int s = blockIdx.z;
     const bool live = lane_u < g.nu && iv0 < g.nv;
-    const int iu = min(lane_u, g.nu - 1);
-    const int ivl = min(iv0 + VR - 1, g.nv - 1);
+    const ColumnA c = column_A<VR>(g, s, iv0, min(lane_u, g.nu - 1), live);
+    const int pitch = c.xdom ? g.pitchX : g.pitchY;
+    const int zstride = c.Na * pitch;
+    const unsigned zs4 = unsigned(zstride) * 4u;
+    // (z = 0, plane 0, b = 0), less the floor constant's share of a row address
+    const char *__restrict__ base = reinterpret_cast<const char *>(c.xdom ? Xc : Yc) +
+                                    4 * (ptrdiff_t(PAD_A) * zstride + PAD_A) -
+                                    ptrdiff_t(FLOOR_MAGIC_BITS) * ptrdiff_t(zs4);
 
-    // geometry shared by the column's rays
-    const float4 *vp = reinterpret_cast<const float4 *>(g.viewA + s);
-    const float4 a = __ldg(vp), b = __ldg(vp + 1);   // (dx0, dxu, dy0, dyu), (dzv, crossu, sx, sy)
-    const float u = (float(iu) - g.cu) * g.du;
-    const float dx = fmaf(u, a.y, a.x);
-    const float dy = fmaf(u, a.w, a.z);
-    const float cross = u * b.y;
-    const bool xdom = fabsf(dx) >= fabsf(dy);
-    const float da = xdom ? dx : dy;
-    const float inv_da = 1.0f / da;
-    const int Na = xdom ? g.nx : g.ny;
-    const int Nb = xdom ? g.ny : g.nx;
-    const float ca = xdom ? g.cx : g.cy;
-    const float gb = (xdom ? dy : dx) * inv_da;
-    const float cterm = cross * inv_da * g.inv_vox;
-    const float fbc = xdom ? g.cy - cterm : g.cx + cterm;
-    const float Sv = (xdom ? b.z : b.w) * g.inv_vox;   // source coordinate along the axis, in voxels
-    const float gz_step = g.dv * b.x * inv_da;           // d gz / d iv
-    const float gz0 = (float(iv0) - g.cv) * gz_step;     // gz of the first ray
-
-    // plane range: the b range of the column met with the planes on which
-    // any of its rays is inside the grid in z, then joined over the warp
-    int p0 = 0, p1 = Na - 1;
-    clip_planes(fbc, gb, -1.0f, float(Nb), ca, Na, p0, p1);
-    {
-        const float gzl = (float(ivl) - g.cv) * gz_step;
-        clip_planes_run(fmaf(-Sv, gz0, g.cz), gz0, fmaf(-Sv, gzl, g.cz), gzl, -1.0f, float(g.nz), ca, Na, p0, p1);
-    }
-    if (!live) {  // idle lanes do not widen the warp's range
-        p0 = Na;
-        p1 = -1;
-    }
-    p0 = __reduce_min_sync(0xffffffffu, p0);
-    p1 = __reduce_max_sync(0xffffffffu, p1);
-    // lanes of one warp can differ in axis (views near 45 degrees); each stays
-    // inside its own plane count
-    p1 = min(p1, Na - 1);
-
-    const float *__restrict__ base = xdom ? Xc : Yc;
-    const int pitch = xdom ? g.pitchX : g.pitchY;
-    const int zstride = Na * pitch;
-    const int bmax = Nb, zmax = g.nz;
-
-    float acc[VR];
+    f32x2 acc[VR / 2];
 #pragma unroll
-    for (int i = 0; i < VR; ++i) acc[i] = 0.0f;
+    for (int i = 0; i < VR / 2; ++i) acc[i] = pack2(0.0f, 0.0f);
+    const f32x2 magic = pack2(FLOOR_MAGIC, FLOOR_MAGIC);
 
-#pragma unroll (BF ? kAPlaneUnrollBF : kAPlaneUnroll)
-    for (int p = p0; p <= p1; ++p) {
-        const float pm = float(p) - ca;
-        const float fb = fmaf(pm, gb, fbc);
+#pragma unroll kAPlaneUnroll
+    for (int p = c.p0; p <= c.p1; ++p) {
+        const float pm = float(p) - c.ca;
+        const float fb = fmaf(pm, c.gb, c.fbc);
         const float b0f = floorf(fb);
         const float wb = fb - b0f;
-        const int b0 = min(max(int(b0f), -PAD_A), bmax);
-        // element offset of (z = 0, plane p, b0) in the padded copy
-        const float *rowp = base + (PAD_A * Na + p) * pitch + b0 + PAD_A;
-        const float q = pm - Sv;
-        const float fz0 = fmaf(gz0, q, g.cz);   // z of the first ray
-        const float dzr = gz_step * q;          // z step from ray to ray
-        float lo_prev = 0.0f, hi_prev = 0.0f;
-        int z_prev = 0;
+        const int b0 = min(max(int(b0f), -PAD_A), c.Nb);
+        const char *rowp = base + 4 * ptrdiff_t(p * pitch + b0);
+        const float q = pm - c.Sv;
+        const float fz0 = fmaf(c.gz0, q, g.cz);   // z of the first ray
+        const float dzr = c.gz_step * q;          // z step from ray to ray
+        const f32x2 fz02 = pack2(fz0, fz0), dzr2 = pack2(dzr, dzr), wb2 = pack2(wb, wb);
+        float lo_prev = 0.0f, hi_prev = 0.0f, t_prev = 0.0f;
 #pragma unroll
-        for (int i = 0; i < VR; ++i) {
-            const float fz = fmaf(float(i), dzr, fz0);
-            const float z0f = floorf(fz);
-            const float wz = fz - z0f;
-            int z0 = ZCLAMP ? min(max(int(z0f), -PAD_A), zmax) : int(z0f);
-            if (!ZCLAMP && !CT_IN_BOUNDS(g, z0 >= -PAD_A && z0 <= zmax + PAD_A - 2, BS_A_Z, s, z0)) z0 = -PAD_A;
-            if (WINDOW && i > 0) (void)CT_IN_BOUNDS(g, z0 == z_prev || z0 == z_prev + 1, BS_A_WINDOW, s, z0 - z_prev);
-            const float *r = rowp + (z0 + 1) * zstride;
-            const float hi = row_lerp<BF>(r, wb);
-            float lo;
-            if (!WINDOW || i == 0) {
-                lo = row_lerp<BF>(r - zstride, wb);
-            } else {
-                // z0 is z_prev or z_prev + 1: the low row is one of the previous rows
-                lo = z0 == z_prev ? lo_prev : hi_prev;
+        for (int i = 0; i < VR; i += 2) {
+            f32x2 fz = fma2(pack2(float(i), float(i + 1)), dzr2, fz02);
+            if (ZCLAMP) {   // a sample off the grid takes both rows from the zero border
+                float f0, f1;
+                unpack2(fz, f0, f1);
+                fz = pack2(fminf(fmaxf(f0, -float(PAD_A)), float(g.nz)), fminf(fmaxf(f1, -float(PAD_A)), float(g.nz)));
             }
-            acc[i] += fmaf(wz, hi - lo, lo);
-            lo_prev = lo;
-            hi_prev = hi;
-            z_prev = z0;
+            const f32x2 t = add2_down(fz, magic);
+            const f32x2 wz = sub2(fz, sub2(t, magic));
+            float t0, t1;
+            unpack2(t, t0, t1);
+            unsigned m0 = __float_as_uint(t0), m1 = __float_as_uint(t1);   // floor(z) + FLOOR_MAGIC_BITS
+            const int z0 = int(m0 - FLOOR_MAGIC_BITS), z1 = int(m1 - FLOOR_MAGIC_BITS);   // checked builds only
+            if (!CT_IN_BOUNDS(g, z0 >= -PAD_A && z0 <= g.nz + PAD_A - 2, BS_A_Z, s, z0)) m0 = FLOOR_MAGIC_BITS - PAD_A;
+            if (!CT_IN_BOUNDS(g, z1 >= -PAD_A && z1 <= g.nz + PAD_A - 2, BS_A_Z, s, z1)) m1 = FLOOR_MAGIC_BITS - PAD_A;
+            if (WINDOW) {
+                const int zp = int(__float_as_uint(t_prev) - FLOOR_MAGIC_BITS);
+                (void)CT_IN_BOUNDS(g, z1 == z0 || z1 == z0 + 1, BS_A_WINDOW, s, z1 - z0);
+                if (i > 0) (void)CT_IN_BOUNDS(g, z0 == zp || z0 == zp + 1, BS_A_WINDOW, s, z0 - zp);
+                (void)zp;
+            }
+            const float *r0 = reinterpret_cast<const float *>(rowp + (unsigned long long)m0 * zs4);
+            const float *r1 = reinterpret_cast<const float *>(rowp + (unsigned long long)m1 * zs4);
+            // high rows of the two samples
+            f32x2 hi;
+            if (BF) {
+                const uint32_t w0 = __ldg(reinterpret_cast<const uint32_t *>(r0 + zstride));
+                const uint32_t w1 = __ldg(reinterpret_cast<const uint32_t *>(r1 + zstride));
+                const f32x2 v0 = pack2(bf16_lo(w0), bf16_lo(w1)), v1 = pack2(bf16_hi(w0), bf16_hi(w1));
+                hi = fma2(wb2, sub2(v1, v0), v0);
+            } else {
+                const f32x2 v0 = pack2(__ldg(r0 + zstride), __ldg(r1 + zstride));
+                const f32x2 v1 = pack2(__ldg(r0 + zstride + 1), __ldg(r1 + zstride + 1));
+                hi = fma2(wb2, sub2(v1, v0), v0);
+            }
+            float h0, h1, lo0, lo1;
+            unpack2(hi, h0, h1);
+            if (WINDOW) {
+                lo0 = i == 0 ? row_lerp<BF>(r0, wb) : (t0 == t_prev ? lo_prev : hi_prev);
+                lo1 = t1 == t0 ? lo0 : h0;
+            } else {
+                lo0 = row_lerp<BF>(r0, wb);
+                lo1 = row_lerp<BF>(r1, wb);
+            }
+            const f32x2 lo = pack2(lo0, lo1);
+            acc[i / 2] = add2(acc[i / 2], fma2(wz, sub2(hi, lo), lo));
+            lo_prev = lo1;
+            hi_prev = h1;
+            t_prev = t1;
         }
     }
     if (!live) return;
-    const float dxy2 = fmaf(dx, dx, dy * dy);
 #pragma unroll
-    for (int i = 0; i < VR; ++i) {
-        const int iv = iv0 + i;
-        if (iv < g.nv) {
-            const float v = (float(iv) - g.cv) * g.dv;
-            const float dz = v * b.x;
-            const float w = g.vox * sqrtf(fmaf(dz, dz, dxy2)) * fabsf(inv_da);
-            store_sino(y, lay, s, iv, iu, acc[i] * w);
-        }
+    for (int i = 0; i < VR; i += 2) {
+        float a0, a1;
+        unpack2(acc[i / 2], a0, a1);
+        if (iv0 + i < g.nv) store_sino(y, lay, s, iv0 + i, lane_u, a0 * step_weight(g, c, iv0 + i));
+        if (iv0 + i + 1 < g.nv) store_sino(y, lay, s, iv0 + i + 1, lane_u, a1 * step_weight(g, c, iv0 + i + 1));
     }
 }
 
@@ -374,23 +520,26 @@ template <bool BF>
 static void launch_joseph_A_t(const GeomDev &g, const float *Xc, const float *Yc, float *y, SinoLayout lay,
                               const int *stop, cudaStream_t st)
 {
-    constexpr int WPB = A_BLOCK / 32;
+    constexpr int WPB = A_BLOCK / 32, VR = A_VR;
     if (g.nv == 1) {
-        dim3 grid((g.nu + 31) / 32, (g.nv + WPB - 1) / WPB, g.n_views);
-        joseph_A_kernel<1, false, true, BF><<<grid, A_BLOCK, 0, st>>>(g, Xc, Yc, y, lay, stop);
+        // warps a ray: as many (up to 8) as keep the grid within 32 warps an SM
+        const int tiles = (g.nu + 31) / 32;
+        int split = 1;
+        while (split < 8 && size_t(tiles) * g.n_views * split * 2 <= size_t(num_sms()) * 32) split *= 2;
+        const dim3 block(32, 8), grid((tiles * split + 7) / 8, 1, g.n_views);
+        if (g.kind == CT_PARALLEL_2D)
+            joseph_A_row_kernel<true, BF><<<grid, block, 0, st>>>(g, Xc, Yc, y, lay, split, stop);
+        else
+            joseph_A_row_kernel<false, BF><<<grid, block, 0, st>>>(g, Xc, Yc, y, lay, split, stop);
         return;
     }
-    constexpr int VR = CT_A_VR;
     dim3 grid((g.nu + 31) / 32, (g.nv + WPB * VR - 1) / (WPB * VR), g.n_views);
-#ifndef CT_A_FORCE_ZCLAMP
-#define CT_A_FORCE_ZCLAMP 0
-#endif
-    if (g.a_window && g.a_zsafe && !CT_A_FORCE_ZCLAMP)
-        joseph_A_kernel<VR, true, false, BF><<<grid, A_BLOCK, 0, st>>>(g, Xc, Yc, y, lay, stop);
+    if (g.a_window && g.a_zsafe)
+        joseph_A_pairs_kernel<VR, true, false, BF><<<grid, A_BLOCK, 0, st>>>(g, Xc, Yc, y, lay, stop);
     else if (g.a_window)
-        joseph_A_kernel<VR, true, true, BF><<<grid, A_BLOCK, 0, st>>>(g, Xc, Yc, y, lay, stop);
+        joseph_A_pairs_kernel<VR, true, true, BF><<<grid, A_BLOCK, 0, st>>>(g, Xc, Yc, y, lay, stop);
     else
-        joseph_A_kernel<VR, false, true, BF><<<grid, A_BLOCK, 0, st>>>(g, Xc, Yc, y, lay, stop);
+        joseph_A_pairs_kernel<VR, false, true, BF><<<grid, A_BLOCK, 0, st>>>(g, Xc, Yc, y, lay, stop);
 }
 
 cudaError_t launch_project_A(const GeomDev &g, const float *Xc, const float *Yc, float *y,
