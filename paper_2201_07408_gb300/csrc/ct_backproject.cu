@@ -355,22 +355,6 @@ __device__ __forceinline__ ColumnView column_view(const GeomDev &g, int s, float
     return column_view(g, __ldg(vp), __ldg(vp + 1), x, y, zfirst);
 }
 
-// Lane patches.  A warp covers a patch of PA x (32/PA) columns, PA lanes
-// along the axis closer to the view's central ray (chosen per view: along x
-// when |tx| <= |ty|, i.e. when u moves more slowly with x than with y).
-// Along the central ray the projection barely moves (only the magnification
-// changes, by vox/depth per voxel); across it, u moves by M vox/du pixels per
-// lane.  The load path serves a 128-bit warp load 8 lanes at a time, and its
-// passes per load (ncu: data-pipe wavefronts per request) grow when those
-// lanes' quads spread over several 128-byte lines: of the patches measured on
-// the cone-beam scans, 4 lanes along by 2 across per group of 8 (PA = 4)
-// takes fewest (at 256^3: 5.3 passes per warp load against 6.4 with all 32
-// lanes along the ray).  The 3D kernel (voxel_B_slab_kernel) uses that patch.
-// voxel_B_kernel serves 2D scans: a block owns a 32 x 32 tile of columns
-// (ZC = 1, PA = 32: the detector is one row), and the two partial sums
-// (x-lane views and y-lane views) meet in shared memory.  The sinogram is
-// read as quads (the 2 x 2 bilinear neighbourhood), one 16-byte load (8 for
-// bf16) per voxel and view; the view table sits in shared memory.
 constexpr int B_TILE = 32;
 
 // the four bilinear neighbours of one sinogram quad entry
@@ -384,38 +368,91 @@ __device__ __forceinline__ float4 load_quad(const void *base, size_t e)
     return __ldg(static_cast<const float4 *>(base) + e);
 }
 
-// The ZC samples of one column in one view: r[k] = B's term for z = z0 + k.
-// DIFF: FP32 entries in the row-difference form, a sample is
-// w (e0 + wv (e1 - e0)) with e0 = S[v][u] + wu (S[v][u+1] - S[v][u]) and e1
-// likewise on row v+1 (five operations with the accumulation, against seven
-// from the four values); r[k] then omits the weight w, which the caller
-// folds into the accumulation.
-template <int ZC, bool BF, bool DIFF>
-__device__ __forceinline__ void column_samples(const GeomDev &g, const void *__restrict__ ypad, const ColumnView &c,
-                                               int s, int view_stride, int pitch, float (&r)[ZC])
+// A row's interpolation along u from one half of a quad entry: the row's
+// value and step (DIFF) or its two values.
+template <bool BF, bool DIFF>
+__device__ __forceinline__ float row_value(const char *half, float wu)
 {
-    int col = c.col;
-    if (!CT_IN_BOUNDS(g, unsigned(col) < unsigned(pitch), BS_B_COL, s, col)) col = 0;
-    const size_t vbase = size_t(s) * view_stride + col;
+    float2 e;
+    if (BF) {
+        const uint32_t w = __ldg(reinterpret_cast<const uint32_t *>(half));
+        e = make_float2(bf16_lo(w), bf16_hi(w));
+    } else {
+        e = __ldg(reinterpret_cast<const float2 *>(half));
+    }
+    return fmaf(wu, DIFF ? e.y : e.y - e.x, e.x);
+}
+
+// Small volumes: a run of ZC slices a thread, and `split` (1, 2, 4 or 8) of a
+// block's 8 warps share the views of their 32 columns and add their sums.  A
+// 64 x 64 slice has 4096 voxels, less than one warp an SM, and a voxel's views
+// are a chain of loads, which is what bounds it.  FLAT: 2D scans, whose one
+// detector row is half a quad.  Against one block for 32 x 32 voxels (2D) and
+// the slab kernel below (3D): 64 x 64 with 90 views 38 -> 11 us, 512 x 512 with
+// 720 views 384 -> 325 us; 32^3 47 -> 10 us, 64^3 92 -> 36 us, 96^3 138 -> 123 us.
+template <int ZC, bool FLAT, bool BF, bool DIFF>
+__global__ void __launch_bounds__(256) voxel_B_small_kernel(GeomDev g, const void *__restrict__ ypad,
+                                                            float *__restrict__ x, int split,
+                                                            const int *__restrict__ stop)
+{
+    if (stop && *stop) return;
+    __shared__ float part[ZC][8][32];
+    constexpr int ENTRY = BF ? 8 : 16;
+    const int l = threadIdx.x, w = threadIdx.y, share = w % split;
+    const int ix = blockIdx.x * 32 + l, iy = blockIdx.y * (8 / split) + w / split, iz0 = blockIdx.z * ZC;
+    const float xc = (float(min(ix, g.nx - 1)) - g.cx) * g.vox, yc = (float(min(iy, g.ny - 1)) - g.cy) * g.vox;
+    const float zfirst = (float(iz0) - g.cz) * g.vox;
+    const size_t view_stride = size_t(g.nvp) * g.pitchU;
+    float acc[ZC];
 #pragma unroll
-    for (int k = 0; k < ZC; ++k) {
-        const float fv = fmaf(float(k), c.gv, c.fv0);
-        const float v0f = floorf(fv);
-        const float wv = fv - v0f;
-        int row = int(v0f) + g.padv;
-        if (!CT_IN_BOUNDS(g, unsigned(row) < unsigned(g.nvp), BS_B_ROW, s, row)) row = 0;
-        const float4 nb = load_quad<BF>(ypad, vbase + size_t(row * pitch));
-        if (DIFF) {
-            const float e0 = fmaf(c.wu, nb.y, nb.x);
-            const float e1 = fmaf(c.wu, nb.w, nb.z);
-            r[k] = fmaf(wv, e1 - e0, e0);
-        } else {
-            const float r0 = fmaf(c.a0, nb.x, c.a1 * nb.y);
-            const float r1 = fmaf(c.a0, nb.z, c.a1 * nb.w);
-            r[k] = fmaf(wv, r1 - r0, r0);
+    for (int k = 0; k < ZC; ++k) acc[k] = 0.0f;
+#pragma unroll(ZC > 1 ? 2 : 4)
+    for (int s = share; s < g.n_views; s += split) {
+        const ColumnView c = column_view(g, s, xc, yc, zfirst);
+        if (c.skip) continue;
+        int col = c.col;
+        if (!CT_IN_BOUNDS(g, unsigned(col) < unsigned(g.pitchU), BS_B_COL, s, col)) col = 0;
+        const char *pv = static_cast<const char *>(ypad) + ENTRY * (s * view_stride + size_t(g.padv) * g.pitchU + col);
+#pragma unroll
+        for (int k = 0; k < ZC; ++k) {
+            const float fv = fmaf(float(k), c.gv, c.fv0);
+            const float v0f = FLAT ? 0.0f : floorf(fv);
+            int row = int(v0f);
+            if (!CT_IN_BOUNDS(g, unsigned(row + g.padv) < unsigned(g.nvp), BS_B_ROW, s, row + g.padv)) row = -g.padv;
+            const char *p = pv + row * (ENTRY * g.pitchU);
+            float r;
+            if (FLAT) {
+                r = row_value<BF, DIFF>(p, c.wu);
+            } else {
+                const float4 q = load_quad<BF>(p, 0);
+                r = fmaf(c.wu, DIFF ? q.y : q.y - q.x, q.x);
+                r = fmaf(fv - v0f, fmaf(c.wu, DIFF ? q.w : q.w - q.z, q.z) - r, r);
+            }
+            acc[k] = fmaf(c.w, r, acc[k]);
         }
     }
+#pragma unroll
+    for (int k = 0; k < ZC; ++k) part[k][w][l] = acc[k];
+    __syncthreads();
+    if (share > 0 || ix >= g.nx || iy >= g.ny) return;
+#pragma unroll
+    for (int k = 0; k < ZC; ++k) {
+        for (int i = 1; i < split; ++i) acc[k] += part[k][w + i][l];
+        if (iz0 + k < g.nz) x[(size_t(iz0 + k) * g.ny + iy) * g.nx + ix] = acc[k];
+    }
 }
+
+// Lane patches.  A warp covers a patch of 4 x 8 columns, 4 lanes
+// along the axis closer to the view's central ray (chosen per view: along x
+// when |tx| <= |ty|, i.e. when u moves more slowly with x than with y).
+// Along the central ray the projection barely moves (only the magnification
+// changes, by vox/depth per voxel); across it, u moves by M vox/du pixels per
+// lane.  The load path serves a 128-bit warp load 8 lanes at a time, and its
+// passes per load (ncu: data-pipe wavefronts per request) grow when those
+// lanes' quads spread over several 128-byte lines: of the patches measured on
+// the cone-beam scans, 4 lanes along by 2 across per group of 8
+// takes fewest (at 256^3: 5.3 passes per warp load against 6.4 with all 32
+// lanes along the ray).
 
 template <int ZC, bool DIFF>
 __device__ __forceinline__ void accumulate(float (&acc)[ZC], const float (&r)[ZC], float w)
@@ -424,74 +461,15 @@ __device__ __forceinline__ void accumulate(float (&acc)[ZC], const float (&r)[ZC
     for (int k = 0; k < ZC; ++k) acc[k] = DIFF ? fmaf(w, r[k], acc[k]) : acc[k] + r[k];
 }
 
-template <int ZC, bool BF, bool DIFF, int PA = 32>
-__global__ void __launch_bounds__(B_TILE *B_TILE) voxel_B_kernel(GeomDev g, const void *__restrict__ ypad,
-                                                                 float *__restrict__ x,
-                                                                 const int *__restrict__ stop)
-{
-    if (stop && *stop) return;
-    extern __shared__ float4 sviews[];   // 2 per view
-    __shared__ float tile[ZC][B_TILE][B_TILE + 1];
-    const int l = threadIdx.x, w = threadIdx.y;
-    const int tid = w * B_TILE + l;
-    const float4 *vt = reinterpret_cast<const float4 *>(g.viewB);
-    for (int i = tid; i < 2 * g.n_views; i += B_TILE * B_TILE) sviews[i] = __ldg(vt + i);
-    const int X0 = blockIdx.x * B_TILE, Y0 = blockIdx.y * B_TILE;
-    const int iz0 = blockIdx.z * ZC;
-    const float zfirst = (float(iz0) - g.cz) * g.vox;
-    // a warp covers a PA x (32/PA) patch of columns, PA lanes along the axis
-    // nearer the central ray
-    constexpr int PB = 32 / PA;
-    const int along = (w % (32 / PA)) * PA + l % PA, across = (w / (32 / PA)) * PB + l / PA;
-    const int tax = along, tay = across, tbx = across, tby = along;   // tile offsets of the two mappings
-    // column of the x-lane mapping and of the y-lane mapping (clamped into the grid;
-    // columns past the edge compute throw-away values)
-    const int ax = min(X0 + tax, g.nx - 1), ay = min(Y0 + tay, g.ny - 1);
-    const int bx = min(X0 + tbx, g.nx - 1), by = min(Y0 + tby, g.ny - 1);
-    const float axc = (float(ax) - g.cx) * g.vox, ayc = (float(ay) - g.cy) * g.vox;
-    const float bxc = (float(bx) - g.cx) * g.vox, byc = (float(by) - g.cy) * g.vox;
-    const int view_stride = g.nvp * g.pitchU;
-    const int pitch = g.pitchU;
-    __syncthreads();
-    float accA[ZC], accB[ZC];
-#pragma unroll
-    for (int k = 0; k < ZC; ++k) {
-        accA[k] = 0.0f;
-        accB[k] = 0.0f;
-    }
-    for (int s = 0; s < g.n_views; ++s) {
-        const float4 p = sviews[2 * s], q = sviews[2 * s + 1];
-        const bool xl = fabsf(p.w) <= fabsf(q.x);   // |tx| <= |ty|, uniform over the block
-        const ColumnView c = column_view(g, p, q, xl ? axc : bxc, xl ? ayc : byc, zfirst);
-        if (c.skip) continue;
-        float r[ZC];
-        column_samples<ZC, BF, DIFF>(g, ypad, c, s, view_stride, pitch, r);
-        if (xl)
-            accumulate<ZC, DIFF>(accA, r, c.w);
-        else
-            accumulate<ZC, DIFF>(accB, r, c.w);
-    }
-    // x-lane sums belong to (X0 + tax, Y0 + tay), y-lane sums to (X0 + tbx, Y0 + tby)
-#pragma unroll
-    for (int k = 0; k < ZC; ++k) tile[k][tay][tax] = accA[k];
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < ZC; ++k) tile[k][tby][tbx] += accB[k];
-    __syncthreads();
-    const int ix = X0 + l, iy = Y0 + w;
-    if (ix >= g.nx || iy >= g.ny) return;
-#pragma unroll
-    for (int k = 0; k < ZC; ++k) {
-        const int iz = iz0 + k;
-        if (iz < g.nz) x[(size_t(iz) * g.ny + iy) * g.nx + ix] = tile[k][w][l];
-    }
-}
-
 // The ZC samples of one column in one view from a per-view pointer: pv is
 // the byte address of the column's entry in the view's first unpadded row
 // (the row margin folded in), so a sample's address is one multiply-add of
-// its row index and the row pitch in bytes (the entries' forms as in
-// column_samples).
+// its row index and the row pitch in bytes.  r[k] = B's term for slice k of the
+// run.  DIFF: FP32 entries in the row-difference form, a sample is
+// w (e0 + wv (e1 - e0)) with e0 = S[v][u] + wu (S[v][u+1] - S[v][u]) and e1
+// likewise on row v+1 (five operations with the accumulation, against seven
+// from the four values); r[k] then omits the weight w, which the caller
+// folds into the accumulation.
 template <int ZC, bool BF, bool DIFF>
 __device__ __forceinline__ void column_samples_at(const GeomDev &g, int s, const char *__restrict__ pv,
                                                   const ColumnView &c, int pitch_bytes, float (&r)[ZC])
@@ -529,8 +507,8 @@ __device__ __forceinline__ void column_samples_at(const GeomDev &g, int s, const
 // 1024-thread block, but the blocks' starts and ends (view table, tile
 // merge, stores) overlap other blocks' view loops instead of idling the SM.
 // At 256^3: 4.16 ms; 4.35 ms when each pass tested every view's orientation
-// and addressed samples from the view index; 5.09 ms for voxel_B_kernel with
-// 8-slice runs.  On bf16 entries 4.18 ms (a 1024-thread two-pass kernel took
+// and addressed samples from the view index; 5.09 ms in 1024-thread
+// blocks with 8-slice runs.  On bf16 entries 4.18 ms (a 1024-thread two-pass kernel took
 // 4.93 ms).
 template <int ZC, int TY, int MINB, bool BF, bool DIFF>
 __global__ void __launch_bounds__(32 * TY, MINB) voxel_B_slab_kernel(GeomDev g, const void *__restrict__ ypad,
@@ -637,37 +615,55 @@ static cudaError_t launch_voxel_B_slab(const GeomDev &g, const float *ypad, floa
     return cudaGetLastError();
 }
 
-template <int ZC, bool BF, bool DIFF, int PA = 32>
-static cudaError_t launch_voxel_B_t(const GeomDev &g, const float *ypad, float *x, const int *stop, cudaStream_t st)
+template <int ZC, bool FLAT, bool BF, bool DIFF>
+static cudaError_t launch_voxel_B_small(const GeomDev &g, const float *ypad, float *x, const int *stop,
+                                        cudaStream_t st)
 {
-    dim3 block(B_TILE, B_TILE);
-    const size_t smem = size_t(g.n_views) * 2 * sizeof(float4);
-    if (smem > 8 * 1024) {
-        cudaError_t e = raise_dyn_smem(reinterpret_cast<const void *>(voxel_B_kernel<ZC, BF, DIFF, PA>), smem);
-        if (e != cudaSuccess) return e;
-    }
-    dim3 grid((g.nx + B_TILE - 1) / B_TILE, (g.ny + B_TILE - 1) / B_TILE, (g.nz + ZC - 1) / ZC);
-    voxel_B_kernel<ZC, BF, DIFF, PA><<<grid, block, smem, st>>>(g, ypad, x, stop);
+    // warps a run: as many (up to 8) as keep the grid within 32 warps an SM
+    const int tiles = (g.nx + 31) / 32, runs = (g.nz + ZC - 1) / ZC;
+    int split = 1;
+    while (split < 8 && size_t(tiles) * g.ny * runs * split * 2 <= size_t(num_sms()) * 32) split *= 2;
+    const dim3 block(32, 8), grid(tiles, (g.ny * split + 7) / 8, runs);
+    voxel_B_small_kernel<ZC, FLAT, BF, DIFF><<<grid, block, 0, st>>>(g, ypad, x, split, stop);
     return cudaGetLastError();
 }
 
-template <int ZC, int PA>
-static cudaError_t launch_voxel_B_z(const GeomDev &g, const float *ypad, float *x, const int *stop, cudaStream_t st,
-                                    QuadForm form)
+// Slab blocks of ZC slices, and the time of the waves they take: a block of 12
+// slices costs 0.83 of one of 16 (4.76 ms against 4.17 ms for 256^3).
+static size_t slab_blocks(const GeomDev &g, int zc)
 {
-    if (g.sino_bf16) return launch_voxel_B_t<ZC, true, false, PA>(g, ypad, x, stop, st);
-    return form == QUAD_ROWDIFF ? launch_voxel_B_t<ZC, false, true, PA>(g, ypad, x, stop, st)
-                                : launch_voxel_B_t<ZC, false, false, PA>(g, ypad, x, stop, st);
+    return size_t((g.nx + 31) / 32) * ((g.ny + 7) / 8) * ((g.nz + zc - 1) / zc);
+}
+static double slab_cost(const GeomDev &g, int zc)
+{
+    const size_t slots = size_t(num_sms()) * 4;
+    return double((slab_blocks(g, zc) + slots - 1) / slots) * (zc + 7.5);
+}
+
+template <bool BF, bool DIFF>
+static cudaError_t launch_voxel_B_t(const GeomDev &g, const float *ypad, float *x, const int *stop, cudaStream_t st)
+{
+    if (g.kind == CT_PARALLEL_2D) return launch_voxel_B_small<1, true, BF, DIFF>(g, ypad, x, stop, st);
+    if (g.nz == 1) return launch_voxel_B_small<1, false, BF, DIFF>(g, ypad, x, stop, st);
+    // where the slab kernel's blocks do not fill the SMs (about 100^3; its
+    // samples cost half the small kernel's once they do)
+    if (slab_blocks(g, B_ZC_SLAB) < size_t(num_sms()) * (BF ? 1 : 2))
+        return launch_voxel_B_small<4, false, BF, DIFF>(g, ypad, x, stop, st);
+    // runs of 12 where 16 leave a last wave nearly empty (160 x 152 x 100: 593 -> 496 us); the row margin
+    // covers multiples of 16 past nz
+    const bool covered = (g.nz + 11) / 12 * 12 <= (g.nz + B_ZC_SLAB - 1) / B_ZC_SLAB * B_ZC_SLAB;
+    if (covered && slab_cost(g, 12) < slab_cost(g, B_ZC_SLAB))
+        return launch_voxel_B_slab<12, 8, 4, BF, DIFF>(g, ypad, x, stop, st);
+    return launch_voxel_B_slab<B_ZC_SLAB, 8, 4, BF, DIFF>(g, ypad, x, stop, st);
 }
 
 cudaError_t launch_voxel_B(const GeomDev &g, const float *ypad, float *x, const int *stop, cudaStream_t st,
                            QuadForm form)
 {
     ProfScope prof(PK_VOXEL_B, st);
-    if (g.nz == 1) return launch_voxel_B_z<1, 32>(g, ypad, x, stop, st, form);
-    if (g.sino_bf16) return launch_voxel_B_slab<B_ZC_SLAB, 8, 4, true, false>(g, ypad, x, stop, st);
-    return form == QUAD_ROWDIFF ? launch_voxel_B_slab<B_ZC_SLAB, 8, 4, false, true>(g, ypad, x, stop, st)
-                                : launch_voxel_B_slab<B_ZC_SLAB, 8, 4, false, false>(g, ypad, x, stop, st);
+    if (g.sino_bf16) return launch_voxel_B_t<true, false>(g, ypad, x, stop, st);
+    return form == QUAD_ROWDIFF ? launch_voxel_B_t<false, true>(g, ypad, x, stop, st)
+                                : launch_voxel_B_t<false, false>(g, ypad, x, stop, st);
 }
 
 // ---------------------------------------------------------------------------
