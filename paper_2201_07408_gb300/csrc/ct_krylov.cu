@@ -15,11 +15,10 @@
 // stop, a lucky breakdown or a non-finite norm.
 #include <algorithm>
 #include <cmath>
-#include <mutex>
-#include <unordered_map>
 #include <cstdio>
 #include <cstring>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "ct_internal.cuh"
@@ -28,7 +27,7 @@ namespace ct {
 
 constexpr int RED_BLOCK = 256;
 
-enum : int { ST_RUN = 0, ST_TOL = 1, ST_LUCKY = 2, ST_NONFINITE = 3 };
+enum : int { ST_RUN = 0, ST_TOL = 1, ST_LUCKY = 2, ST_NONFINITE = 3, ST_TIMEOUT = 4 };
 
 // Device-resident solver state.
 struct SolverState {
@@ -47,81 +46,212 @@ struct SolverState {
 // ---------------------------------------------------------------------------
 // accumulators
 // ---------------------------------------------------------------------------
+// a + b as a rounded sum (returned) and its rounding error
+__device__ __forceinline__ float two_sum(float a, float b, float &err)
+{
+    const float t = __fadd_rn(a, b);
+    const float bp = __fsub_rn(t, a);
+    err = __fadd_rn(__fsub_rn(a, __fsub_rn(t, bp)), __fsub_rn(b, bp));
+    return t;
+}
+
+// An unevaluated sum s + c + d of FP32 numbers of falling size (about 70 bits).
+struct Sum3 {
+    float s, c, d;
+    __device__ __forceinline__ void add(const Sum3 &o)
+    {
+        float e1, e2, e3;
+        s = two_sum(s, o.s, e1);
+        c = two_sum(c, o.c, e2);
+        c = two_sum(c, e1, e3);
+        d = __fadd_rn(__fadd_rn(d, o.d), __fadd_rn(e2, e3));
+    }
+    __device__ __forceinline__ Sum3 lane_down(int o) const
+    {
+        return Sum3{__shfl_down_sync(0xffffffffu, s, o), __shfl_down_sync(0xffffffffu, c, o),
+                    __shfl_down_sync(0xffffffffu, d, o)};
+    }
+    __device__ __forceinline__ double value() const { return double(s) + (double(c) + double(d)); }
+};
+
 template <int MODE>
 struct Acc;
 
+// Thread sums of products, one for each position in a group of 4 elements (four
+// short chains: less rounding, and their steps overlap).
 template <>
-struct Acc<1> {  // FP32 FMA accumulation, FP64 reduction
-    float s = 0.0f;
-    __device__ __forceinline__ void add(float a, float b) { s = fmaf(a, b, s); }
-    __device__ __forceinline__ double value() const { return double(s); }
+struct Acc<1> {  // FP32 FMA accumulation
+    float p[4] = {};
+    __device__ __forceinline__ void add(float a, float b, int e = 0) { p[e & 3] = fmaf(a, b, p[e & 3]); }
+    __device__ __forceinline__ Sum3 part(int e) const { return Sum3{p[e], 0.0f, 0.0f}; }
 };
 
 template <>
 struct Acc<0> {  // compensated: two-product (FMA) + two-sum in FP32
-    float s = 0.0f, c = 0.0f;
-    __device__ __forceinline__ void add(float a, float b)
+    float s[4] = {}, c[4] = {};
+    __device__ __forceinline__ void add(float a, float b, int e = 0)
     {
         const float p = __fmul_rn(a, b);
         const float pe = fmaf(a, b, -p);
-        const float t = __fadd_rn(s, p);
-        const float bp = __fsub_rn(t, s);
-        const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(p, bp));
-        s = t;
-        c = __fadd_rn(c, __fadd_rn(e, pe));
+        float err;
+        s[e & 3] = two_sum(s[e & 3], p, err);
+        c[e & 3] = __fadd_rn(c[e & 3], __fadd_rn(err, pe));
     }
-    __device__ __forceinline__ double value() const { return double(s) + double(c); }
+    __device__ __forceinline__ Sum3 part(int e) const { return Sum3{s[e], c[e], 0.0f}; }
 };
 
-__device__ __forceinline__ double warp_sum(double v)
+template <int MODE>
+__device__ __forceinline__ Sum3 thread_sum(const Acc<MODE> &a)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
+    Sum3 r = a.part(0), r2 = a.part(2);
+    r.add(a.part(1));
+    r2.add(a.part(3));
+    r.add(r2);
+    return r;
 }
 
-// Block sum of two values; result valid in thread 0.
-__device__ __forceinline__ void block_sum2(double &a, double &b)
+// Sums over a block of NT threads of two values (each only if wanted, the same
+// for all threads), valid in thread 0.  FP64 additions run at 2 a clock on an
+// SM: a warp-wide one occupies the unit for 16 cycles, and a tree of them in
+// each of a streaming pass's warps took longer than the pass's memory traffic.
+// So lanes and warps add triples of FP32 numbers that keep the rounding errors
+// (Sum3), and only the block's sum goes on in FP64.  Sums near the end of
+// FP32's range are added in FP64 throughout.
+struct BlockPart {
+    Sum3 sum;
+    int big;
+    double v;
+};
+template <int MODE>
+__device__ __forceinline__ void warp_part(const Acc<MODE> &acc, BlockPart &out)
 {
-    __shared__ double sa[RED_BLOCK / 32], sb[RED_BLOCK / 32];
-    a = warp_sum(a);
-    b = warp_sum(b);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) {
-        sa[w] = a;
-        sb[w] = b;
+    Sum3 r = thread_sum(acc);
+    const bool big = __any_sync(0xffffffffu, !(fabsf(r.s) <= 1e30f));
+    double v = 0.0;
+    if (big) {
+        v = MODE == 0 || fabsf(r.s) <= 1e30f ? r.value() : double(r.s);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    } else {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) r.add(r.lane_down(o));
     }
+    if ((threadIdx.x & 31) == 0) out = BlockPart{r, big, v};
+}
+template <int NW>
+__device__ __forceinline__ double warps_total(const BlockPart *part)
+{
+    const int lane = threadIdx.x & 31;
+    BlockPart p = lane < NW ? part[lane] : BlockPart{{0.0f, 0.0f, 0.0f}, 0, 0.0};
+    if (__any_sync(0xffffffffu, p.big)) {
+        double v = p.big ? p.v : p.sum.value();
+#pragma unroll
+        for (int o = NW / 2; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        return v;
+    }
+#pragma unroll
+    for (int o = NW / 2; o > 0; o >>= 1) p.sum.add(p.sum.lane_down(o));
+    return p.sum.value();
+}
+
+template <int NT, int MODE>
+__device__ __forceinline__ void block_total2(const Acc<MODE> &a, const Acc<MODE> &b, bool want_a, bool want_b,
+                                             double &ta, double &tb)
+{
+    __shared__ BlockPart part[2][NT / 32];
+    const int w = threadIdx.x >> 5;
+    if (want_a) warp_part(a, part[0][w]);
+    if (want_b) warp_part(b, part[1][w]);
     __syncthreads();
+    ta = tb = 0.0;
     if (w == 0) {
-        a = lane < RED_BLOCK / 32 ? sa[lane] : 0.0;
-        b = lane < RED_BLOCK / 32 ? sb[lane] : 0.0;
-        a = warp_sum(a);
-        b = warp_sum(b);
+        if (want_a) ta = warps_total<NT / 32>(part[0]);
+        if (want_b) tb = warps_total<NT / 32>(part[1]);
     }
+}
+
+// The sums of n partials in a fixed order, valid in thread 0 afterwards (every
+// thread of the block calls it).  load(i, a, b) reads partial i and says
+// whether it is there yet; a partial that stays away for SLOT_POLLS reads ends
+// the wait (false, in every thread).  Four warps add: few FP64 additions in
+// all, and a lane's reads go out together.
+constexpr int SLOT_POLLS = 1 << 22;
+template <typename F>
+__device__ __forceinline__ bool sum_partials(F load, int n, bool want_a, bool want_b, double &ta, double &tb)
+{
+    __shared__ double sum[2][4];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    bool ok = true;
+    if (w < 4) {
+        ta = tb = 0.0;
+        for (int i0 = threadIdx.x; i0 < n; i0 += 4 * 128) {
+            double a[4], b[4];
+            int polls = 0;
+            bool all;
+            do {
+                all = true;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    a[k] = b[k] = 0.0;
+                    if (i0 + 128 * k < n) all = load(i0 + 128 * k, a[k], b[k]) && all;
+                }
+            } while (!all && ++polls < SLOT_POLLS);
+            ok = ok && all;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                if (want_a) ta += a[k];
+                if (want_b) tb += b[k];
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            if (want_a) ta += __shfl_down_sync(0xffffffffu, ta, o);
+            if (want_b) tb += __shfl_down_sync(0xffffffffu, tb, o);
+        }
+        if (lane == 0) {
+            sum[0][w] = ta;
+            sum[1][w] = tb;
+        }
+    }
+    if (w < 4) __threadfence();   // reads of the next partials stay behind these
+    ok = __syncthreads_and(ok);
+    if (threadIdx.x == 0) {
+        ta = (sum[0][0] + sum[0][1]) + (sum[0][2] + sum[0][3]);
+        tb = (sum[1][0] + sum[1][1]) + (sum[1][2] + sum[1][3]);
+    }
+    return ok;
 }
 
 // Stores the block's partial sums; the last block to finish sums all
-// partials in block order and writes the outputs.
-__device__ __forceinline__ void grid_finish(double a, double b, double *partials, unsigned *counter,
-                                            double *out_a, double *out_b)
+// partials in a fixed order and writes the outputs (either may be null).
+template <int NT, int MODE>
+__device__ __forceinline__ void grid_finish(const Acc<MODE> &a, const Acc<MODE> &b, double *partials,
+                                            unsigned *counter, double *out_a, double *out_b)
 {
     __shared__ bool last;
-    block_sum2(a, b);
+    double ta, tb;
+    block_total2<NT, MODE>(a, b, out_a != nullptr, out_b != nullptr, ta, tb);
+    if (gridDim.x == 1) {
+        if (threadIdx.x == 0) {
+            if (out_a) *out_a = ta;
+            if (out_b) *out_b = tb;
+        }
+        return;
+    }
     if (threadIdx.x == 0) {
-        partials[2 * blockIdx.x] = a;
-        partials[2 * blockIdx.x + 1] = b;
+        partials[2 * blockIdx.x] = ta;
+        partials[2 * blockIdx.x + 1] = tb;
         __threadfence();
         last = atomicAdd(counter, 1u) == gridDim.x - 1;
     }
     __syncthreads();
     if (!last) return;
     __threadfence();
-    double ta = 0.0, tb = 0.0;
-    for (int i = threadIdx.x; i < int(gridDim.x); i += RED_BLOCK) {
-        ta += __ldcg(partials + 2 * i);
-        tb += __ldcg(partials + 2 * i + 1);
-    }
-    block_sum2(ta, tb);
+    sum_partials([&](int i, double &va, double &vb) {
+        if (out_a) va = __ldcg(partials + 2 * i);
+        if (out_b) vb = __ldcg(partials + 2 * i + 1);
+        return true;
+    }, gridDim.x, out_a != nullptr, out_b != nullptr, ta, tb);
     if (threadIdx.x == 0) {
         if (out_a) *out_a = ta;
         if (out_b) *out_b = tb;
@@ -147,33 +277,27 @@ __device__ __forceinline__ void mgs_group4(float4 *q4, float4 a, float4 p, float
         *q4 = a;
     }
     if (has_cur) {
-        dot.add(a.x, c.x);
-        dot.add(a.y, c.y);
-        dot.add(a.z, c.z);
-        dot.add(a.w, c.w);
+        dot.add(a.x, c.x, 0);
+        dot.add(a.y, c.y, 1);
+        dot.add(a.z, c.z, 2);
+        dot.add(a.w, c.w, 3);
     }
     if (sumsq) {
-        ss.add(a.x, a.x);
-        ss.add(a.y, a.y);
-        ss.add(a.z, a.z);
-        ss.add(a.w, a.w);
+        ss.add(a.x, a.x, 0);
+        ss.add(a.y, a.y, 1);
+        ss.add(a.z, a.z, 2);
+        ss.add(a.w, a.w, 3);
     }
 }
 
+// The elements tid, tid + nth, ... of a pass over an FP32 basis.
 template <int MODE>
-__global__ void __launch_bounds__(RED_BLOCK) mgs_pass_kernel(
-    float *__restrict__ q, const float *__restrict__ vprev, const double *__restrict__ hprev,
-    const float *__restrict__ vcur, size_t len, int vec4, double *__restrict__ partials,
-    unsigned *__restrict__ counter, double *__restrict__ out_dot, double *__restrict__ out_sumsq,
-    const int *__restrict__ stop, const int *__restrict__ skip)
+__device__ __forceinline__ void pass_elements(float *__restrict__ q, const float *__restrict__ vprev, float h,
+                                              const float *__restrict__ vcur, size_t len, bool vec, bool sumsq,
+                                              size_t tid, size_t nth, Acc<MODE> &dot, Acc<MODE> &ss)
 {
-    if ((stop && *stop) || (skip && *skip)) return;
-    const float h = vprev ? float(*hprev) : 0.0f;
-    Acc<MODE> dot, ss;
-    const size_t tid = blockIdx.x * size_t(RED_BLOCK) + threadIdx.x;
-    const size_t nth = size_t(gridDim.x) * RED_BLOCK;
     size_t start = 0;
-    if (vec4) {
+    if (vec) {
         const size_t n4 = len / 4;
         float4 *q4 = reinterpret_cast<float4 *>(q);
         const float4 *p4 = reinterpret_cast<const float4 *>(vprev);
@@ -187,12 +311,12 @@ __global__ void __launch_bounds__(RED_BLOCK) mgs_pass_kernel(
             const float4 a0 = q4[i], a1 = q4[i1];
             const float4 p0 = vprev ? __ldcs(p4 + i) : zero, p1 = vprev ? __ldcs(p4 + i1) : zero;
             const float4 c0 = vcur ? __ldcs(c4 + i) : zero, c1 = vcur ? __ldcs(c4 + i1) : zero;
-            mgs_group4(q4 + i, a0, p0, c0, vprev != nullptr, vcur != nullptr, out_sumsq != nullptr, h, dot, ss);
-            mgs_group4(q4 + i1, a1, p1, c1, vprev != nullptr, vcur != nullptr, out_sumsq != nullptr, h, dot, ss);
+            mgs_group4(q4 + i, a0, p0, c0, vprev != nullptr, vcur != nullptr, sumsq, h, dot, ss);
+            mgs_group4(q4 + i1, a1, p1, c1, vprev != nullptr, vcur != nullptr, sumsq, h, dot, ss);
         }
         if (i < n4)
             mgs_group4(q4 + i, q4[i], vprev ? __ldcs(p4 + i) : zero, vcur ? __ldcs(c4 + i) : zero, vprev != nullptr,
-                       vcur != nullptr, out_sumsq != nullptr, h, dot, ss);
+                       vcur != nullptr, sumsq, h, dot, ss);
         start = n4 * 4;
     }
     for (size_t i = start + tid; i < len; i += nth) {
@@ -202,9 +326,8 @@ __global__ void __launch_bounds__(RED_BLOCK) mgs_pass_kernel(
             q[i] = a;
         }
         if (vcur) dot.add(a, vcur[i]);
-        if (out_sumsq) ss.add(a, a);
+        if (sumsq) ss.add(a, a);
     }
-    grid_finish(dot.value(), ss.value(), partials, counter, out_dot, out_sumsq);
 }
 
 // The same pass with a bf16 basis (FP32 work vector q): eight elements per
@@ -234,28 +357,21 @@ __device__ __forceinline__ void mgs_group8(float4 *q4, float4 lo, float4 hi, uin
         float cv[8];
         unpack8(cw, cv);
 #pragma unroll
-        for (int e = 0; e < 8; ++e) dot.add(a[e], cv[e]);
+        for (int e = 0; e < 8; ++e) dot.add(a[e], cv[e], e);
     }
     if (sumsq) {
 #pragma unroll
-        for (int e = 0; e < 8; ++e) ss.add(a[e], a[e]);
+        for (int e = 0; e < 8; ++e) ss.add(a[e], a[e], e);
     }
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(RED_BLOCK) mgs_pass_bf16_kernel(
-    float *__restrict__ q, const __nv_bfloat16 *__restrict__ vprev, const double *__restrict__ hprev,
-    const __nv_bfloat16 *__restrict__ vcur, size_t len, int vec8, double *__restrict__ partials,
-    unsigned *__restrict__ counter, double *__restrict__ out_dot, double *__restrict__ out_sumsq,
-    const int *__restrict__ stop, const int *__restrict__ skip)
+__device__ __forceinline__ void pass_elements(float *__restrict__ q, const __nv_bfloat16 *__restrict__ vprev, float h,
+                                              const __nv_bfloat16 *__restrict__ vcur, size_t len, bool vec,
+                                              bool sumsq, size_t tid, size_t nth, Acc<MODE> &dot, Acc<MODE> &ss)
 {
-    if ((stop && *stop) || (skip && *skip)) return;
-    const float h = vprev ? float(*hprev) : 0.0f;
-    Acc<MODE> dot, ss;
-    const size_t tid = blockIdx.x * size_t(RED_BLOCK) + threadIdx.x;
-    const size_t nth = size_t(gridDim.x) * RED_BLOCK;
     size_t start = 0;
-    if (vec8) {
+    if (vec) {
         const size_t n8 = len / 8;
         float4 *q4 = reinterpret_cast<float4 *>(q);
         const uint4 *p8 = reinterpret_cast<const uint4 *>(vprev);
@@ -268,14 +384,12 @@ __global__ void __launch_bounds__(RED_BLOCK) mgs_pass_bf16_kernel(
             const float4 l0 = q4[2 * i], h0 = q4[2 * i + 1], l1 = q4[2 * i1], h1 = q4[2 * i1 + 1];
             const uint4 p0 = vprev ? __ldcs(p8 + i) : zero, p1 = vprev ? __ldcs(p8 + i1) : zero;
             const uint4 c0 = vcur ? __ldcs(c8 + i) : zero, c1 = vcur ? __ldcs(c8 + i1) : zero;
-            mgs_group8(q4 + 2 * i, l0, h0, p0, c0, vprev != nullptr, vcur != nullptr, out_sumsq != nullptr, h, dot, ss);
-            mgs_group8(q4 + 2 * i1, l1, h1, p1, c1, vprev != nullptr, vcur != nullptr, out_sumsq != nullptr, h, dot,
-                       ss);
+            mgs_group8(q4 + 2 * i, l0, h0, p0, c0, vprev != nullptr, vcur != nullptr, sumsq, h, dot, ss);
+            mgs_group8(q4 + 2 * i1, l1, h1, p1, c1, vprev != nullptr, vcur != nullptr, sumsq, h, dot, ss);
         }
         if (i < n8)
             mgs_group8(q4 + 2 * i, q4[2 * i], q4[2 * i + 1], vprev ? __ldcs(p8 + i) : zero,
-                       vcur ? __ldcs(c8 + i) : zero, vprev != nullptr, vcur != nullptr, out_sumsq != nullptr, h, dot,
-                       ss);
+                       vcur ? __ldcs(c8 + i) : zero, vprev != nullptr, vcur != nullptr, sumsq, h, dot, ss);
         start = n8 * 8;
     }
     for (size_t i = start + tid; i < len; i += nth) {
@@ -285,9 +399,23 @@ __global__ void __launch_bounds__(RED_BLOCK) mgs_pass_bf16_kernel(
             q[i] = a;
         }
         if (vcur) dot.add(a, __bfloat162float(vcur[i]));
-        if (out_sumsq) ss.add(a, a);
+        if (sumsq) ss.add(a, a);
     }
-    grid_finish(dot.value(), ss.value(), partials, counter, out_dot, out_sumsq);
+}
+
+template <int MODE, typename TB, int NT>
+__global__ void __launch_bounds__(NT) mgs_pass_kernel(float *__restrict__ q, const TB *__restrict__ vprev,
+                                                      const double *__restrict__ hprev, const TB *__restrict__ vcur,
+                                                      size_t len, int vec, double *__restrict__ partials,
+                                                      unsigned *__restrict__ counter, double *__restrict__ out_dot,
+                                                      double *__restrict__ out_sumsq, const int *__restrict__ stop,
+                                                      const int *__restrict__ skip)
+{
+    if ((stop && *stop) || (skip && *skip)) return;
+    Acc<MODE> dot, ss;
+    pass_elements<MODE>(q, vprev, vprev ? float(*hprev) : 0.0f, vcur, len, vec, out_sumsq != nullptr,
+                        blockIdx.x * size_t(NT) + threadIdx.x, gridDim.x * size_t(NT), dot, ss);
+    grid_finish<NT, MODE>(dot, ss, partials, counter, vcur ? out_dot : nullptr, out_sumsq);
 }
 
 // sum (a - b)^2 -> *out (recomputed data residuals)
@@ -305,7 +433,7 @@ __global__ void __launch_bounds__(RED_BLOCK) diff_sumsq_kernel(const float *__re
         const float d = a[i] - b[i];
         ss.add(d, d);
     }
-    grid_finish(0.0, ss.value(), partials, counter, nullptr, out);
+    grid_finish<RED_BLOCK, 1>(Acc<1>(), ss, partials, counter, nullptr, out);
 }
 
 static unsigned red_blocks(size_t len)
@@ -315,80 +443,71 @@ static unsigned red_blocks(size_t len)
     return unsigned(std::max<size_t>(1, std::min(want, cap)));
 }
 
-// Blocks of a grid-stride pass over len elements (elems per thread-step):
-// every SM gets as many blocks as can be resident at once (at most 8, the
-// size of the partials array), so no partial second wave runs.
-static unsigned resident_blocks(const void *kernel, size_t len, size_t elems)
-{
-    static std::mutex mu;
-    static std::unordered_map<const void *, int> occ;
-    int per_sm = 0;
-    {
-        std::lock_guard<std::mutex> lock(mu);
-        auto it = occ.find(kernel);
-        if (it == occ.end()) {
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, RED_BLOCK, 0) != cudaSuccess) {
-                cudaGetLastError();
-                per_sm = 4;
-            }
-            occ.emplace(kernel, per_sm);
-        } else {
-            per_sm = it->second;
-        }
-    }
-    per_sm = std::min(std::max(per_sm, 1), 8);
-    const size_t want = (len / elems + RED_BLOCK - 1) / RED_BLOCK;
-    return unsigned(std::max<size_t>(1, std::min(want, size_t(num_sms()) * per_sm)));
-}
-
 static size_t partials_count() { return size_t(num_sms()) * 8 * 2; }
 
-static cudaError_t mgs_pass(int mode, float *q, const float *vprev, const double *hprev,
-                            const float *vcur, size_t len, double *partials, unsigned *counter,
-                            double *out_dot, double *out_sumsq, const int *stop, const int *skip,
-                            cudaStream_t st)
+
+// Vectors of up to sweep_max() elements are orthogonalised by one kernel that
+// keeps q in registers (mgs_sweep_kernel): one block of SWEEP_NT threads an SM,
+// 32 elements a thread at most.
+constexpr int SWEEP_NT = 512, SWEEP_ELEMS = 32;
+static size_t slots_count() { return size_t(num_sms()) * 2 * 3 * 2; }
+static size_t sweep_max() { return size_t(num_sms()) * SWEEP_NT * SWEEP_ELEMS; }
+
+// Blocks of the sweep kernel, and of a single pass over as many elements (the
+// same sums in the same order either way): 16 elements a thread until every SM
+// has a block.
+static unsigned sweep_blocks(size_t len)
 {
-    const int vec4 = (len % 4 == 0) && (reinterpret_cast<uintptr_t>(q) % 16 == 0) &&
-                     (!vprev || reinterpret_cast<uintptr_t>(vprev) % 16 == 0) &&
-                     (!vcur || reinterpret_cast<uintptr_t>(vcur) % 16 == 0);
-    const unsigned blocks = resident_blocks(
-        mode == 0 ? reinterpret_cast<const void *>(mgs_pass_kernel<0>)
-                  : reinterpret_cast<const void *>(mgs_pass_kernel<1>), len, 4);
-    ProfScope prof(PK_MGS, st);
-    if (mode == 0)
-        mgs_pass_kernel<0><<<blocks, RED_BLOCK, 0, st>>>(q, vprev, hprev, vcur, len, vec4, partials,
-                                                         counter, out_dot, out_sumsq, stop, skip);
-    else
-        mgs_pass_kernel<1><<<blocks, RED_BLOCK, 0, st>>>(q, vprev, hprev, vcur, len, vec4, partials,
-                                                         counter, out_dot, out_sumsq, stop, skip);
-    return cudaGetLastError();
+    return unsigned(std::min((len + 16 * SWEEP_NT - 1) / (16 * SWEEP_NT), size_t(num_sms())));
 }
 
 // MGS pass over a typed basis (float or bf16 vectors; q is always float).
+template <int MODE, typename TB>
+static cudaError_t mgs_pass_t(float *q, const TB *vprev, const double *hprev, const TB *vcur, size_t len,
+                              double *partials, unsigned *counter, double *out_dot, double *out_sumsq,
+                              const int *stop, const int *skip, cudaStream_t st)
+{
+    constexpr size_t G = 16 / sizeof(TB);   // elements of a 16-byte group of the basis
+    const int vec = (len % G == 0) && (reinterpret_cast<uintptr_t>(q) % 16 == 0) &&
+                    (!vprev || reinterpret_cast<uintptr_t>(vprev) % 16 == 0) &&
+                    (!vcur || reinterpret_cast<uintptr_t>(vcur) % 16 == 0);
+    ProfScope prof(PK_MGS, st);
+    if (len <= sweep_max()) {
+        mgs_pass_kernel<MODE, TB, SWEEP_NT><<<sweep_blocks(len), SWEEP_NT, 0, st>>>(
+            q, vprev, hprev, vcur, len, vec, partials, counter, out_dot, out_sumsq, stop, skip);
+        return cudaGetLastError();
+    }
+    // a thread's two groups a step put six 16-byte loads in flight, and 4 blocks an SM of them cover the memory's
+    // latency (256^3: 32.8 us a pass; 2, 6 and 8 blocks 38.3, 39.2, 35.8)
+    const unsigned blocks = unsigned(std::min((len / G + RED_BLOCK - 1) / RED_BLOCK, size_t(num_sms()) * 4));
+    mgs_pass_kernel<MODE, TB, RED_BLOCK><<<blocks, RED_BLOCK, 0, st>>>(q, vprev, hprev, vcur, len, vec, partials,
+                                                                       counter, out_dot, out_sumsq, stop, skip);
+    return cudaGetLastError();
+}
+
 static cudaError_t mgs_pass_typed(int mode, bool vbf16, float *q, const void *vprev, const double *hprev,
                                   const void *vcur, size_t len, double *partials, unsigned *counter,
                                   double *out_dot, double *out_sumsq, const int *stop, const int *skip,
                                   cudaStream_t st)
 {
-    if (!vbf16)
-        return mgs_pass(mode, q, static_cast<const float *>(vprev), hprev, static_cast<const float *>(vcur), len,
-                        partials, counter, out_dot, out_sumsq, stop, skip, st);
-    const int vec8 = (len % 8 == 0) && (reinterpret_cast<uintptr_t>(q) % 16 == 0) &&
-                     (!vprev || reinterpret_cast<uintptr_t>(vprev) % 16 == 0) &&
-                     (!vcur || reinterpret_cast<uintptr_t>(vcur) % 16 == 0);
-    const unsigned blocks = resident_blocks(
-        mode == 0 ? reinterpret_cast<const void *>(mgs_pass_bf16_kernel<0>)
-                  : reinterpret_cast<const void *>(mgs_pass_bf16_kernel<1>), len, 16);
-    ProfScope prof(PK_MGS, st);
-    const auto *p = static_cast<const __nv_bfloat16 *>(vprev);
-    const auto *c = static_cast<const __nv_bfloat16 *>(vcur);
-    if (mode == 0)
-        mgs_pass_bf16_kernel<0><<<blocks, RED_BLOCK, 0, st>>>(q, p, hprev, c, len, vec8, partials, counter, out_dot,
-                                                              out_sumsq, stop, skip);
-    else
-        mgs_pass_bf16_kernel<1><<<blocks, RED_BLOCK, 0, st>>>(q, p, hprev, c, len, vec8, partials, counter, out_dot,
-                                                              out_sumsq, stop, skip);
-    return cudaGetLastError();
+    auto run = [&](auto m, auto tb) {
+        using TB = decltype(tb);
+        return mgs_pass_t<decltype(m)::value, TB>(q, static_cast<const TB *>(vprev), hprev,
+                                                  static_cast<const TB *>(vcur), len, partials, counter, out_dot,
+                                                  out_sumsq, stop, skip, st);
+    };
+    using M0 = std::integral_constant<int, 0>;
+    using M1 = std::integral_constant<int, 1>;
+    if (vbf16) return mode == 0 ? run(M0(), __nv_bfloat16()) : run(M1(), __nv_bfloat16());
+    return mode == 0 ? run(M0(), float()) : run(M1(), float());
+}
+
+static cudaError_t mgs_pass(int mode, float *q, const float *vprev, const double *hprev, const float *vcur, size_t len,
+                            double *partials, unsigned *counter, double *out_dot, double *out_sumsq, const int *stop,
+                            const int *skip, cudaStream_t st)
+{
+    return mgs_pass_typed(mode, false, q, vprev, hprev, vcur, len, partials, counter, out_dot, out_sumsq, stop, skip,
+                          st);
 }
 
 // ---------------------------------------------------------------------------
@@ -425,56 +544,244 @@ __global__ void reorth_decide_kernel(SolverState *st)
     st->sumsq_pre2 = st->sumsq;
 }
 
-__global__ void givens_kernel(int j, int k, double *H, const double *H2, double *R, double *cs,
-                              double *sn, double *g, double *resid, SolverState *st, double tol)
+// One warp.  The column's loads (32 rows at a time, a row a lane) are in flight
+// together; only the chain of rotations is serial.
+struct GivensArgs {
+    int j, k;
+    double *H;
+    const double *H2;   // the second sweep's coefficients, or null
+    double *R, *cs, *sn, *g, *resid;
+    SolverState *st;
+    double tol;
+};
+__device__ __forceinline__ void givens_step(const GivensArgs &A)
 {
-    if (st->status != ST_RUN) return;
-    const int ld = k + 1;
-    double *h = H + size_t(j) * ld;
-    if (H2 && !st->reorth_skip)
-        for (int i = 0; i <= j; ++i) h[i] += H2[i];
-    const double hnext = sqrt(st->sumsq);
-    const double ref = sqrt(st->ref_sumsq);
+    const int lane = threadIdx.x & 31, j = A.j;
+    const int ld = A.k + 1;
+    double *h = A.H + size_t(j) * ld, *r = A.R + size_t(j) * ld;
+    const double *H2 = A.H2;
+    double *cs = A.cs, *sn = A.sn, *g = A.g, *resid = A.resid;
+    SolverState *st = A.st;
+    const double tol = A.tol;
+    const double sumsq = st->sumsq, ref_sumsq = st->ref_sumsq;
+    const bool second = H2 && !st->reorth_skip;
+    const double g_j = g[j], resid0 = resid[0];
+    bool bad = !isfinite(sumsq) || !isfinite(ref_sumsq);
+    double x = 0.0;   // entry i of the column after the rotations before it
+    for (int i0 = 0; i0 <= j; i0 += 32) {
+        const int i = i0 + lane;
+        double hv = 0.0, c = 0.0, s = 0.0, done = 0.0;
+        if (i <= j) {
+            hv = h[i];
+            if (second) {
+                hv += H2[i];
+                h[i] = hv;
+            }
+            bad = bad || !isfinite(hv);
+            if (i > 0) {   // the rotation of rows i - 1 and i
+                c = cs[i - 1];
+                s = sn[i - 1];
+            }
+        }
+        const double ch = c * hv, sh = s * hv;
+        for (int l = 0; l < 32 && i0 + l <= j; ++l) {
+            const double cl = __shfl_sync(0xffffffffu, c, l), sl = __shfl_sync(0xffffffffu, s, l);
+            const double t = fma(cl, x, __shfl_sync(0xffffffffu, sh, l));
+            x = i0 + l == 0 ? __shfl_sync(0xffffffffu, hv, l) : fma(-sl, x, __shfl_sync(0xffffffffu, ch, l));
+            if (lane == l) done = t;
+        }
+        if (i > 0 && i <= j) r[i - 1] = done;
+    }
+    bad = __any_sync(0xffffffffu, bad);
+    // FP64 roots and quotients are long chains of slow operations: lane 0, 1, 2
+    // take the roots of ||q||^2, of its value before the sweep, and of
+    // x^2 + ||q||^2 at once, then the three quotients.  (Squares of sums of FP32
+    // data are far inside FP64's range.)
+    const double root = sqrt(lane == 0 ? sumsq : lane == 1 ? ref_sumsq : fma(x, x, sumsq));
+    const double hnext = __shfl_sync(0xffffffffu, root, 0), ref = __shfl_sync(0xffffffffu, root, 1);
+    const bool lucky = hnext <= 1e-14 * ref;
+    const double rr = lucky ? fabs(x) : __shfl_sync(0xffffffffu, root, 2);
+    const double quot = (lane == 0 ? x : lane == 1 ? (lucky ? 0.0 : hnext) : 1.0) / (lane < 2 ? rr : hnext);
+    const double qc = __shfl_sync(0xffffffffu, quot, 0), qs = __shfl_sync(0xffffffffu, quot, 1);
+    const double inv = __shfl_sync(0xffffffffu, quot, 2);
+    if (lane > 0) return;
     h[j + 1] = hnext;
-    bool bad = !isfinite(hnext) || !isfinite(ref);
-    for (int i = 0; i <= j; ++i) bad = bad || !isfinite(h[i]);
     if (bad) {
         st->status = ST_NONFINITE;
         return;
     }
-    const bool lucky = hnext <= 1e-14 * ref;
-    double *r = R + size_t(j) * ld;
-    for (int i = 0; i <= j; ++i) r[i] = h[i];
-    r[j + 1] = lucky ? 0.0 : hnext;
-    for (int i = 0; i < j; ++i) {
-        const double t = cs[i] * r[i] + sn[i] * r[i + 1];
-        r[i + 1] = -sn[i] * r[i] + cs[i] * r[i + 1];
-        r[i] = t;
-    }
-    const double a = r[j], b = r[j + 1];
-    const double rr = hypot(a, b);
-    double c = 1.0, s = 0.0;
-    if (rr != 0.0) {
-        c = a / rr;
-        s = b / rr;
-    }
+    const double c = rr != 0.0 ? qc : 1.0, s = rr != 0.0 ? qs : 0.0;
     cs[j] = c;
     sn[j] = s;
     r[j] = rr;
     r[j + 1] = 0.0;
-    g[j + 1] = -s * g[j];
-    g[j] = c * g[j];
+    const double g1 = -s * g_j, g0 = c * g_j;
+    g[j + 1] = g1;
+    g[j] = g0;
     // a column that vanishes after the rotations (a breakdown on which the
     // operator is singular) cannot reduce g[j]: the least-squares residual
     // stays, and the back substitution gives that coefficient 0
-    resid[j + 1] = rr != 0.0 ? fabs(g[j + 1]) : hypot(g[j], g[j + 1]);
+    const double res = rr != 0.0 ? fabs(g1) : hypot(g0, g1);
+    resid[j + 1] = res;
     st->iters = j + 1;
     if (lucky || rr == 0.0) {
         st->status = ST_LUCKY;
     } else {
-        st->inv_norm = 1.0 / hnext;
-        if (tol > 0.0 && resid[j + 1] <= tol * resid[0]) st->status = ST_TOL;
+        st->inv_norm = inv;
+        if (tol > 0.0 && res <= tol * resid0) st->status = ST_TOL;
     }
+}
+__global__ void givens_kernel(GivensArgs A)
+{
+    if (A.st->status != ST_RUN) return;
+    givens_step(A);
+}
+
+// ---------------------------------------------------------------------------
+// A whole MGS sweep of q against V_0 .. V_j in one launch, for vectors that fit
+// the registers.  A pass a vector has to wait for the sum over all of q before
+// it can go on, and as separate launches it spent most of its time on that
+// (about 11 us a pass for 2.1 M elements, 5 us of it memory traffic; 8 us for
+// 4096).  Here q stays in registers, the next basis vector is loaded while the
+// sum is on its way, and the blocks exchange their partial sums through `slots`:
+// each block publishes its partial and reads everyone's, adding them up in the
+// order in which a single pass does, so the coefficients have the same bits.
+// A slot holds SLOT_EMPTY until its block publishes; pass p uses slots p mod 3,
+// and a block empties its slots of pass p - 1 once it has seen all of pass p
+// (by then everyone has read them).  Two sets take turns from launch to launch:
+// a launch empties the other set.  Launched cooperatively (all blocks
+// resident); a wait that runs out marks the solve and ends the kernel.
+// ---------------------------------------------------------------------------
+constexpr unsigned long long SLOT_EMPTY = ~0ull;
+
+__device__ __forceinline__ bool slot_get(const unsigned long long *p, double &v)
+{
+    unsigned long long b;
+    asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(b) : "l"(p) : "memory");
+    v = __longlong_as_double((long long)b);
+    return b != SLOT_EMPTY;
+}
+__device__ __forceinline__ void slot_put(unsigned long long *p, double v)
+{
+    unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    if (b == SLOT_EMPTY) b = 0x7ff8000000000000ull;   // (another NaN)
+    asm volatile("st.release.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(b) : "memory");
+}
+
+// unpacked group of 16 bytes of the basis
+__device__ __forceinline__ void unpack_group(const uint4 w, float (&o)[4])
+{
+    o[0] = __uint_as_float(w.x); o[1] = __uint_as_float(w.y); o[2] = __uint_as_float(w.z); o[3] = __uint_as_float(w.w);
+}
+__device__ __forceinline__ void unpack_group(const uint4 w, float (&o)[8]) { unpack8(w, o); }
+
+template <int MODE, typename TB, int ELEMS>
+__global__ void __launch_bounds__(SWEEP_NT)
+    mgs_sweep_kernel(float *q, const TB *V, size_t ldv, int j, size_t len, double *h, double *first_ss,
+                     double *last_ss, unsigned long long *slots, int set, const int *stop, const int *skip,
+                     SolverState *st, GivensArgs giv)
+{
+    constexpr int G = 16 / sizeof(TB), NG = ELEMS / G;
+    const int nb = gridDim.x;
+    // slots[set][pass mod 3][sum][block]
+    unsigned long long *mine = slots + size_t(set) * 6 * nb + blockIdx.x;
+    if (nb > 1 && threadIdx.x < 6) slots[size_t((1 - set) * 6 + threadIdx.x) * nb + blockIdx.x] = SLOT_EMPTY;
+    const size_t ng = len / G, tid = blockIdx.x * size_t(SWEEP_NT) + threadIdx.x, nth = nb * size_t(SWEEP_NT);
+    __shared__ double bcast;
+    float a[NG][G];
+    uint4 prev[NG], cur[NG];
+    auto group = [&](int m) { return tid + m * nth; };
+#pragma unroll
+    for (int m = 0; m < NG; ++m) {
+        prev[m] = cur[m] = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int e = 0; e < G; ++e) a[m][e] = 0.0f;
+        if (group(m) < ng) {
+            const float4 *q4 = reinterpret_cast<const float4 *>(q) + group(m) * (G / 4);
+#pragma unroll
+            for (int e = 0; e < G; e += 4) {
+                const float4 v = q4[e / 4];
+                a[m][e] = v.x; a[m][e + 1] = v.y; a[m][e + 2] = v.z; a[m][e + 3] = v.w;
+            }
+            cur[m] = __ldcs(reinterpret_cast<const uint4 *>(V) + group(m));
+        }
+    }
+    if ((stop && *stop) || (skip && *skip)) return;   // (read while the loads are under way)
+    float hf = 0.0f;   // coefficient of V_{i-1}
+    for (int i = 0; i <= j + 1; ++i) {
+        Acc<MODE> dot, ss;
+        const bool want_dot = i <= j, want_ss = (i == 0 && first_ss) || (i == j + 1 && last_ss);
+        // (groups past the end are zero and add nothing)
+#pragma unroll
+        for (int m = 0; m < NG; ++m) {
+            float p[G], c[G];
+            unpack_group(prev[m], p);
+            unpack_group(cur[m], c);
+#pragma unroll
+            for (int e = 0; e < G; ++e) a[m][e] = fmaf(-hf, p[e], a[m][e]);
+            if (want_dot) {
+#pragma unroll
+                for (int e = 0; e < G; ++e) dot.add(a[m][e], c[e], e);
+            }
+        }
+        if (want_ss) {
+#pragma unroll
+            for (int m = 0; m < NG; ++m) {
+#pragma unroll
+                for (int e = 0; e < G; ++e) ss.add(a[m][e], a[m][e], e);
+            }
+        }
+        if (i == j + 1) {   // q is final
+#pragma unroll
+            for (int m = 0; m < NG; ++m) {
+                if (group(m) < ng) {
+                    float4 *q4 = reinterpret_cast<float4 *>(q) + group(m) * (G / 4);
+#pragma unroll
+                    for (int e = 0; e < G; e += 4)
+                        q4[e / 4] = make_float4(a[m][e], a[m][e + 1], a[m][e + 2], a[m][e + 3]);
+                }
+            }
+            if (!want_ss) break;
+        }
+        double ta, tb;
+        block_total2<SWEEP_NT, MODE>(dot, ss, want_dot, want_ss, ta, tb);
+        if (nb > 1) {
+            unsigned long long *out = mine + (i % 3) * 2 * nb;
+            if (threadIdx.x == 0) {
+                if (want_dot) slot_put(out, ta);
+                if (want_ss) slot_put(out + nb, tb);
+            }
+        }
+        // the next vector comes in meanwhile
+#pragma unroll
+        for (int m = 0; m < NG; ++m) {
+            prev[m] = cur[m];
+            if (i < j && group(m) < ng) cur[m] = __ldcs(reinterpret_cast<const uint4 *>(V + size_t(i + 1) * ldv) + group(m));
+        }
+        if (nb > 1) {
+            if (i == j + 1 && blockIdx.x > 0) break;   // the last sum is block 0's
+            const unsigned long long *in = slots + size_t(set) * 6 * nb + (i % 3) * 2 * nb;
+            const bool ok = sum_partials([&](int b, double &va, double &vb) {
+                const bool ga = !want_dot || slot_get(in + b, va), gb = !want_ss || slot_get(in + nb + b, vb);
+                return ga && gb;
+            }, nb, want_dot, want_ss, ta, tb);
+            if (!ok) {
+                if (threadIdx.x == 0) st->status = ST_TIMEOUT;
+                return;
+            }
+            if (i > 0 && threadIdx.x < 2) mine[(((i - 1) % 3) * 2 + threadIdx.x) * nb] = SLOT_EMPTY;
+        }
+        if (threadIdx.x == 0) {
+            bcast = ta;
+            if (blockIdx.x == 0) {
+                if (want_dot) h[i] = ta;
+                if (want_ss) *(i == 0 ? first_ss : last_ss) = tb;
+            }
+        }
+        __syncthreads();
+        hf = float(bcast);
+    }
+    if (blockIdx.x == 0 && threadIdx.x < 32 && giv.H) givens_step(giv);
 }
 
 // *cnt = j when iterate j exists (j <= iterations done), else 0
@@ -485,35 +792,43 @@ __global__ void iterate_upto_kernel(const SolverState *st, int k, int *cnt) { *c
 
 // y = R_j^{-1} g_j for the first *cnt columns: the least-squares coefficients
 // of iterate x_j (R's first j columns and g's first j entries are final once
-// iteration j is done)
-__global__ void backsolve_count_kernel(const double *R, const double *g, double *y, const int *cnt, int k)
+// iteration j is done).  One warp, a column at a time: y_i, then row l < i
+// loses R[l][i] y_i; the next column's first 64 entries are loaded meanwhile.
+__global__ void backsolve_kernel(const double *__restrict__ R, const double *__restrict__ g, double *__restrict__ y,
+                                 const int *__restrict__ cnt, int k)
 {
-    const int it = *cnt;
-    const int ld = k + 1;
+    extern __shared__ double rhs[];   // k
+    const int it = min(*cnt, k);
+    const int ld = k + 1, lane = threadIdx.x;
+    for (int i = lane; i < it; i += 32) rhs[i] = g[i];
+    __syncwarp();
+    auto at = [&](int i, int l) { return i >= 0 && l <= i ? R[size_t(i) * ld + l] : 0.0; };
+    double n0 = at(it - 1, lane), n1 = at(it - 1, lane + 32), nd = at(it - 1, it - 1);
     for (int i = it - 1; i >= 0; --i) {
-        double acc = g[i];
-        for (int l = i + 1; l < it; ++l) acc -= R[size_t(l) * ld + i] * y[l];
-        const double d = R[size_t(i) * ld + i];
-        y[i] = d != 0.0 ? acc / d : 0.0;
+        const double c0 = n0, c1 = n1, d = nd;
+        n0 = at(i - 1, lane);
+        n1 = at(i - 1, lane + 32);
+        nd = at(i - 1, i - 1);
+        const double yi = d != 0.0 ? rhs[i] / d : 0.0;
+        if (lane == 0) y[i] = yi;
+        if (lane < i) rhs[lane] -= c0 * yi;
+        if (lane + 32 < i) rhs[lane + 32] -= c1 * yi;
+        for (int l = lane + 64; l < i; l += 32) rhs[l] -= R[size_t(i) * ld + l] * yi;
+        __syncwarp();
     }
+}
+
+static cudaError_t backsolve(const double *R, const double *g, double *y, const int *cnt, int k, cudaStream_t st)
+{
+    ProfScope prof(PK_SMALL, st);
+    backsolve_kernel<<<1, 32, size_t(k) * sizeof(double), st>>>(R, g, y, cnt, k);
+    return cudaGetLastError();
 }
 
 // err[j] = sqrt(err[j]) for the iterates that exist, -1 after them
 __global__ void err_finish_kernel(double *err, const SolverState *st, int k)
 {
     for (int j = 0; j <= k; ++j) err[j] = j <= st->iters ? sqrt(err[j]) : -1.0;
-}
-
-__global__ void backsolve_kernel(const double *R, const double *g, double *y, const SolverState *st, int k)
-{
-    const int it = st->iters;
-    const int ld = k + 1;
-    for (int i = it - 1; i >= 0; --i) {
-        double acc = g[i];
-        for (int l = i + 1; l < it; ++l) acc -= R[size_t(l) * ld + i] * y[l];
-        const double d = R[size_t(i) * ld + i];
-        y[i] = d != 0.0 ? acc / d : 0.0;
-    }
 }
 
 // x = sum_{i < count} y_i V_i ; count = *count_ptr when given, else k
@@ -579,7 +894,7 @@ __global__ void __launch_bounds__(RED_BLOCK) axpy_ratio_kernel(float *__restrict
         y[i] = v;
         ss.add(v, v);
     }
-    if (out_sumsq) grid_finish(0.0, ss.value(), partials, counter, nullptr, out_sumsq);
+    if (out_sumsq) grid_finish<RED_BLOCK, 1>(Acc<1>(), ss, partials, counter, nullptr, out_sumsq);
 }
 
 // p = s + (*num / *den) p
@@ -705,6 +1020,7 @@ struct GmresWs {
            *resid = nullptr, *y = nullptr, *partials = nullptr;
     double *err = nullptr;  // squared distances of the iterates to a reference image
     int *cnt = nullptr;     // iterate count for the error history
+    unsigned long long *slots = nullptr;   // the blocks' partial sums of a sweep kernel
     SolverState *st = nullptr;
     const void *vec(int i) const
     {
@@ -712,6 +1028,12 @@ struct GmresWs {
     }
     void *vec(int i) { return static_cast<char *>(V) + size_t(i) * ldv * (vbf16 ? 2 : 4); }
 };
+
+static cudaError_t gmres_state_reset(GmresWs &w, cudaStream_t s)
+{
+    cudaError_t e = cudaMemsetAsync(w.slots, 0xff, slots_count() * sizeof(unsigned long long), s);
+    return e == cudaSuccess ? cudaMemsetAsync(w.st, 0, sizeof(SolverState), s) : e;
+}
 
 // Bytes of the k+1 basis vectors of a BA (ab = false) or AB workspace.
 static size_t basis_bytes(const GeomDev &g, int k, bool ab)
@@ -751,6 +1073,7 @@ static bool carve_gmres(Arena &ar, const GeomDev &g, int k, bool ab, int b_kind,
     w.partials = ar.take<double>(partials_count());
     w.err = ar.take<double>(ld);
     w.cnt = ar.take<int>(1);
+    w.slots = ar.take<unsigned long long>(slots_count());
     w.st = ar.take<SolverState>(1);
     return w.st != nullptr;
 }
@@ -843,6 +1166,62 @@ static cudaError_t staged_sweep(Stager &sg, int mode, bool vbf16, float *q, int 
     return e;
 }
 
+// One MGS sweep (passes i = 0..j+1) over a device basis: the sweep kernel where
+// the vectors fit it, with the Givens step at its end when `giv` is given
+// (givens_done), else a launch a pass.
+template <int MODE, typename TB>
+static cudaError_t launch_sweep(GmresWs &w, float *q, int j, double *hcol, size_t len, double *first_ss,
+                                double *last_ss, int set, const int *stop, const int *skip, const GivensArgs *giv,
+                                cudaStream_t s)
+{
+    const TB *V = static_cast<const TB *>(w.V);
+    GivensArgs g{};
+    if (giv) g = *giv;
+    void *args[] = {&q, &V, &w.ldv, &j, &len, &hcol, &first_ss, &last_ss, &w.slots, &set, &stop, &skip, &w.st, &g};
+    ProfScope prof(PK_MGS, s);
+    const unsigned blocks = sweep_blocks(len);
+    if (blocks == 1) {   // nobody to wait for
+        mgs_sweep_kernel<MODE, TB, 16><<<1, SWEEP_NT, 0, s>>>(q, V, w.ldv, j, len, hcol, first_ss, last_ss, w.slots, set,
+                                                              stop, skip, w.st, g);
+        return cudaGetLastError();
+    }
+    const void *kernel = len <= size_t(blocks) * SWEEP_NT * 16
+                             ? reinterpret_cast<const void *>(mgs_sweep_kernel<MODE, TB, 16>)
+                             : reinterpret_cast<const void *>(mgs_sweep_kernel<MODE, TB, SWEEP_ELEMS>);
+    return cudaLaunchCooperativeKernel(kernel, dim3(blocks), dim3(SWEEP_NT), args, 0, s);
+}
+
+static cudaError_t device_sweep(GmresWs &w, int mode, float *q, int j, double *hcol, size_t len, double *first_ss,
+                                double *last_ss, int set, const int *stop, const int *skip, const GivensArgs *giv,
+                                bool &givens_done, cudaStream_t s)
+{
+    // the kernel reads 16-byte groups (the basis' stride is a multiple of 64 elements, its start 256-byte aligned)
+    if (len <= sweep_max() && len % (w.vbf16 ? 8 : 4) == 0 && reinterpret_cast<uintptr_t>(q) % 16 == 0) {
+        cudaError_t e;
+        if (w.vbf16)
+            e = mode == 0 ? launch_sweep<0, __nv_bfloat16>(w, q, j, hcol, len, first_ss, last_ss, set, stop, skip, giv, s)
+                          : launch_sweep<1, __nv_bfloat16>(w, q, j, hcol, len, first_ss, last_ss, set, stop, skip, giv, s);
+        else
+            e = mode == 0 ? launch_sweep<0, float>(w, q, j, hcol, len, first_ss, last_ss, set, stop, skip, giv, s)
+                          : launch_sweep<1, float>(w, q, j, hcol, len, first_ss, last_ss, set, stop, skip, giv, s);
+        if (e == cudaSuccess) {
+            givens_done = giv != nullptr;
+            return e;
+        }
+        // not all blocks can be resident (a device with part of its SMs): a launch a pass gives the same sums
+        if (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorLaunchOutOfResources &&
+            e != cudaErrorNotSupported)
+            return e;
+        cudaGetLastError();
+    }
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i <= j + 1 && e == cudaSuccess; ++i)
+        e = mgs_pass_typed(mode, w.vbf16, q, i > 0 ? w.vec(i - 1) : nullptr, i > 0 ? hcol + (i - 1) : nullptr,
+                           i <= j ? w.vec(i) : nullptr, len, w.partials, &w.st->counter, i <= j ? hcol + i : nullptr,
+                           i == 0 ? first_ss : (i == j + 1 ? last_ss : nullptr), stop, skip, s);
+    return e;
+}
+
 // Enqueues the MGS sweep of iteration j (the new vector q against
 // V_0..V_j) and its Givens step.
 static cudaError_t arnoldi_orthogonalise(GmresWs &w, float *q, int j, int k, size_t len, const ct_solve_opts &o,
@@ -865,36 +1244,22 @@ static cudaError_t arnoldi_orthogonalise(GmresWs &w, float *q, int j, int k, siz
             if (e != cudaSuccess) return e;
             H2s = w.H2;
         }
-        { ProfScope prof(PK_SMALL, s); givens_kernel<<<1, 1, 0, s>>>(j, k, w.H, H2s, w.R, w.cs, w.sn, w.g, w.resid, w.st, o.tol); }
+        { ProfScope prof(PK_SMALL, s); givens_kernel<<<1, 32, 0, s>>>(GivensArgs{j, k, w.H, H2s, w.R, w.cs, w.sn, w.g, w.resid, w.st, o.tol}); }
         return cudaGetLastError();
     }
-    for (int i = 0; i <= j + 1 && e == cudaSuccess; ++i) {
-        const void *vprev = i > 0 ? w.vec(i - 1) : nullptr;
-        const double *hprev = i > 0 ? hcol + (i - 1) : nullptr;
-        const void *vcur = i <= j ? w.vec(i) : nullptr;
-        double *odot = i <= j ? hcol + i : nullptr;
-        double *oss = i == 0 ? &w.st->ref_sumsq : (i == j + 1 ? &w.st->sumsq : nullptr);
-        e = mgs_pass_typed(o.dot_mode, w.vbf16, q, vprev, hprev, vcur, len, w.partials, ctr, odot, oss, stop,
-                           nullptr, s);
-    }
-    if (e != cudaSuccess) return e;
-    const double *H2 = nullptr;
-    if (o.reorth) {
+    GivensArgs giv{j, k, w.H, o.reorth ? w.H2 : nullptr, w.R, w.cs, w.sn, w.g, w.resid, w.st, o.tol};
+    bool givens_done = false;
+    if (e == cudaSuccess)
+        e = device_sweep(w, o.dot_mode, q, j, hcol, len, &w.st->ref_sumsq, &w.st->sumsq, o.reorth ? 0 : j & 1, stop,
+                         nullptr, o.reorth ? nullptr : &giv, givens_done, s);
+    if (e == cudaSuccess && o.reorth) {
         { ProfScope prof(PK_SMALL, s); reorth_decide_kernel<<<1, 1, 0, s>>>(w.st); }
-        const int *skip = &w.st->reorth_skip;
-        for (int i = 0; i <= j + 1 && e == cudaSuccess; ++i) {
-            const void *vprev = i > 0 ? w.vec(i - 1) : nullptr;
-            const double *hprev = i > 0 ? w.H2 + (i - 1) : nullptr;
-            const void *vcur = i <= j ? w.vec(i) : nullptr;
-            double *odot = i <= j ? w.H2 + i : nullptr;
-            double *oss = i == j + 1 ? &w.st->sumsq : nullptr;
-            e = mgs_pass_typed(o.dot_mode, w.vbf16, q, vprev, hprev, vcur, len, w.partials, ctr, odot, oss, stop,
-                               skip, s);
-        }
-        if (e != cudaSuccess) return e;
-        H2 = w.H2;
+        bool unused = false;
+        e = device_sweep(w, o.dot_mode, q, j, w.H2, len, nullptr, &w.st->sumsq, 1, stop, &w.st->reorth_skip, nullptr,
+                         unused, s);
     }
-    { ProfScope prof(PK_SMALL, s); givens_kernel<<<1, 1, 0, s>>>(j, k, w.H, H2, w.R, w.cs, w.sn, w.g, w.resid, w.st, o.tol); }
+    if (e != cudaSuccess || givens_done) return e;
+    { ProfScope prof(PK_SMALL, s); givens_kernel<<<1, 32, 0, s>>>(giv); }
     return cudaGetLastError();
 }
 
@@ -910,6 +1275,8 @@ static ct_status finish_solve(SolverState *st_dev, const double *resid_dev, int 
     if (iters_done) *iters_done = hst.iters;
     if (hst.status == ST_NONFINITE)
         return set_error(CT_ENONFINITE, "%s: a norm became NaN/Inf after %d iterations", who, hst.iters);
+    if (hst.status == ST_TIMEOUT)
+        return set_error(CT_ETIMEOUT, "%s: a wait between blocks ran out after %d iterations", who, hst.iters);
     if (hst.status == ST_LUCKY) return CT_BREAKDOWN_LUCKY;
     return CT_OK;
 }
@@ -929,7 +1296,7 @@ static ct_status open_ws(Arena &ar, size_t bytes, const ct_solve_opts &o, cudaSt
 static cudaError_t ba_start(const GeomDev &g, GmresWs &w, const float *b, int kmax, size_t n,
                             const ct_solve_opts &o, cudaStream_t s)
 {
-    cudaError_t e = cudaMemsetAsync(w.st, 0, sizeof(SolverState), s);
+    cudaError_t e = gmres_state_reset(w, s);
     // zero the padded sinogram once: its border is never written afterwards
     if (e == cudaSuccess)
         e = cudaMemsetAsync(w.ob.ypad, 0, padded_sino_floats(g) * sizeof(float), s);
@@ -1000,8 +1367,9 @@ static ct_status bagmres(const ct_geom *geom, const float *b, int k, float *x, d
             {
                 ProfScope prof(PK_SMALL, s);
                 iterate_count_kernel<<<1, 1, 0, s>>>(w.st, j, w.cnt);
-                backsolve_count_kernel<<<1, 1, 0, s>>>(w.R, w.g, w.y, w.cnt, k);
             }
+            e = backsolve(w.R, w.g, w.y, w.cnt, k, s);
+            if (e != cudaSuccess) break;
             e = w.vbf16 ? combine_t(static_cast<const __nv_bfloat16 *>(w.V), w.ldv, k, n, w.y, w.cnt, x, s)
                         : combine(static_cast<const float *>(w.V), w.ldv, k, n, w.y, w.cnt, x, s);
             if (e == cudaSuccess) {
@@ -1018,10 +1386,7 @@ static ct_status bagmres(const ct_geom *geom, const float *b, int k, float *x, d
         if (e == cudaSuccess && err_hist)
             e = cudaMemcpyAsync(err_hist, w.err, sizeof(double) * (k + 1), cudaMemcpyDeviceToHost, s);
     }
-    if (e == cudaSuccess) {
-        { ProfScope prof(PK_SMALL, s); backsolve_kernel<<<1, 1, 0, s>>>(w.R, w.g, w.y, w.st, k); }
-        e = cudaGetLastError();
-    }
+    if (e == cudaSuccess) e = backsolve(w.R, w.g, w.y, &w.st->iters, k, s);
     if (e == cudaSuccess)
         e = w.vbf16 ? combine_t(static_cast<const __nv_bfloat16 *>(w.V), w.ldv, k, n, w.y, &w.st->iters, x, s)
                     : combine(static_cast<const float *>(w.V), w.ldv, k, n, w.y, &w.st->iters, x, s);
@@ -1122,7 +1487,7 @@ static ct_status abgmres(const ct_geom *geom, const float *b, int k, float *x, d
     carve_gmres(ar, g, k, true, o.b_kind, w);
     float *Vf = static_cast<float *>(w.V);   // data-space basis, FP32
     const int *stop = &w.st->status;
-    cudaError_t e = cudaMemsetAsync(w.st, 0, sizeof(SolverState), s);
+    cudaError_t e = gmres_state_reset(w, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(w.ob.ypad, 0, padded_sino_floats(g) * sizeof(float), s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(Vf, b, m * sizeof(float), cudaMemcpyDeviceToDevice, s);
     if (e == cudaSuccess)
@@ -1141,10 +1506,7 @@ static ct_status abgmres(const ct_geom *geom, const float *b, int k, float *x, d
         if (e == cudaSuccess) e = launch_project_A(g, w.ob.Xc, w.ob.Yc, q, plain_layout(g), stop, s);
         if (e == cudaSuccess) e = arnoldi_orthogonalise(w, q, j, k, m, o, s);
     }
-    if (e == cudaSuccess) {
-        { ProfScope prof(PK_SMALL, s); backsolve_kernel<<<1, 1, 0, s>>>(w.R, w.g, w.y, w.st, k); }
-        e = cudaGetLastError();
-    }
+    if (e == cudaSuccess) e = backsolve(w.R, w.g, w.y, &w.st->iters, k, s);
     // u = V y (data space) into the last basis slot, then x = B u
     float *u = Vf + size_t(k) * w.ldv;
     if (e == cudaSuccess) e = combine(Vf, w.ldv, k, m, w.y, &w.st->iters, u, s);
@@ -1191,6 +1553,7 @@ static void carve_vjp(Arena &ar, const GeomDev &g, int k, int b_kind, VjpWs &w)
     w.gm.resid = ar.take<double>(ld);
     w.gm.y = ar.take<double>(k);
     w.gm.partials = ar.take<double>(partials_count());
+    w.gm.slots = ar.take<unsigned long long>(slots_count());
     w.gm.st = ar.take<SolverState>(1);
 }
 
@@ -1242,7 +1605,7 @@ static ct_status bagmres_vjp(const ct_geom *geom, const float *gx, int k, float 
     const unsigned vb = red_blocks(n);
     float *Vf = static_cast<float *>(gm.V);   // image-space basis, FP32
     float *sino = o.b_kind == CT_B_FBP ? w.tf : w.t;   // B^T v lands here
-    cudaError_t e = cudaMemsetAsync(gm.st, 0, sizeof(SolverState), s);
+    cudaError_t e = gmres_state_reset(gm, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(Vf, gx, n * sizeof(float), cudaMemcpyDeviceToDevice, s);
     if (e == cudaSuccess)
         e = mgs_pass(o.dot_mode, Vf, nullptr, nullptr, nullptr, n, gm.partials, &gm.st->counter, nullptr,
@@ -1264,10 +1627,7 @@ static ct_status bagmres_vjp(const ct_geom *geom, const float *gx, int k, float 
         if (e == cudaSuccess) e = launch_project_At(g, sino, q, w.Xa, w.Ya, stop, s);
         if (e == cudaSuccess) e = arnoldi_orthogonalise(gm, q, j, k, n, o, s);
     }
-    if (e == cudaSuccess) {
-        { ProfScope prof(PK_SMALL, s); backsolve_kernel<<<1, 1, 0, s>>>(gm.R, gm.g, gm.y, gm.st, k); }
-        e = cudaGetLastError();
-    }
+    if (e == cudaSuccess) e = backsolve(gm.R, gm.g, gm.y, &gm.st->iters, k, s);
     float *z = Vf + size_t(k) * gm.ldv;
     if (e == cudaSuccess) e = combine(Vf, gm.ldv, k, n, gm.y, &gm.st->iters, z, s);
     if (e == cudaSuccess) e = apply_Bt(g, o.b_kind, z, w.t, w.tf, gb, nullptr, s);
@@ -1780,10 +2140,11 @@ ct_status ct_bagmres_state_extend(ct_gmres_state *state, int k, float *x_out_dev
             e = ba_iteration(g, w, j, state->kmax, n, state->o, s, sg);
     // x = V_c y_c with c = min(k, iterations done)
     if (e == cudaSuccess) {
-        ProfScope prof(PK_SMALL, s);
-        iterate_upto_kernel<<<1, 1, 0, s>>>(w.st, k, w.cnt);
-        backsolve_count_kernel<<<1, 1, 0, s>>>(w.R, w.g, w.y, w.cnt, state->kmax);
-        e = cudaGetLastError();
+        {
+            ProfScope prof(PK_SMALL, s);
+            iterate_upto_kernel<<<1, 1, 0, s>>>(w.st, k, w.cnt);
+        }
+        e = backsolve(w.R, w.g, w.y, w.cnt, state->kmax, s);
     }
     SolverState hst;
     std::vector<double> hres(size_t(k) + 1);
@@ -1809,6 +2170,9 @@ ct_status ct_bagmres_state_extend(ct_gmres_state *state, int k, float *x_out_dev
     if (iters_done) *iters_done = hst.iters < k ? hst.iters : k;
     if (hst.status == ST_NONFINITE)
         return set_error(CT_ENONFINITE, "ct_bagmres_state_extend: a norm became NaN/Inf after %d iterations",
+                         hst.iters);
+    if (hst.status == ST_TIMEOUT)
+        return set_error(CT_ETIMEOUT, "ct_bagmres_state_extend: a wait between blocks ran out after %d iterations",
                          hst.iters);
     if (hst.status == ST_LUCKY) return CT_BREAKDOWN_LUCKY;
     return CT_OK;
@@ -1941,6 +2305,7 @@ ct_status ct_gmres_state_load(const ct_geom *geom, const char *path, int kmax, i
     if (e == cudaSuccess) e = cudaMemset(w.R, 0, sizeof(double) * ld * kmax);
     if (e == cudaSuccess) e = cudaMemset(w.g, 0, sizeof(double) * ld);
     if (e == cudaSuccess) e = cudaMemset(w.ob.ypad, 0, padded_sino_floats(geom->g) * sizeof(float));
+    if (e == cudaSuccess) e = cudaMemset(w.slots, 0xff, slots_count() * sizeof(unsigned long long));
     for (int j = 0; j < kd && e == cudaSuccess; ++j) {
         e = cudaMemcpy(w.H + j * ld, H.data() + j * rows, rows * sizeof(double), cudaMemcpyHostToDevice);
         if (e == cudaSuccess)
