@@ -242,8 +242,11 @@ struct Arena {
         return p;
     }
 };
+// Stream-ordered memory from the current device's scratch pool (the default
+// pool where no geometry lives); freed with cudaFreeAsync.
+cudaError_t scratch_alloc(void **ptr, size_t bytes, cudaStream_t stream);
 // Opens an arena of `bytes`: uses the caller's workspace when given (and
-// large enough), else cudaMallocAsync on `stream`.
+// large enough), else scratch memory in the order of `stream`.
 ct_status arena_open(Arena &a, size_t bytes, void *workspace, size_t workspace_bytes,
                      cudaStream_t stream);
 void arena_close(Arena &a);

@@ -1423,7 +1423,7 @@ static ct_status bagmres_restarted(const ct_geom *geom, const float *b, int m, i
     const size_t n = geom->n, mm = geom->m;
     const size_t copies = size_t(g.nzp) * g.nx * g.pitchX + size_t(g.nzp) * g.ny * g.pitchY;
     float *buf = nullptr;
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void **>(&buf), sizeof(float) * (copies + 2 * mm + n), s);
+    cudaError_t e = scratch_alloc(reinterpret_cast<void **>(&buf), sizeof(float) * (copies + 2 * mm + n), s);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return set_error(CT_ENOMEM, "ct_bagmres_restarted: %zu bytes of scratch: %s",
