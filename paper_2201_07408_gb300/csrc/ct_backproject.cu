@@ -667,62 +667,69 @@ cudaError_t launch_voxel_B(const GeomDev &g, const float *ypad, float *x, const 
 }
 
 // ---------------------------------------------------------------------------
-// y += B_un^T x: voxel splatting with the same weights (FP32 atomics into
-// the plain sinogram, bounds-checked).
+// y = B_un^T x: voxel splatting with the same weights.  FP32 reductions into an
+// accumulator with a border column on both sides, Y[view][v][u + 1], kept twice
+// so that the two pixels of a row go as one request (add_pair); a last pass adds
+// the two up.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void splat(float *y, const GeomDev &g, int s, int iu, int iv, float val)
+static size_t bt_floats(const GeomDev &g) { return pair_acc_floats(size_t(g.n_views) * g.nv * (g.nu + 2)); }
+size_t bt_scratch_floats(const GeomDev &g) { return 2 * bt_floats(g); }
+
+// the pair (u0, u0 + 1), u0 in [-1, nu - 1], of detector row v; rows off the detector are not entries of B
+__device__ __forceinline__ void splat(const GeomDev &g, float *acc, size_t odd, int s, int u0, int v, float lo,
+                                      float hi)
 {
-    if (iu < 0 || iu >= g.nu || iv < 0 || iv >= g.nv || val == 0.0f) return;
-    atomicAdd(y + (size_t(s) * g.nv + iv) * g.nu + iu, val);
+    if (v < 0 || v >= g.nv) return;
+    add_pair(acc, odd, (size_t(s) * g.nv + v) * (g.nu + 2) + u0 + 1, lo, hi);
 }
 
+// `split` blocks share the views of a voxel
 __global__ void __launch_bounds__(B_BX *B_BY) voxel_Bt_kernel(GeomDev g, const float *__restrict__ x,
-                                                              float *__restrict__ y,
+                                                              float *__restrict__ acc, size_t odd, int split,
                                                               const int *__restrict__ stop)
 {
     if (stop && *stop) return;
     const int ix = blockIdx.x * B_BX + threadIdx.x;
     const int iy = blockIdx.y * B_BY + threadIdx.y;
-    const int iz = blockIdx.z;
+    const int iz = blockIdx.z / split;
     if (ix >= g.nx || iy >= g.ny) return;
     const float xv = x[(size_t(iz) * g.ny + iy) * g.nx + ix];
     if (xv == 0.0f) return;
     const float xc = (float(ix) - g.cx) * g.vox;
     const float yc = (float(iy) - g.cy) * g.vox;
     const float zc = (float(iz) - g.cz) * g.vox;
-    for (int s = 0; s < g.n_views; ++s) {
+#pragma unroll 4
+    for (int s = blockIdx.z % split; s < g.n_views; s += split) {
         const ColumnView c = column_view(g, s, xc, yc, zc);
         if (c.skip) continue;
         const float fv = c.fv0;
         const float v0f = floorf(fv);
         const float wv = fv - v0f;
         if (v0f < -1.0f || v0f > float(g.nv - 1)) continue;
-        const int v0 = int(v0f);
-        const int u0 = c.col - PAD_U;
-        splat(y, g, s, u0, v0, xv * c.a0 * (1.0f - wv));
-        splat(y, g, s, u0 + 1, v0, xv * c.a1 * (1.0f - wv));
-        splat(y, g, s, u0, v0 + 1, xv * c.a0 * wv);
-        splat(y, g, s, u0 + 1, v0 + 1, xv * c.a1 * wv);
+        const int v0 = int(v0f), u0 = c.col - PAD_U;
+        const float lo = xv * (1.0f - wv), hi = xv * wv;
+        if (lo != 0.0f) splat(g, acc, odd, s, u0, v0, lo * c.a0, lo * c.a1);
+        if (hi != 0.0f) splat(g, acc, odd, s, u0, v0 + 1, hi * c.a0, hi * c.a1);
     }
 }
 
-// y += B_un^T x for 3D scans by splatting voxel runs.  Per view the lanes
+// 3D scans by splatting voxel runs.  Per view the lanes
 // run across the central ray (along x when u moves faster with x than with
-// y), so a warp's atomics land on different pixels along u.  A thread's ZC
+// y), so a warp's reductions land on different pixels along u.  A thread's ZC
 // voxels (consecutive z of one column) share the column's u and u-weights,
 // and their rows increase with z: contributions to one row are summed in
-// registers and added with two atomics (pixels u0, u0 + 1) when the run
+// registers and added (pixels u0, u0 + 1) when the run
 // moves past the row; the flushes are predicated and the running sums
 // selected, so lanes whose runs change rows at different slices share one
-// copy of the atomics.  One launch per lane orientation, in 256-thread
+// copy of the reductions.  One launch per lane orientation, in 256-thread
 // blocks (MINB resident per SM): XL takes the views whose lanes run along x
-// on 32 x 8 column tiles, !XL those along y on 8 x 32 tiles.  Against one
-// launch of 1024-thread blocks with both orientations (two value sets per
-// thread): 3.23 against 4.05 ms on phantom projections at 256^3, 16.5
-// against 17.0 ms dense.
+// on 32 x 8 column tiles, !XL those along y on 8 x 32 tiles.  `split` blocks
+// share a run's views (small volumes).  Dense data, 256^3: 16.5 ms with a
+// request a pixel, 12.2 ms with one a pair (runs of 16 slices 11.7 ms, but 10 %
+// slower at 128^3: 0.66 -> 0.73 ms); 44^3 0.129 -> 0.043 ms.
 template <int ZC, bool XL, int MINB>
 __global__ void __launch_bounds__(256, MINB) voxel_Bt_slab_kernel(GeomDev g, const float *__restrict__ x,
-                                                                  float *__restrict__ y,
+                                                                  float *__restrict__ acc, size_t odd, int split,
                                                                   const int *__restrict__ stop)
 {
     if (stop && *stop) return;
@@ -733,7 +740,7 @@ __global__ void __launch_bounds__(256, MINB) voxel_Bt_slab_kernel(GeomDev g, con
     for (int i = tid; i < 2 * g.n_views; i += 256) bt_views[i] = __ldg(vt + i);
     const int ax = XL ? blockIdx.x * 32 + l : blockIdx.x * 8 + w;
     const int ay = XL ? blockIdx.y * 8 + w : blockIdx.y * 32 + l;
-    const int Z0 = blockIdx.z * ZC;
+    const int Z0 = (blockIdx.z / split) * ZC;
     float xa[ZC];
     bool anya = false;
 #pragma unroll
@@ -746,7 +753,7 @@ __global__ void __launch_bounds__(256, MINB) voxel_Bt_slab_kernel(GeomDev g, con
     const float zfirst = (float(Z0) - g.cz) * g.vox;
     __syncthreads();
     if (!anya) return;
-    for (int s = 0; s < g.n_views; ++s) {
+    for (int s = blockIdx.z % split; s < g.n_views; s += split) {
         const float4 p = bt_views[2 * s], q = bt_views[2 * s + 1];
         const bool xl = fabsf(p.w) > fabsf(q.x);
         if (xl != XL) continue;
@@ -755,8 +762,7 @@ __global__ void __launch_bounds__(256, MINB) voxel_Bt_slab_kernel(GeomDev g, con
         const int u0 = c.col - PAD_U;
         auto flush = [&](int v, float r) {
             if (r == 0.0f) return;
-            splat(y, g, s, u0, v, r * c.a0);
-            splat(y, g, s, u0 + 1, v, r * c.a1);
+            splat(g, acc, odd, s, u0, v, r * c.a0, r * c.a1);
         };
         int vc = 0;
         float acc_lo = 0.0f, acc_hi = 0.0f;
@@ -786,32 +792,64 @@ __global__ void __launch_bounds__(256, MINB) voxel_Bt_slab_kernel(GeomDev g, con
     }
 }
 
+// y = the sum of the accumulator's two copies, without the border columns
+__global__ void __launch_bounds__(256) unpair_sino_kernel(const float *__restrict__ acc, size_t odd, int nu,
+                                                          size_t rows, float *__restrict__ y,
+                                                          const int *__restrict__ stop)
+{
+    if (stop && *stop) return;
+    for (size_t r = blockIdx.x * size_t(8) + threadIdx.y; r < rows; r += size_t(gridDim.x) * 8)
+        for (int u = threadIdx.x; u < nu; u += 32) {
+            const size_t e = r * (nu + 2) + u + 1;
+            y[r * nu + u] = acc[e] + acc[odd + e + 1];
+        }
+}
+
 template <int ZC, int MINB>
-static cudaError_t launch_voxel_Bt_slab(const GeomDev &g, const float *x, float *y, const int *stop, cudaStream_t st)
+static cudaError_t launch_voxel_Bt_slab(const GeomDev &g, const float *x, float *acc, size_t odd, const int *stop,
+                                        cudaStream_t st)
 {
     const size_t smem = size_t(g.n_views) * 2 * sizeof(float4);
     cudaError_t e = raise_dyn_smem(reinterpret_cast<const void *>(voxel_Bt_slab_kernel<ZC, true, MINB>), smem);
     if (e == cudaSuccess)
         e = raise_dyn_smem(reinterpret_cast<const void *>(voxel_Bt_slab_kernel<ZC, false, MINB>), smem);
     if (e != cudaSuccess) return e;
+    const int runs = (g.nz + ZC - 1) / ZC;
     dim3 block(32, 8);
-    dim3 gx((g.nx + 31) / 32, (g.ny + 7) / 8, (g.nz + ZC - 1) / ZC);
-    dim3 gy((g.nx + 7) / 8, (g.ny + 31) / 32, (g.nz + ZC - 1) / ZC);
-    voxel_Bt_slab_kernel<ZC, true, MINB><<<gx, block, smem, st>>>(g, x, y, stop);
-    voxel_Bt_slab_kernel<ZC, false, MINB><<<gy, block, smem, st>>>(g, x, y, stop);
+    dim3 gx((g.nx + 31) / 32, (g.ny + 7) / 8, runs);
+    dim3 gy((g.nx + 7) / 8, (g.ny + 31) / 32, runs);
+    // small volumes: blocks share a run's views until the grid has 4 blocks an SM
+    int split = 1;
+    while (split < 16 && size_t(gx.x) * gx.y * runs * split * 2 <= size_t(num_sms()) * 4) split *= 2;
+    gx.z *= split;
+    gy.z *= split;
+    voxel_Bt_slab_kernel<ZC, true, MINB><<<gx, block, smem, st>>>(g, x, acc, odd, split, stop);
+    voxel_Bt_slab_kernel<ZC, false, MINB><<<gy, block, smem, st>>>(g, x, acc, odd, split, stop);
     return cudaGetLastError();
 }
 
-cudaError_t launch_voxel_Bt(const GeomDev &g, const float *x, float *y, const int *stop, cudaStream_t st)
+cudaError_t launch_voxel_Bt(const GeomDev &g, const float *x, float *y, float *acc, const int *stop,
+                            cudaStream_t st)
 {
     ProfScope prof(PK_VOXEL_BT, st);
+    const size_t odd = bt_floats(g), rows = size_t(g.n_views) * g.nv;
+    cudaError_t e = cudaMemsetAsync(acc, 0, 2 * odd * sizeof(float), st);
+    if (e != cudaSuccess) return e;
     if (g.nz < B_ZC) {   // 2D, or a slab thinner than a z run: one voxel per thread
         dim3 block(B_BX, B_BY);
         dim3 grid((g.nx + B_BX - 1) / B_BX, (g.ny + B_BY - 1) / B_BY, g.nz);
-        voxel_Bt_kernel<<<grid, block, 0, st>>>(g, x, y, stop);
-        return cudaGetLastError();
+        int split = 1;
+        while (split < 32 && size_t(grid.x) * grid.y * g.nz * split * 2 <= size_t(num_sms()) * 8) split *= 2;
+        grid.z *= split;
+        voxel_Bt_kernel<<<grid, block, 0, st>>>(g, x, acc, odd, split, stop);
+        e = cudaGetLastError();
+    } else {
+        e = launch_voxel_Bt_slab<B_ZC, 4>(g, x, acc, odd, stop, st);
     }
-    return launch_voxel_Bt_slab<B_ZC, 4>(g, x, y, stop, st);
+    if (e != cudaSuccess) return e;
+    const unsigned blocks = unsigned(std::min<size_t>((rows + 7) / 8, size_t(num_sms()) * 16));
+    unpair_sino_kernel<<<blocks, dim3(32, 8), 0, st>>>(acc, odd, g.nu, rows, y, stop);
+    return cudaGetLastError();
 }
 
 }  // namespace ct
@@ -867,19 +905,15 @@ extern "C" ct_status ct_adjoint_Bt(const ct_geom *geom, const float *x_dev, floa
     if (b_kind != CT_B_UN && b_kind != CT_B_FBP)
         return set_error(CT_EINVAL, "ct_adjoint_Bt: unknown b_kind %d", b_kind);
     const GeomDev &g = geom->g;
-    if (b_kind == CT_B_UN) {
-        CT_CUDA(cudaMemsetAsync(y_dev, 0, geom->m * sizeof(float), st));
-        cudaError_t e = launch_voxel_Bt(g, x_dev, y_dev, nullptr, st);
-        if (e != cudaSuccess) return cuda_error(e, "ct_adjoint_Bt launch");
-        return CT_OK;
-    }
+    const bool fbp = b_kind == CT_B_FBP;
+    const size_t acc_bytes = Arena::align(bt_scratch_floats(g) * sizeof(float));
     Arena ar;
-    ct_status rc = arena_open(ar, Arena::align(geom->m * sizeof(float)), nullptr, 0, st);
+    ct_status rc = arena_open(ar, acc_bytes + (fbp ? Arena::align(geom->m * sizeof(float)) : 0), nullptr, 0, st);
     if (rc != CT_OK) return rc;
-    float *tmp = ar.take<float>(geom->m);
-    cudaError_t e = cudaMemsetAsync(tmp, 0, geom->m * sizeof(float), st);
-    if (e == cudaSuccess) e = launch_voxel_Bt(g, x_dev, tmp, nullptr, st);
-    if (e == cudaSuccess) e = launch_ramp(g, tmp, y_dev, plain_layout(g), true, nullptr, st);
+    float *acc = ar.take<float>(bt_scratch_floats(g));
+    float *dst = fbp ? ar.take<float>(geom->m) : y_dev;
+    cudaError_t e = launch_voxel_Bt(g, x_dev, dst, acc, nullptr, st);
+    if (e == cudaSuccess && fbp) e = launch_ramp(g, dst, y_dev, plain_layout(g), true, nullptr, st);
     arena_close(ar);
     if (e != cudaSuccess) return cuda_error(e, "ct_adjoint_Bt launch");
     return CT_OK;

@@ -309,7 +309,7 @@ ct_status ct_geom_create(const ct_geom_desc *d, ct_geom **out)
     k.a_zsafe = 1;
     if (cone) {
         double smin = 1e300, smax = -1e300;
-        const int nv_run = (d->nv + A_VR_MAX - 1) / A_VR_MAX * A_VR_MAX;
+        const int nv_run = (d->nv + A_VR - 1) / A_VR * A_VR;
         const double vmax = std::max(0.5 * (d->nv - 1), nv_run - 1 - 0.5 * (d->nv - 1)) * d->dv_mm;
         for (int s = 0; s < d->n_views; ++s) {
             double th = d->angle_start_rad + double(s) * d->angle_span_rad / double(d->n_views);

@@ -19,19 +19,8 @@ constexpr int PAD_A = 2;   // voxels, around the in-plane and z axes of the plan
 constexpr int PAD_U = 1;   // pixels, both ends of each detector row
 constexpr int PAD_V = 2;   // rows, above and below each view
 // rays per projector thread along a detector column (the last group of a
-// column runs past nv when nv is not a multiple; those rays are discarded):
-// A_VR for A, AT_VR for its exact transpose (tuning; at 256^3, 16 rays took
-// A 5.31 / 5.74 ms with FP32 / bf16 copies and A^T 5.74 ms, against 5.39 /
-// 6.16 ms and 6.06 ms with 8 rays, and A 8.16 / 9.01 ms with 12)
-#ifndef CT_A_VR
-#define CT_A_VR 16
-#endif
-#ifndef CT_AT_VR
-#define CT_AT_VR 16
-#endif
-constexpr int A_VR = CT_A_VR;
-constexpr int AT_VR = CT_AT_VR;
-constexpr int A_VR_MAX = A_VR > AT_VR ? A_VR : AT_VR;
+// column runs past nv when nv is not a multiple; those rays are discarded)
+constexpr int A_VR = 16;
 // consecutive z slices per thread: B_ZC_SLAB for the 3D back-projector
 // (voxel_B_slab_kernel), B_ZC for its transpose.  The last run of a column
 // may pass nz: those slices are computed and discarded, and the padded
@@ -302,9 +291,10 @@ cudaError_t launch_plane_copies(const GeomDev &g, const float *vol, const double
 // reads Yc only), written in `lay`.
 cudaError_t launch_project_A(const GeomDev &g, const float *Xc, const float *Yc, float *y,
                             SinoLayout lay, const int *stop, cudaStream_t st);
-// x = A^T y (overwritten); y in plain layout.  Xa, Ya: accumulators of the
-// projector's copy sizes (contents overwritten).
-cudaError_t launch_project_At(const GeomDev &g, const float *y, float *x, float *Xa, float *Ya, const int *stop,
+// x = A^T y (overwritten); y in plain layout.  acc: at_scratch_floats(g) floats
+// (none for the line-intersection projector), 256-byte aligned, contents overwritten.
+size_t at_scratch_floats(const GeomDev &g);
+cudaError_t launch_project_At(const GeomDev &g, const float *y, float *x, float *acc, const int *stop,
                              cudaStream_t st);
 // the line-intersection projector and its transpose (ct_siddon.cu); x overwritten
 cudaError_t launch_siddon_A(const GeomDev &g, const float *Yc, float *y, SinoLayout lay, const int *stop,
@@ -327,9 +317,24 @@ enum QuadForm { QUAD_ROWDIFF, QUAD_CORNERS };
 // launch_ramp, QUAD_CORNERS after a projector wrote it with store_sino.
 cudaError_t launch_voxel_B(const GeomDev &g, const float *ypad, float *x, const int *stop,
                            cudaStream_t st, QuadForm form);
-// y += B_un^T x (y plain, zeroed by the caller).
-cudaError_t launch_voxel_Bt(const GeomDev &g, const float *x, float *y, const int *stop,
+// y = B_un^T x (y plain).  acc: bt_scratch_floats(g) floats, 256-byte aligned,
+// contents overwritten.
+size_t bt_scratch_floats(const GeomDev &g);
+cudaError_t launch_voxel_Bt(const GeomDev &g, const float *x, float *y, float *acc, const int *stop,
                             cudaStream_t st);
+
+// The scatters (A^T, B_un^T) are bound by the rate of reduction requests, about
+// 2.8e10 warp requests a second whatever each carries.  Their contributions
+// come in pairs of neighbouring elements, so an accumulator is kept twice, the
+// second copy shifted by one element: every pair is 8-byte aligned in one of
+// them and goes as one request.  Element e is acc[e] + acc[odd + e + 1].
+__device__ __forceinline__ void add_pair(float *acc, size_t odd, size_t e, float lo, float hi)
+{
+    float *o = acc + e + ((e & 1) ? odd + 1 : 0);
+    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(o), "f"(lo), "f"(hi) : "memory");
+}
+// floats of one copy of an accumulator of n elements (keeps the next 256-byte aligned)
+inline size_t pair_acc_floats(size_t n) { return (n + 1 + 63) & ~size_t(63); }
 
 // --- vector kernels (ct_krylov.cu) ---------------------------------------------
 int num_sms();

@@ -954,14 +954,16 @@ struct OpBufs {
     float *Xc = nullptr, *Yc = nullptr;  // plane-major volume copies
     float *ypad = nullptr;               // padded sinogram
     float *t = nullptr;                  // plain sinogram
+    float *acc = nullptr;                // A^T's accumulators (b_kind CT_B_AT)
 };
 
-static void take_op_bufs(Arena &ar, const GeomDev &g, OpBufs &b, bool need_t)
+static void take_op_bufs(Arena &ar, const GeomDev &g, OpBufs &b, bool need_t, bool need_acc)
 {
     b.Xc = ar.take<float>(size_t(g.nzp) * g.nx * g.pitchX);
     b.Yc = ar.take<float>(size_t(g.nzp) * g.ny * g.pitchY);
     b.ypad = ar.take<float>(padded_sino_floats(g));
     b.t = need_t ? ar.take<float>(size_t(g.n_views) * g.nv * g.nu) : nullptr;
+    b.acc = need_acc ? ar.take<float>(at_scratch_floats(g)) : nullptr;
 }
 
 // out_vol = B sino.  `sino` is a plain sinogram, scaled by (*scale) first when
@@ -987,8 +989,7 @@ static cudaError_t apply_B(const GeomDev &g, int b_kind, float *sino, const doub
         if (e == cudaSuccess) e = launch_voxel_B(g, b.ypad, out_vol, stop, st, QUAD_ROWDIFF);
         return e;
     }
-    // exact transpose A^T (the projector's copies serve as its accumulators)
-    return launch_project_At(g, sino, out_vol, b.Xc, b.Yc, stop, st);
+    return launch_project_At(g, sino, out_vol, b.acc, stop, st);   // exact transpose A^T
 }
 
 static ct_status check_common(const ct_geom *geom, const float *b, int k, const float *x,
@@ -1059,7 +1060,7 @@ static bool carve_gmres(Arena &ar, const GeomDev &g, int k, bool ab, int b_kind,
         w.V = ar.take<float>(w.ldv * size_t(k + 1));
     if (!ab) w.q = ar.take<float>(n);
     // BA needs a plain sinogram when B reads one (F or A^T); AB never does
-    take_op_bufs(ar, g, w.ob, !ab && b_kind != CT_B_UN);
+    take_op_bufs(ar, g, w.ob, !ab && b_kind != CT_B_UN, b_kind == CT_B_AT);
     if (ab) w.tvol = ar.take<float>(n);
     const size_t ld = size_t(k) + 1;
     w.H = ar.take<double>(ld * k);
@@ -1530,7 +1531,8 @@ static ct_status abgmres(const ct_geom *geom, const float *b, int k, float *x, d
 struct VjpWs {
     GmresWs gm;
     float *t = nullptr, *tf = nullptr;   // sinogram-space temporaries
-    float *Xa = nullptr, *Ya = nullptr;  // A^T accumulators (the projector's copy layout)
+    float *acc = nullptr;                // A^T's accumulators
+    float *bt_acc = nullptr;             // B_un^T's accumulators
 };
 
 static void carve_vjp(Arena &ar, const GeomDev &g, int k, int b_kind, VjpWs &w)
@@ -1541,8 +1543,8 @@ static void carve_vjp(Arena &ar, const GeomDev &g, int k, int b_kind, VjpWs &w)
     w.gm.V = ar.take<float>(w.gm.ldv * size_t(k + 1));
     w.t = ar.take<float>(m);
     w.tf = b_kind == CT_B_FBP ? ar.take<float>(m) : nullptr;
-    w.Xa = ar.take<float>(size_t(g.nzp) * g.nx * g.pitchX);
-    w.Ya = ar.take<float>(size_t(g.nzp) * g.ny * g.pitchY);
+    w.acc = ar.take<float>(at_scratch_floats(g));
+    w.bt_acc = ar.take<float>(bt_scratch_floats(g));
     const size_t ld = size_t(k) + 1;
     w.gm.H = ar.take<double>(ld * k);
     w.gm.H2 = ar.take<double>(ld);
@@ -1576,13 +1578,10 @@ __global__ void scale_vec_kernel(float *__restrict__ v, size_t len, const double
 }
 
 // out_sino = B^T vol (plain layout); b_kind B_UN or B_FBP
-static cudaError_t apply_Bt(const GeomDev &g, int b_kind, const float *vol, float *t, float *tf, float *out,
-                            const int *stop, cudaStream_t s)
+static cudaError_t apply_Bt(const GeomDev &g, int b_kind, const float *vol, float *t, float *tf, float *bt_acc,
+                            float *out, const int *stop, cudaStream_t s)
 {
-    const size_t m = size_t(g.n_views) * g.nv * g.nu;
-    float *dst = b_kind == CT_B_FBP ? t : out;
-    cudaError_t e = cudaMemsetAsync(dst, 0, m * sizeof(float), s);
-    if (e == cudaSuccess) e = launch_voxel_Bt(g, vol, dst, stop, s);
+    cudaError_t e = launch_voxel_Bt(g, vol, b_kind == CT_B_FBP ? t : out, bt_acc, stop, s);
     if (e == cudaSuccess && b_kind == CT_B_FBP) e = launch_ramp(g, t, out, plain_layout(g), true, stop, s);
     (void)tf;
     return e;
@@ -1623,14 +1622,14 @@ static ct_status bagmres_vjp(const ct_geom *geom, const float *gx, int k, float 
             scale_vec_kernel<<<vb, RED_BLOCK, 0, s>>>(vj, n, &gm.st->inv_norm, stop);
             e = cudaGetLastError();
         }
-        if (e == cudaSuccess) e = apply_Bt(g, o.b_kind, vj, w.t, w.tf, sino, stop, s);
-        if (e == cudaSuccess) e = launch_project_At(g, sino, q, w.Xa, w.Ya, stop, s);
+        if (e == cudaSuccess) e = apply_Bt(g, o.b_kind, vj, w.t, w.tf, w.bt_acc, sino, stop, s);
+        if (e == cudaSuccess) e = launch_project_At(g, sino, q, w.acc, stop, s);
         if (e == cudaSuccess) e = arnoldi_orthogonalise(gm, q, j, k, n, o, s);
     }
     if (e == cudaSuccess) e = backsolve(gm.R, gm.g, gm.y, &gm.st->iters, k, s);
     float *z = Vf + size_t(k) * gm.ldv;
     if (e == cudaSuccess) e = combine(Vf, gm.ldv, k, n, gm.y, &gm.st->iters, z, s);
-    if (e == cudaSuccess) e = apply_Bt(g, o.b_kind, z, w.t, w.tf, gb, nullptr, s);
+    if (e == cudaSuccess) e = apply_Bt(g, o.b_kind, z, w.t, w.tf, w.bt_acc, gb, nullptr, s);
     if (e != cudaSuccess) {
         arena_close(ar);
         return cuda_error(e, "ct_bagmres_vjp launch");
@@ -1650,11 +1649,11 @@ struct CglsWs {
     SolverState *st = nullptr;
 };
 
-static void carve_cgls(Arena &ar, const GeomDev &g, int k, bool data_resid, CglsWs &w)
+static void carve_cgls(Arena &ar, const GeomDev &g, int k, int b_kind, bool data_resid, CglsWs &w)
 {
     const size_t n = size_t(g.nx) * g.ny * g.nz;
     const size_t m = size_t(g.n_views) * g.nv * g.nu;
-    take_op_bufs(ar, g, w.ob, false);
+    take_op_bufs(ar, g, w.ob, false, b_kind == CT_B_AT);
     w.r = ar.take<float>(m);
     w.q = ar.take<float>(m);
     w.s = ar.take<float>(n);
@@ -1665,12 +1664,12 @@ static void carve_cgls(Arena &ar, const GeomDev &g, int k, bool data_resid, Cgls
     w.st = ar.take<SolverState>(1);
 }
 
-static size_t cgls_ws_bytes(const GeomDev &g, int k, bool data_resid)
+static size_t cgls_ws_bytes(const GeomDev &g, int k, int b_kind, bool data_resid)
 {
     Arena ar;
     ar.size = ~size_t(0) >> 1;
     CglsWs w;
-    carve_cgls(ar, g, k, data_resid, w);
+    carve_cgls(ar, g, k, b_kind, data_resid, w);
     return ar.used;
 }
 
@@ -1681,10 +1680,10 @@ static ct_status cgls(const ct_geom *geom, const float *b, int k, float *x, doub
     const size_t n = geom->n, m = geom->m;
     const bool data = o.record_data_resid != 0;
     Arena ar;
-    ct_status rc = open_ws(ar, cgls_ws_bytes(g, k, data), o, s);
+    ct_status rc = open_ws(ar, cgls_ws_bytes(g, k, o.b_kind, data), o, s);
     if (rc != CT_OK) return rc;
     CglsWs w;
-    carve_cgls(ar, g, k, data, w);
+    carve_cgls(ar, g, k, o.b_kind, data, w);
     SolverState *st = w.st;
     const int *stop = &st->status;
     unsigned *ctr = &st->counter;
@@ -1962,7 +1961,7 @@ size_t ct_workspace_bytes(const ct_geom *geom, int k, int solver, const ct_solve
     switch (solver) {
     case CT_SOLVER_BA: return gmres_bytes(geom->g, k, false, o.b_kind);
     case CT_SOLVER_AB: return gmres_bytes(geom->g, k, true, o.b_kind);
-    case CT_SOLVER_CGLS: return cgls_ws_bytes(geom->g, k, o.record_data_resid != 0);
+    case CT_SOLVER_CGLS: return cgls_ws_bytes(geom->g, k, o.b_kind, o.record_data_resid != 0);
     case CT_SOLVER_BA_VJP: return vjp_bytes(geom->g, k, o.b_kind);
     default: return 0;
     }

@@ -232,18 +232,25 @@ struct ColumnA {
     float dxy2, inv_da, dzv;
 };
 
-// All lanes of the warp call it; lanes that are not live do not widen the range.
-template <int VR>
-__device__ __forceinline__ ColumnA column_A(const GeomDev &g, int s, int iv0, int iu, bool live)
+// In-plane direction (d_x, d_y) of detector column iu of view s.
+__device__ __forceinline__ float2 column_dir(const GeomDev &g, int s, int iu)
 {
-    const float4 *vp = reinterpret_cast<const float4 *>(g.viewA + s);
-    const float4 a = __ldg(vp), b = __ldg(vp + 1);   // (dx0, dxu, dy0, dyu), (dzv, crossu, sx, sy)
+    const float4 a = __ldg(reinterpret_cast<const float4 *>(g.viewA + s));   // (dx0, dxu, dy0, dyu)
     const float u = (float(iu) - g.cu) * g.du;
-    const float dx = fmaf(u, a.y, a.x);
-    const float dy = fmaf(u, a.w, a.z);
-    const float cross = u * b.y;
+    return make_float2(fmaf(u, a.y, a.x), fmaf(u, a.w, a.z));
+}
+
+// The column's rays walked along x (xdom) or y.  All lanes of the warp call
+// it; lanes that are not live do not widen the range.
+template <int VR>
+__device__ __forceinline__ ColumnA column_A(const GeomDev &g, int s, int iv0, int iu, bool live, bool xdom)
+{
+    const float4 b = __ldg(reinterpret_cast<const float4 *>(g.viewA + s) + 1);   // (dzv, crossu, sx, sy)
+    const float2 d = column_dir(g, s, iu);
+    const float dx = d.x, dy = d.y;
+    const float cross = (float(iu) - g.cu) * g.du * b.y;
     ColumnA c;
-    c.xdom = fabsf(dx) >= fabsf(dy);
+    c.xdom = xdom;
     const float da = c.xdom ? dx : dy;
     c.inv_da = 1.0f / da;
     c.Na = c.xdom ? g.nx : g.ny;
@@ -274,6 +281,14 @@ __device__ __forceinline__ ColumnA column_A(const GeomDev &g, int s, int iv0, in
     // inside its own plane count
     c.p1 = min(__reduce_max_sync(0xffffffffu, p1), c.Na - 1);
     return c;
+}
+
+// The same along the column's dominant axis.
+template <int VR>
+__device__ __forceinline__ ColumnA column_A(const GeomDev &g, int s, int iv0, int iu, bool live)
+{
+    const float2 d = column_dir(g, s, iu);
+    return column_A<VR>(g, s, iv0, iu, live, fabsf(d.x) >= fabsf(d.y));
 }
 
 // Step length vox |d| / |d_a| of ray iv of a column.
@@ -556,107 +571,88 @@ cudaError_t launch_project_A(const GeomDev &g, const float *Xc, const float *Yc,
 
 // ---------------------------------------------------------------------------
 // x = A^T y, the exact transpose of the projector above: the same column
-// walk (AT_VR rays of one detector column per thread, warp-uniform plane
+// walk (A_VR rays of one detector column per thread, warp-uniform plane
 // range, the same sample positions and bilinear weights), scattering
-// instead of gathering.  Contributions go with FP32 atomics into
+// instead of gathering.  Contributions go with FP32 reductions into
 // plane-major accumulators laid out like the projector's copies
-// (Xa[zp][x][yp] for x-dominant rays, Ya[zp][y][xp]), so the lanes of a
+// (X[zp][x][yp] for x-dominant rays, Y[zp][y][xp]), so the lanes of a
 // warp (consecutive u) add to neighbouring words of one row.  Within a
 // thread the rays of a column add to a two-row window per plane, as the
 // projector reads one: contributions to the same row are summed in
-// registers and a row is flushed (two atomics: cells b0 and b0 + 1) when
-// the window moves past it.  Samples on the zero border are skipped (they
-// are zero entries of A).  A last pass adds the two accumulators into x.
+// registers and a row is flushed when the window moves past it.
+//
+// A flush adds to two neighbouring cells, b0 and b0 + 1, as one request to one
+// of an orientation's two accumulators (add_pair).  Samples on the zero border
+// add to the border or are skipped (they are zero entries of A); a last pass
+// adds the four accumulators up.  Dense data, 256^3: 13.9 ms with a request a
+// cell, 12.1 ms so (128^3 1.01 -> 0.63 ms); what binds then is the rate at which
+// L2 adds words, about 1.5e12 a second (32 and 48 rays a thread, 11.9 and 12.3
+// ms).  Small scans were bound by a warp's chain of planes: 44^3 0.121 -> 0.039
+// ms, 64 x 64 30 -> 19 us.
 // ---------------------------------------------------------------------------
+static size_t at_floats(const GeomDev &g, bool x)
+{
+    return pair_acc_floats(size_t(g.nzp) * (x ? size_t(g.nx) * g.pitchX : size_t(g.ny) * g.pitchY));
+}
+
+size_t at_scratch_floats(const GeomDev &g)
+{
+    return g.siddon ? 0 : 2 * (at_floats(g, true) + at_floats(g, false));
+}
+
 template <int VR, bool WINDOW, bool ZCLAMP>
 __global__ void __launch_bounds__(A_BLOCK) joseph_At_kernel(GeomDev g, const float *__restrict__ y,
-                                                            float *__restrict__ Xa, float *__restrict__ Ya,
-                                                            const int *__restrict__ stop)
+                                                            float *__restrict__ X, size_t x_odd,
+                                                            float *__restrict__ Y, size_t y_odd, int v_tiles,
+                                                            int p_split, const int *__restrict__ stop)
 {
     if (stop && *stop) return;
     const int lane_u = blockIdx.x * 32 + (threadIdx.x & 31);
-    const int iv0 = (blockIdx.y * (A_BLOCK / 32) + (threadIdx.x >> 5)) * VR;
+    const int job = blockIdx.y * (A_BLOCK / 32) + (threadIdx.x >> 5);   // (tile of VR rows, share of the planes)
+    const int iv0 = (job / p_split) * VR, share = job % p_split;
     const int s = blockIdx.z;
-    const bool live = lane_u < g.nu && iv0 < g.nv;
+    const bool live = lane_u < g.nu && job < v_tiles * p_split;
     const int iu = min(lane_u, g.nu - 1);
-    const int ivl = min(iv0 + VR - 1, g.nv - 1);
-
-    const float4 *vp = reinterpret_cast<const float4 *>(g.viewA + s);
-    const float4 a = __ldg(vp), b = __ldg(vp + 1);   // (dx0, dxu, dy0, dyu), (dzv, crossu, sx, sy)
-    const float u = (float(iu) - g.cu) * g.du;
-    const float dx = fmaf(u, a.y, a.x);
-    const float dy = fmaf(u, a.w, a.z);
-    const float cross = u * b.y;
-    const bool xdom = fabsf(dx) >= fabsf(dy);
-    const float da = xdom ? dx : dy;
-    const float inv_da = 1.0f / da;
-    const int Na = xdom ? g.nx : g.ny;
-    const int Nb = xdom ? g.ny : g.nx;
-    const float ca = xdom ? g.cx : g.cy;
-    const float gb = (xdom ? dy : dx) * inv_da;
-    const float cterm = cross * inv_da * g.inv_vox;
-    const float fbc = xdom ? g.cy - cterm : g.cx + cterm;
-    const float Sv = (xdom ? b.z : b.w) * g.inv_vox;
-    const float gz_step = g.dv * b.x * inv_da;
-    const float gz0 = (float(iv0) - g.cv) * gz_step;
+    float2 d = column_dir(g, s, iu);
+    ColumnA c = column_A<VR>(g, s, iv0, iu, live, fabsf(d.x) >= fabsf(d.y));
 
     // each ray's value times its step weight (zero past nv and for idle lanes)
     float val[VR];
     bool any = false;
-    {
-        const float dxy2 = fmaf(dx, dx, dy * dy);
 #pragma unroll
-        for (int i = 0; i < VR; ++i) {
-            const int iv = iv0 + i;
-            val[i] = 0.0f;
-            if (live && iv < g.nv) {
-                const float v = (float(iv) - g.cv) * g.dv;
-                const float dz = v * b.x;
-                const float w = g.vox * sqrtf(fmaf(dz, dz, dxy2)) * fabsf(inv_da);
-                val[i] = y[(size_t(s) * g.nv + iv) * g.nu + iu] * w;
-                any = any || val[i] != 0.0f;
-            }
-        }
+    for (int i = 0; i < VR; ++i) {
+        val[i] = 0.0f;
+        if (live && iv0 + i < g.nv) val[i] = y[(size_t(s) * g.nv + iv0 + i) * g.nu + iu] * step_weight(g, c, iv0 + i);
+        any = any || val[i] != 0.0f;
     }
-
-    int p0 = 0, p1 = Na - 1;
-    clip_planes(fbc, gb, -1.0f, float(Nb), ca, Na, p0, p1);
-    {
-        const float gzl = (float(ivl) - g.cv) * gz_step;
-        clip_planes_run(fmaf(-Sv, gz0, g.cz), gz0, fmaf(-Sv, gzl, g.cz), gzl, -1.0f, float(g.nz), ca, Na, p0, p1);
-    }
-    if (!any) {   // nothing to add: this thread's rays do not widen the warp's range
-        p0 = Na;
-        p1 = -1;
-    }
-    p0 = __reduce_min_sync(0xffffffffu, p0);
-    p1 = __reduce_max_sync(0xffffffffu, p1);
-    p1 = min(p1, Na - 1);
+    if (!__any_sync(0xffffffffu, any)) return;
+    // lanes with nothing to add do not widen the warp's range
+    c = column_A<VR>(g, s, iv0, iu, any, c.xdom);
     if (!any) return;   // after the warp-wide reductions
+    const int each = (max(c.p1 - c.p0 + 1, 0) + p_split - 1) / p_split;
+    const int pa = c.p0 + share * each, pb = min(pa + each - 1, c.p1);
 
-    float *__restrict__ base = xdom ? Xa : Ya;
-    const int pitch = xdom ? g.pitchX : g.pitchY;
-    const int zstride = Na * pitch;
-    const int bmax = Nb, zmax = g.nz;
+    float *__restrict__ base = c.xdom ? X : Y;
+    const size_t odd = c.xdom ? x_odd : y_odd;
+    const int pitch = c.xdom ? g.pitchX : g.pitchY;
+    const unsigned zstride = unsigned(c.Na) * pitch;
+    const int zmax = g.nz;
 
-    for (int p = p0; p <= p1; ++p) {
-        const float pm = float(p) - ca;
-        const float fb = fmaf(pm, gb, fbc);
+    for (int p = pa; p <= pb; ++p) {
+        const float pm = float(p) - c.ca;
+        const float fb = fmaf(pm, c.gb, c.fbc);
         const float b0f = floorf(fb);
         const float wb = fb - b0f;
-        const int b0 = min(max(int(b0f), -PAD_A), bmax);
-        const bool bl = b0 >= 0, bh = b0 + 1 < Nb;   // the two cells inside the grid
-        if (!bl && !bh) continue;
-        float *rowp = base + (PAD_A * Na + p) * pitch + b0 + PAD_A;   // (z = 0, plane p, b0)
-        const float q = pm - Sv;
-        const float fz0 = fmaf(gz0, q, g.cz);
-        const float dzr = gz_step * q;
+        const int b0 = min(max(int(b0f), -PAD_A), c.Nb);
+        if (b0 < -1 || b0 >= c.Nb) continue;   // both cells on the border
+        const unsigned row0 = PAD_A * zstride + unsigned(p) * pitch + b0 + PAD_A;   // (z = 0, plane p, b0)
+        const float q = pm - c.Sv;
+        const float fz0 = fmaf(c.gz0, q, g.cz);
+        const float dzr = c.gz_step * q;
         // adds a row's summed contribution r to cells b0, b0 + 1 of grid row z
         auto flush = [&](int z, float r) {
             if (r == 0.0f || z < 0 || z >= zmax) return;
-            float *c = rowp + z * zstride;
-            if (bl) atomicAdd(c, r * (1.0f - wb));
-            if (bh) atomicAdd(c + 1, r * wb);
+            add_pair(base, odd, row0 + unsigned(z) * zstride, r * (1.0f - wb), r * wb);
         };
         int zc = 0;
         float acc_lo = 0.0f, acc_hi = 0.0f;   // rows zc and zc + 1
@@ -692,55 +688,58 @@ __global__ void __launch_bounds__(A_BLOCK) joseph_At_kernel(GeomDev g, const flo
     }
 }
 
-// x[z][y][x] = Xa[z][x][y] + Ya[z][y][x] over the grid (padded indices)
-__global__ void __launch_bounds__(256) unplane_kernel(GeomDev g, const float *__restrict__ Xa,
-                                                      const float *__restrict__ Ya, float *__restrict__ x,
-                                                      const int *__restrict__ stop)
+// x[z][y][x] = X[z][x][y] + Y[z][y][x] over the grid (padded indices), each from its two accumulators
+__global__ void __launch_bounds__(256) unplane_kernel(GeomDev g, const float *__restrict__ X, size_t x_odd,
+                                                      const float *__restrict__ Y, size_t y_odd,
+                                                      float *__restrict__ x, const int *__restrict__ stop)
 {
     if (stop && *stop) return;
     __shared__ float tile[32][33];
     const int tx = threadIdx.x, ty = threadIdx.y;   // 32 x 8
     const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 32, z = blockIdx.z;
     const size_t zp = size_t(z) + PAD_A;
-    // tile[xl][yl] = Xa[zp][x0 + xl][y0 + yl + PAD_A], read along y
+    // tile[xl][yl] = X[zp][x0 + xl][y0 + yl + PAD_A], read along y
     for (int r = ty; r < 32; r += 8) {
         const int xx = x0 + r, yy = y0 + tx;
-        tile[r][tx] = (xx < g.nx && yy < g.ny) ? Xa[(zp * g.nx + xx) * g.pitchX + yy + PAD_A] : 0.0f;
+        const size_t e = (zp * g.nx + xx) * g.pitchX + yy + PAD_A;
+        tile[r][tx] = (xx < g.nx && yy < g.ny) ? X[e] + X[x_odd + e + 1] : 0.0f;
     }
     __syncthreads();
     for (int r = ty; r < 32; r += 8) {
         const int yy = y0 + r, xx = x0 + tx;
+        const size_t e = (zp * g.ny + yy) * g.pitchY + xx + PAD_A;
         if (xx < g.nx && yy < g.ny)
-            x[(size_t(z) * g.ny + yy) * g.nx + xx] = tile[tx][r] + Ya[(zp * g.ny + yy) * g.pitchY + xx + PAD_A];
+            x[(size_t(z) * g.ny + yy) * g.nx + xx] = tile[tx][r] + (Y[e] + Y[y_odd + e + 1]);
     }
 }
 
-cudaError_t launch_project_At(const GeomDev &g, const float *y, float *x, float *Xa, float *Ya, const int *stop,
+cudaError_t launch_project_At(const GeomDev &g, const float *y, float *x, float *acc, const int *stop,
                              cudaStream_t st)
 {
     ProfScope prof(PK_JOSEPH_AT, st);
     if (g.siddon) return launch_siddon_At(g, y, x, stop, st);
-    cudaError_t e = cudaMemsetAsync(Xa, 0, sizeof(float) * size_t(g.nzp) * g.nx * g.pitchX, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(Ya, 0, sizeof(float) * size_t(g.nzp) * g.ny * g.pitchY, st);
+    const size_t x_odd = at_floats(g, true), y_odd = at_floats(g, false);
+    float *X = acc, *Y = acc + 2 * x_odd;
+    cudaError_t e = cudaMemsetAsync(acc, 0, sizeof(float) * at_scratch_floats(g), st);
     if (e != cudaSuccess) return e;
     constexpr int WPB = A_BLOCK / 32;
-    if (g.nv == 1) {
-        dim3 grid((g.nu + 31) / 32, (g.nv + WPB - 1) / WPB, g.n_views);
-        joseph_At_kernel<1, false, true><<<grid, A_BLOCK, 0, st>>>(g, y, Xa, Ya, stop);
-    } else {
-        constexpr int VR = AT_VR;
-        dim3 grid((g.nu + 31) / 32, (g.nv + WPB * VR - 1) / (WPB * VR), g.n_views);
-        if (g.a_window && g.a_zsafe)
-            joseph_At_kernel<VR, true, false><<<grid, A_BLOCK, 0, st>>>(g, y, Xa, Ya, stop);
-        else if (g.a_window)
-            joseph_At_kernel<VR, true, true><<<grid, A_BLOCK, 0, st>>>(g, y, Xa, Ya, stop);
-        else
-            joseph_At_kernel<VR, false, true><<<grid, A_BLOCK, 0, st>>>(g, y, Xa, Ya, stop);
-    }
+    const int u_tiles = (g.nu + 31) / 32, v_tiles = g.nv == 1 ? 1 : (g.nv + A_VR - 1) / A_VR;
+    // small scans: warps share a tile's planes until the grid has 32 warps an SM
+    int split = 1;
+    while (split < 16 && size_t(u_tiles) * v_tiles * g.n_views * split * 2 <= size_t(num_sms()) * 32) split *= 2;
+    const dim3 grid(u_tiles, (v_tiles * split + WPB - 1) / WPB, g.n_views);
+    if (g.nv == 1)
+        joseph_At_kernel<1, false, true><<<grid, A_BLOCK, 0, st>>>(g, y, X, x_odd, Y, y_odd, v_tiles, split, stop);
+    else if (g.a_window && g.a_zsafe)
+        joseph_At_kernel<A_VR, true, false><<<grid, A_BLOCK, 0, st>>>(g, y, X, x_odd, Y, y_odd, v_tiles, split, stop);
+    else if (g.a_window)
+        joseph_At_kernel<A_VR, true, true><<<grid, A_BLOCK, 0, st>>>(g, y, X, x_odd, Y, y_odd, v_tiles, split, stop);
+    else
+        joseph_At_kernel<A_VR, false, true><<<grid, A_BLOCK, 0, st>>>(g, y, X, x_odd, Y, y_odd, v_tiles, split, stop);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     dim3 ublock(32, 8), ugrid((g.nx + 31) / 32, (g.ny + 31) / 32, g.nz);
-    unplane_kernel<<<ugrid, ublock, 0, st>>>(g, Xa, Ya, x, stop);
+    unplane_kernel<<<ugrid, ublock, 0, st>>>(g, X, x_odd, Y, y_odd, x, stop);
     return cudaGetLastError();
 }
 
@@ -773,11 +772,10 @@ extern "C" ct_status ct_adjoint_At(const ct_geom *geom, const float *y_dev, floa
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const GeomDev &g = geom->g;
     Arena ar;
-    ct_status rc = arena_open(ar, plane_copies_bytes(g), nullptr, 0, st);
+    const size_t floats = at_scratch_floats(g);
+    ct_status rc = arena_open(ar, Arena::align(floats * sizeof(float)), nullptr, 0, st);
     if (rc != CT_OK) return rc;
-    float *Xa = ar.take<float>(size_t(g.nzp) * g.nx * g.pitchX);
-    float *Ya = ar.take<float>(size_t(g.nzp) * g.ny * g.pitchY);
-    cudaError_t e = launch_project_At(g, y_dev, x_dev, Xa, Ya, nullptr, st);
+    cudaError_t e = launch_project_At(g, y_dev, x_dev, floats ? ar.take<float>(floats) : nullptr, nullptr, st);
     arena_close(ar);
     if (e != cudaSuccess) return cuda_error(e, "ct_adjoint_At launch");
     return CT_OK;
