@@ -95,8 +95,12 @@ __device__ __forceinline__ float cosine_weight(const GeomDev &g, int iu, int iv)
 // inverse is taken as a forward transform of the conjugate,
 // IFFT(Y) = conj(FFT(conj(Y))) / N, with 1/N folded into H.
 //
-// The transform is a Stockham autosort FFT in shared memory, radix 4 (a
-// radix-2 stage last when N is not a power of 4), output in natural order.
+// The transform is a Stockham autosort FFT in shared memory, radix 4, then a
+// radix-2 stage and a radix-3 stage where N has those factors left, output in
+// natural order.  N = 3 2^a fits detectors of 192, 384 and 768 columns with 3/4
+// of the points that a power of two takes (the kernel is bound by issue slots,
+// so by points and stages): 128^3 scan 52 -> 41 us, 256^3 0.51 -> 0.41 ms, 512^3
+// 5.2 -> 3.9 ms.
 // A stage of radix R after Ns points have been combined: butterfly j reads
 // element j + r N/R (r < R), multiplies it by exp(-2 pi i r (j mod Ns) /
 // (R Ns)), transforms the R values and writes value r to
@@ -114,14 +118,16 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b)
 // Ns combined points uses exp(-2 pi i r k / (4 Ns)), r = 1..3, k < Ns, stored
 // at stw[(Ns - 1) + (r - 1) Ns + k] (stages Ns = 1, 4, 16, ... take 3 Ns
 // entries each, starting at Ns - 1 = 4^s - 1); the radix-2 stage's
-// exp(-2 pi i k / N), k < N/2, follow.  Lanes with consecutive k read
+// exp(-2 pi i k / (2 Ns)), k < Ns, and the radix-3 stage's exp(-2 pi i r k / N),
+// r = 1, 2, k < N/3, follow.  Lanes with consecutive k read
 // consecutive entries (in the full-length table they are N/(4 Ns) entries
 // apart, all in one bank).
-__device__ __forceinline__ int fft_stage_table(int N)
+__device__ __forceinline__ int fft_radix4_points(int N)
 {
+    const int P = N % 3 == 0 ? N / 3 : N;   // the power of two in N
     int Ns = 1;
-    while (Ns * 4 <= N) Ns *= 4;
-    return Ns - 1;   // radix-4 entries: the sum over the stages of 3 Ns
+    while (Ns * 4 <= P) Ns *= 4;
+    return Ns;
 }
 
 // Buffer element i lives at slot fsw(i): within each aligned block of 16
@@ -138,9 +144,9 @@ __device__ __forceinline__ int fsw(int i) { return i ^ (5 * ((i >> 4) & 3)); }
 // (it synchronises the block).
 __device__ __forceinline__ void fft_group(float2 *&a, float2 *&b, const float2 *__restrict__ stw, int N, int t)
 {
-    const int T = N >> 2;
+    const int T = N >> 2, P = N % 3 == 0 ? N / 3 : N;
     int Ns = 1;
-    for (; Ns * 4 <= N; Ns *= 4) {
+    for (; Ns * 4 <= P; Ns *= 4) {
         const int k = t & (Ns - 1);
         float2 v0 = a[fsw(t)], v1 = a[fsw(t + T)], v2 = a[fsw(t + 2 * T)], v3 = a[fsw(t + 3 * T)];
         if (Ns > 1) {
@@ -161,16 +167,34 @@ __device__ __forceinline__ void fft_group(float2 *&a, float2 *&b, const float2 *
         a = b;
         b = tmp;
     }
-    if (Ns < N) {   // N = 2 Ns: one radix-2 stage, two butterflies per thread
-        const float2 *w2 = stw + (Ns - 1);
+    const float2 *w = stw + (Ns - 1);
+    if (Ns < P) {   // one radix-2 stage over N = 2 Ns (x 3): two butterflies per thread
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const int j = t + h * T;
             const int k = j & (Ns - 1);
-            const float2 v0 = a[fsw(j)], v1 = cmul(a[fsw(j + N / 2)], w2[k]);
+            const float2 v0 = a[fsw(j)], v1 = cmul(a[fsw(j + N / 2)], w[k]);
             const int d = ((j - k) << 1) + k;
             b[fsw(d)] = make_float2(v0.x + v1.x, v0.y + v1.y);
             b[fsw(d + Ns)] = make_float2(v0.x - v1.x, v0.y - v1.y);
+        }
+        __syncthreads();
+        float2 *tmp = a;
+        a = b;
+        b = tmp;
+        w += Ns;
+        Ns *= 2;
+    }
+    if (P < N) {   // a last radix-3 stage, Ns = N / 3: one butterfly a thread and a third one for every third
+        for (int j = t; j < Ns; j += T) {
+            const float2 v0 = a[fsw(j)], v1 = cmul(a[fsw(j + Ns)], w[j]), v2 = cmul(a[fsw(j + 2 * Ns)], w[Ns + j]);
+            const float2 s = make_float2(v1.x + v2.x, v1.y + v2.y);
+            constexpr float S60 = 0.866025403784438647f;
+            const float2 m = make_float2(fmaf(-0.5f, s.x, v0.x), fmaf(-0.5f, s.y, v0.y));
+            const float2 q = make_float2(S60 * (v1.y - v2.y), -S60 * (v1.x - v2.x));   // -i sin(60) (v1 - v2)
+            b[fsw(j)] = make_float2(v0.x + s.x, v0.y + s.y);
+            b[fsw(j + Ns)] = make_float2(m.x + q.x, m.y + q.y);
+            b[fsw(j + 2 * Ns)] = make_float2(m.x - q.x, m.y - q.y);
         }
         __syncthreads();
         float2 *tmp = a;
@@ -210,15 +234,21 @@ __global__ void ramp_fft_kernel(GeomDev g, const float *__restrict__ src, float 
     float2 *a = fsm + 2 * N + size_t(grp) * 2 * N;                 // this group's two buffers
     float2 *b = a + N;
     for (int i = threadIdx.x; i < N; i += blockDim.x) H[i] = g.fft_h[i];
-    for (int Ns = 1; Ns * 4 <= N; Ns *= 4)   // radix-4 entries (Ns - 1) + (r - 1) Ns + k = tw[r k N / (4 Ns)]
-        for (int i = threadIdx.x; i < 3 * Ns; i += blockDim.x) {
-            const int r = i / Ns + 1, k = i - (r - 1) * Ns;
-            stw[(Ns - 1) + i] = g.fft_tw[r * k * (N / (4 * Ns))];
-        }
     {
-        const int r4 = fft_stage_table(N);
-        if (r4 + 1 < N)   // a radix-2 stage (Ns = N / 2) follows: tw[k], k < N / 2
-            for (int i = threadIdx.x; i < N / 2; i += blockDim.x) stw[r4 + i] = g.fft_tw[i];
+        int Ns = 1;
+        const int P = N % 3 == 0 ? N / 3 : N, N4 = fft_radix4_points(N);
+        for (; Ns < N4; Ns *= 4)   // radix-4 entries (Ns - 1) + (r - 1) Ns + k = tw[r k N / (4 Ns)]
+            for (int i = threadIdx.x; i < 3 * Ns; i += blockDim.x) {
+                const int r = i / Ns + 1, k = i - (r - 1) * Ns;
+                stw[(Ns - 1) + i] = g.fft_tw[r * k * (N / (4 * Ns))];
+            }
+        float2 *w = stw + (Ns - 1);
+        if (Ns < P) {   // a radix-2 stage follows: tw[k N / (2 Ns)], k < Ns
+            for (int i = threadIdx.x; i < Ns; i += blockDim.x) w[i] = g.fft_tw[i * (N / (2 * Ns))];
+            w += Ns;
+        }
+        if (P < N)      // and a radix-3 stage: tw[r k], k < N / 3
+            for (int i = threadIdx.x; i < 2 * P; i += blockDim.x) w[i] = g.fft_tw[i < P ? i : 2 * (i - P)];
     }
     const int nu = g.nu;
     const int nrows = g.n_views * g.nv;

@@ -360,8 +360,10 @@ ct_status ct_geom_create(const ct_geom_desc *d, ct_geom **out)
     // the kernel wrapped (h[q] at q and N - q) equals the linear one on the
     // first nu outputs when N >= 2 nu - 1; h is even, so H is real:
     //   H[k] = h[0] + 2 sum_{q >= 1} h[q] cos(2 pi q k / N)
+    // the smallest N of the form 2^a, or 3 2^a from 96 on
     int fft_n = 8;
     while (fft_n < 2 * d->nu - 1) fft_n *= 2;
+    if (fft_n >= 128 && fft_n / 4 * 3 >= 2 * d->nu - 1) fft_n = fft_n / 4 * 3;
     std::vector<float2> fft_tw(fft_n);
     std::vector<float> fft_h(fft_n);
     {

@@ -89,7 +89,7 @@ struct GeomDev {
     int vol_bf16, sino_bf16;
     // ramp filter by FFT: the linear convolution of a row with the ramp
     // kernel is the circular one of length fft_n >= 2 nu - 1 (a power of
-    // two); the kernel is even, so its spectrum is real.
+    // two, or three times one); the kernel is even, so its spectrum is real.
     //   fft_tw[t] = exp(-2 pi i t / fft_n), t < fft_n
     //   fft_h[k]  = spectrum of the scaled kernel / fft_n, k < fft_n
     int fft_n;

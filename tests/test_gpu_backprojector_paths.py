@@ -72,3 +72,15 @@ def test_projector_written_entries(ct, spec):
     xg = x.double().cpu().numpy().reshape(-1)
     assert np.linalg.norm(xg - ref["x_final"]) <= 1e-4 * np.linalg.norm(ref["x_final"])
     assert np.max(np.abs(res.resid - ref["resid"])) <= 1e-4 * ref["resid"][0]
+
+
+# transform lengths 8, 2^a, 3 2^a with and without a radix-2 stage, and the first row length past each
+@pytest.mark.parametrize("nu", [1, 3, 47, 48, 49, 64, 65, 96, 97, 128, 129, 192, 193, 384, 385, 768, 769])
+@pytest.mark.parametrize("transpose", [False, True])
+def test_ramp_lengths(ct, nu, transpose):
+    spec = par2d(40, 40, 7, nu)   # an odd row count: the last row has no partner
+    g = ct.Geometry.from_spec(spec)
+    y = ci.random_vector(spec.m, seed=87).astype(np.float32).reshape(spec.sino_shape)
+    out = ct.ramp_F(g, torch.from_numpy(y).cuda(), transpose).double().cpu().numpy()
+    ref = (oracle.ramp_Ft if transpose else oracle.ramp_F)(spec, y.astype(np.float64)).reshape(out.shape)
+    assert np.linalg.norm(out - ref) <= 1e-5 * np.linalg.norm(ref)
