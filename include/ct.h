@@ -19,9 +19,10 @@
  *     their result and residual history are complete (they synchronise the
  *     stream once at the end).
  *   - Scratch memory: operator calls and solvers take their temporary device
- *     memory from the stream-ordered allocator (cudaMallocAsync on `stream`)
- *     and release it before returning, unless the solver options supply a
- *     workspace.
+ *     memory in the order of `stream` from a pool of the library's and release
+ *     it before returning, unless the solver options supply a workspace.  While
+ *     a geometry lives on a device, its pool keeps up to 1/32 of the device's
+ *     memory between calls; destroying the device's last geometry returns it.
  *   - Errors: every call returns a ct_status; on failure the outputs are
  *     unspecified (except CT_BREAKDOWN_LUCKY, whose outputs are valid) and
  *     ct_last_error() gives a message for the calling thread.  No call

@@ -287,19 +287,20 @@ __device__ __forceinline__ void store_sino_pair(float *out, const SinoLayout &la
 // (the Arnoldi normalisation), as float or, when g.vol_bf16, as bf16.
 cudaError_t launch_plane_copies(const GeomDev &g, const float *vol, const double *scale, void *basis_out,
                                 float *Xc, float *Yc, const int *stop, cudaStream_t st);
-// y = A x from the plane copies (Joseph; the line-intersection projector
-// reads Yc only), written in `lay`.
+// y = A x from the plane copies, written in `lay`.
 cudaError_t launch_project_A(const GeomDev &g, const float *Xc, const float *Yc, float *y,
                             SinoLayout lay, const int *stop, cudaStream_t st);
-// x = A^T y (overwritten); y in plain layout.  acc: at_scratch_floats(g) floats
-// (none for the line-intersection projector), 256-byte aligned, contents overwritten.
+// x = A^T y (overwritten); y in plain layout.  acc: at_scratch_floats(g) floats,
+// 256-byte aligned, contents overwritten.
 size_t at_scratch_floats(const GeomDev &g);
 cudaError_t launch_project_At(const GeomDev &g, const float *y, float *x, float *acc, const int *stop,
                              cudaStream_t st);
-// the line-intersection projector and its transpose (ct_siddon.cu); x overwritten
-cudaError_t launch_siddon_A(const GeomDev &g, const float *Yc, float *y, SinoLayout lay, const int *stop,
-                            cudaStream_t st);
-cudaError_t launch_siddon_At(const GeomDev &g, const float *y, float *x, const int *stop, cudaStream_t st);
+// the line-intersection projector and its transpose (ct_siddon.cu); the
+// transpose adds to the zeroed accumulators Xa, Ya, laid out like the copies
+cudaError_t launch_siddon_A(const GeomDev &g, const float *Xc, const float *Yc, float *y, SinoLayout lay,
+                            const int *stop, cudaStream_t st);
+cudaError_t launch_siddon_At(const GeomDev &g, const float *y, float *Xa, float *Ya, const int *stop,
+                             cudaStream_t st);
 
 // --- back-projector (ct_backproject.cu) ------------------------------------------
 // Copies a plain sinogram into the padded layout, scaled by (*scale) when

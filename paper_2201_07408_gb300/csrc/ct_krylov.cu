@@ -1,16 +1,18 @@
 // Krylov solvers: BA-GMRES (Eq. 5), AB-GMRES (Eq. 4) and CGLS (Eqs. 2-3).
 //
 // Arnoldi with modified Gram-Schmidt (Sec. II): the newest Krylov vector q
-// is orthogonalised against the basis one vector at a time.  Each pass is
-// one streaming kernel that applies the previous projection
-// (q -= h_{i-1} v_{i-1}) and forms the next inner product <q, v_i> in the
-// same sweep over memory, so pass i reads q, v_{i-1}, v_i and writes q once.
+// is orthogonalised against the basis one vector at a time.  A pass
+// applies the previous projection (q -= h_{i-1} v_{i-1}) and forms the next
+// inner product <q, v_i> in the same sweep over memory, so pass i reads q,
+// v_{i-1}, v_i and writes q once.  Vectors that fit the registers of the chip
+// are swept in one launch that keeps q there; longer ones take a launch a
+// pass.
 // Inner products: per-thread FP32 accumulation (plain FMA, or compensated
-// with an FMA two-product and a two-sum), warp-shuffle and block reductions
-// in FP64, and a last-block grid reduction in a fixed order (deterministic,
-// no spin-waits).  The Hessenberg column, the Givens rotations, the
+// with an FMA two-product and a two-sum), sums within a block in FP32 triples
+// that keep the rounding errors, between blocks in FP64, in a fixed order
+// (deterministic).  The Hessenberg column, the Givens rotations, the
 // residual estimate |g_{j+1}| and the final triangular solve run in FP64 in
-// one-thread kernels, so the whole solve is enqueued without host round
+// one warp, so the whole solve is enqueued without host round
 // trips; a device status word stops the remaining kernels on a tolerance
 // stop, a lucky breakdown or a non-finite norm.
 #include <algorithm>
@@ -1182,7 +1184,8 @@ static cudaError_t launch_sweep(GmresWs &w, float *q, int j, double *hcol, size_
     ProfScope prof(PK_MGS, s);
     const unsigned blocks = sweep_blocks(len);
     if (blocks == 1) {   // nobody to wait for
-        mgs_sweep_kernel<MODE, TB, 16><<<1, SWEEP_NT, 0, s>>>(q, V, w.ldv, j, len, hcol, first_ss, last_ss, w.slots, set,
+        auto *kernel = len <= SWEEP_NT * 8 ? mgs_sweep_kernel<MODE, TB, 8> : mgs_sweep_kernel<MODE, TB, 16>;
+        kernel<<<1, SWEEP_NT, 0, s>>>(q, V, w.ldv, j, len, hcol, first_ss, last_ss, w.slots, set,
                                                               stop, skip, w.st, g);
         return cudaGetLastError();
     }

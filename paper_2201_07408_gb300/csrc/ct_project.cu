@@ -21,6 +21,7 @@
 // (S x d)_z rather than from S + t d, which in FP32 would cancel two terms of
 // the size of the source distance; (S x d)_z = sod*u exactly for this
 // geometry, so the intercept keeps full relative precision.
+#include <algorithm>
 #include <mutex>
 
 #include "ct_internal.cuh"
@@ -561,7 +562,7 @@ cudaError_t launch_project_A(const GeomDev &g, const float *Xc, const float *Yc,
                             SinoLayout lay, const int *stop, cudaStream_t st)
 {
     ProfScope prof(PK_JOSEPH_A, st);
-    if (g.siddon) return launch_siddon_A(g, Yc, y, lay, stop, st);
+    if (g.siddon) return launch_siddon_A(g, Xc, Yc, y, lay, stop, st);
     if (g.vol_bf16)
         launch_joseph_A_t<true>(g, Xc, Yc, y, lay, stop, st);
     else
@@ -595,9 +596,10 @@ static size_t at_floats(const GeomDev &g, bool x)
     return pair_acc_floats(size_t(g.nzp) * (x ? size_t(g.nx) * g.pitchX : size_t(g.ny) * g.pitchY));
 }
 
+// Joseph's transpose keeps each accumulator twice, the line-intersection one's once
 size_t at_scratch_floats(const GeomDev &g)
 {
-    return g.siddon ? 0 : 2 * (at_floats(g, true) + at_floats(g, false));
+    return (g.siddon ? 1 : 2) * (at_floats(g, true) + at_floats(g, false));
 }
 
 template <int VR, bool WINDOW, bool ZCLAMP>
@@ -688,7 +690,8 @@ __global__ void __launch_bounds__(A_BLOCK) joseph_At_kernel(GeomDev g, const flo
     }
 }
 
-// x[z][y][x] = X[z][x][y] + Y[z][y][x] over the grid (padded indices), each from its two accumulators
+// x[z][y][x] = X[z][x][y] + Y[z][y][x] over the grid (padded indices), each from its two copies (PAIRS) or its one
+template <bool PAIRS>
 __global__ void __launch_bounds__(256) unplane_kernel(GeomDev g, const float *__restrict__ X, size_t x_odd,
                                                       const float *__restrict__ Y, size_t y_odd,
                                                       float *__restrict__ x, const int *__restrict__ stop)
@@ -696,20 +699,23 @@ __global__ void __launch_bounds__(256) unplane_kernel(GeomDev g, const float *__
     if (stop && *stop) return;
     __shared__ float tile[32][33];
     const int tx = threadIdx.x, ty = threadIdx.y;   // 32 x 8
-    const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 32, z = blockIdx.z;
-    const size_t zp = size_t(z) + PAD_A;
-    // tile[xl][yl] = X[zp][x0 + xl][y0 + yl + PAD_A], read along y
-    for (int r = ty; r < 32; r += 8) {
-        const int xx = x0 + r, yy = y0 + tx;
-        const size_t e = (zp * g.nx + xx) * g.pitchX + yy + PAD_A;
-        tile[r][tx] = (xx < g.nx && yy < g.ny) ? X[e] + X[x_odd + e + 1] : 0.0f;
-    }
-    __syncthreads();
-    for (int r = ty; r < 32; r += 8) {
-        const int yy = y0 + r, xx = x0 + tx;
-        const size_t e = (zp * g.ny + yy) * g.pitchY + xx + PAD_A;
-        if (xx < g.nx && yy < g.ny)
-            x[(size_t(z) * g.ny + yy) * g.nx + xx] = tile[tx][r] + (Y[e] + Y[y_odd + e + 1]);
+    const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 32;
+    for (int z = blockIdx.z; z < g.nz; z += gridDim.z) {
+        const size_t zp = size_t(z) + PAD_A;
+        __syncthreads();
+        // tile[xl][yl] = X[zp][x0 + xl][y0 + yl + PAD_A], read along y
+        for (int r = ty; r < 32; r += 8) {
+            const int xx = x0 + r, yy = y0 + tx;
+            const size_t e = (zp * g.nx + xx) * g.pitchX + yy + PAD_A;
+            tile[r][tx] = (xx < g.nx && yy < g.ny) ? (PAIRS ? X[e] + X[x_odd + e + 1] : X[e]) : 0.0f;
+        }
+        __syncthreads();
+        for (int r = ty; r < 32; r += 8) {
+            const int yy = y0 + r, xx = x0 + tx;
+            const size_t e = (zp * g.ny + yy) * g.pitchY + xx + PAD_A;
+            if (xx < g.nx && yy < g.ny)
+                x[(size_t(z) * g.ny + yy) * g.nx + xx] = tile[tx][r] + (PAIRS ? Y[e] + Y[y_odd + e + 1] : Y[e]);
+        }
     }
 }
 
@@ -717,11 +723,17 @@ cudaError_t launch_project_At(const GeomDev &g, const float *y, float *x, float 
                              cudaStream_t st)
 {
     ProfScope prof(PK_JOSEPH_AT, st);
-    if (g.siddon) return launch_siddon_At(g, y, x, stop, st);
     const size_t x_odd = at_floats(g, true), y_odd = at_floats(g, false);
-    float *X = acc, *Y = acc + 2 * x_odd;
+    float *X = acc, *Y = acc + (g.siddon ? 1 : 2) * x_odd;
     cudaError_t e = cudaMemsetAsync(acc, 0, sizeof(float) * at_scratch_floats(g), st);
     if (e != cudaSuccess) return e;
+    const dim3 ublock(32, 8), ugrid((g.nx + 31) / 32, (g.ny + 31) / 32, std::min(g.nz, 65535));
+    if (g.siddon) {
+        e = launch_siddon_At(g, y, X, Y, stop, st);
+        if (e != cudaSuccess) return e;
+        unplane_kernel<false><<<ugrid, ublock, 0, st>>>(g, X, x_odd, Y, y_odd, x, stop);
+        return cudaGetLastError();
+    }
     constexpr int WPB = A_BLOCK / 32;
     const int u_tiles = (g.nu + 31) / 32, v_tiles = g.nv == 1 ? 1 : (g.nv + A_VR - 1) / A_VR;
     // small scans: warps share a tile's planes until the grid has 32 warps an SM
@@ -738,8 +750,7 @@ cudaError_t launch_project_At(const GeomDev &g, const float *y, float *x, float 
         joseph_At_kernel<A_VR, false, true><<<grid, A_BLOCK, 0, st>>>(g, y, X, x_odd, Y, y_odd, v_tiles, split, stop);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    dim3 ublock(32, 8), ugrid((g.nx + 31) / 32, (g.ny + 31) / 32, g.nz);
-    unplane_kernel<<<ugrid, ublock, 0, st>>>(g, X, x_odd, Y, y_odd, x, stop);
+    unplane_kernel<true><<<ugrid, ublock, 0, st>>>(g, X, x_odd, Y, y_odd, x, stop);
     return cudaGetLastError();
 }
 
@@ -775,7 +786,7 @@ extern "C" ct_status ct_adjoint_At(const ct_geom *geom, const float *y_dev, floa
     const size_t floats = at_scratch_floats(g);
     ct_status rc = arena_open(ar, Arena::align(floats * sizeof(float)), nullptr, 0, st);
     if (rc != CT_OK) return rc;
-    cudaError_t e = launch_project_At(g, y_dev, x_dev, floats ? ar.take<float>(floats) : nullptr, nullptr, st);
+    cudaError_t e = launch_project_At(g, y_dev, x_dev, ar.take<float>(floats), nullptr, st);
     arena_close(ar);
     if (e != cudaSuccess) return cuda_error(e, "ct_adjoint_At launch");
     return CT_OK;
