@@ -429,7 +429,8 @@ __global__ void __launch_bounds__(256) voxel_B_small_kernel(GeomDev g, const voi
     __shared__ float part[ZC][8][32];
     constexpr int ENTRY = BF ? 8 : 16;
     const int l = threadIdx.x, w = threadIdx.y, share = w % split;
-    const int ix = blockIdx.x * 32 + l, iy = blockIdx.y * (8 / split) + w / split, iz0 = blockIdx.z * ZC;
+    const int tiles = (g.nx + 31) / 32;   // tiles along x, then groups of rows: one grid axis, of 2^31 blocks
+    const int ix = blockIdx.x % tiles * 32 + l, iy = blockIdx.x / tiles * (8 / split) + w / split, iz0 = blockIdx.y * ZC;
     const float xc = (float(min(ix, g.nx - 1)) - g.cx) * g.vox, yc = (float(min(iy, g.ny - 1)) - g.cy) * g.vox;
     const float zfirst = (float(iz0) - g.cz) * g.vox;
     const size_t view_stride = size_t(g.nvp) * g.pitchU;
@@ -449,7 +450,7 @@ __global__ void __launch_bounds__(256) voxel_B_small_kernel(GeomDev g, const voi
             const float v0f = FLAT ? 0.0f : floorf(fv);
             int row = int(v0f);
             if (!CT_IN_BOUNDS(g, unsigned(row + g.padv) < unsigned(g.nvp), BS_B_ROW, s, row + g.padv)) row = -g.padv;
-            const char *p = pv + row * (ENTRY * g.pitchU);
+            const char *p = pv + ptrdiff_t(row) * (ENTRY * g.pitchU);
             float r;
             if (FLAT) {
                 r = row_value<BF, DIFF>(p, c.wu);
@@ -653,7 +654,7 @@ static cudaError_t launch_voxel_B_small(const GeomDev &g, const float *ypad, flo
     const int tiles = (g.nx + 31) / 32, runs = (g.nz + ZC - 1) / ZC;
     int split = 1;
     while (split < 8 && size_t(tiles) * g.ny * runs * split * 2 <= size_t(num_sms()) * 32) split *= 2;
-    const dim3 block(32, 8), grid(tiles, (g.ny * split + 7) / 8, runs);
+    const dim3 block(32, 8), grid(tiles * ((g.ny * split + 7) / 8), runs);
     voxel_B_small_kernel<ZC, FLAT, BF, DIFF><<<grid, block, 0, st>>>(g, ypad, x, split, stop);
     return cudaGetLastError();
 }
