@@ -50,8 +50,11 @@ __device__ __forceinline__ void clip_planes(float fc, float g, float lo, float h
     float ig = 1.0f / g;
     float t1 = (lo - 0.5f - fc) * ig + ca;
     float t2 = (hi + 0.5f - fc) * ig + ca;
-    float tl = fmaxf(fminf(t1, t2), -1.0f);
-    float th = fminf(fmaxf(t1, t2), float(Na));
+    // both ends are held to [-1, Na]: a ray nearly parallel to a grid side that
+    // passes beside it has t of 1e17, and plane numbers that saturate would
+    // overflow in the kernels' sums (a warp's share is added to p0)
+    float tl = fminf(fmaxf(fminf(t1, t2), -1.0f), float(Na));
+    float th = fmaxf(fminf(fmaxf(t1, t2), float(Na)), -1.0f);
     p0 = max(p0, int(ceilf(tl)));
     p1 = min(p1, int(floorf(th)));
 }

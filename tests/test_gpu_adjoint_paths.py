@@ -27,9 +27,9 @@ def ct():
     return _ct
 
 
-def par2d(nx, ny, views, nu):
+def par2d(nx, ny, views, nu, ang0=0.15):
     return ci.Geometry(name="par2d_%dx%d" % (nx, ny), kind=ci.PARALLEL_2D, nx=nx, ny=ny, nz=1, vox=1.0,
-                       n_views=views, ang0=0.15, span=math.pi, nu=nu, nv=1, du=1.0, dv=1.0)
+                       n_views=views, ang0=ang0, span=math.pi, nu=nu, nv=1, du=1.0, dv=1.0)
 
 
 def cone(name, nx, ny, nz, views, nu, nv, du, **kw):
@@ -37,6 +37,7 @@ def cone(name, nx, ny, nz, views, nu, nv, du, **kw):
 
 
 SCANS = [par2d(9, 7, 3, 33), par2d(100, 81, 60, 150),
+         par2d(24, 22, 10, 160, ang0=0.0),   # warps of rays beside the image, parallel to its sides
          cone("thin", 31, 33, 5, 9, 41, 9, 1.7),
          cone("odd_rows", 33, 31, 17, 11, 47, 21, 1.5),
          cone("mid", 65, 60, 40, 40, 97, 47, 1.6),
@@ -62,7 +63,7 @@ def test_transposes_match_oracle(ct, spec):
 def test_matched_solve_uses_the_transpose(ct):
     """CGLS and BA-GMRES with B = A^T, whose workspaces hold the accumulators."""
     from oracle import krylov
-    spec = SCANS[3]
+    spec = SCANS[4]
     g = ct.Geometry.from_spec(spec)
     b = oracle.project_A(spec, ci.phantom(spec)[0].astype(np.float64)).astype(np.float32)
     bd = torch.from_numpy(b.reshape(spec.sino_shape)).cuda()
@@ -77,7 +78,7 @@ def test_matched_solve_uses_the_transpose(ct):
 
 
 def test_nonfinite_reading_touches_its_own_cells_only(ct):
-    spec = SCANS[3]
+    spec = SCANS[4]
     g = ct.Geometry.from_spec(spec)
     r = (spec.n_views // 2 * spec.nv + 9) * spec.nu + 20
     y = np.zeros(spec.m, dtype=np.float32)

@@ -28,9 +28,9 @@ def ct():
     return _ct
 
 
-def par2d(nx, ny, views, nu):
+def par2d(nx, ny, views, nu, ang0=0.15):
     return ci.Geometry(name="par2d_%dx%d_%d_%d" % (nx, ny, views, nu), kind=ci.PARALLEL_2D, nx=nx, ny=ny, nz=1,
-                       vox=1.0, n_views=views, ang0=0.15, span=math.pi, nu=nu, nv=1, du=1.0, dv=1.0)
+                       vox=1.0, n_views=views, ang0=ang0, span=math.pi, nu=nu, nv=1, du=1.0, dv=1.0)
 
 
 SCANS = [
@@ -43,6 +43,9 @@ SCANS = [
     par2d(61, 70, 80, 450),   # 4
     par2d(40, 48, 150, 500),  # 2
     par2d(130, 97, 500, 400),  # 1
+    # whole warps of rays beside the image, parallel to its sides but for a slope of 1e-17
+    par2d(24, 22, 10, 160, ang0=0.0),
+    par2d(181, 181, 270, 257, ang0=0.0),
 ]
 
 
