@@ -43,6 +43,9 @@ SCANS = [
     par2d(61, 70, 80, 450),   # 4
     par2d(40, 48, 150, 500),  # 2
     par2d(130, 97, 500, 400),  # 1
+    # the largest image that is read without copies, and the next
+    par2d(96, 96, 500, 400),
+    par2d(97, 96, 60, 150),
     # whole warps of rays beside the image, parallel to its sides but for a slope of 1e-17
     par2d(24, 22, 10, 160, ang0=0.0),
     par2d(181, 181, 270, 257, ang0=0.0),
