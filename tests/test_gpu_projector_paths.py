@@ -64,3 +64,14 @@ def test_projector_kernels_match_oracle(ct, spec, dtype):
     ref = oracle.project_A(spec, xd.double().numpy()).reshape(y.shape)
     assert np.linalg.norm(y - ref) <= OP_TOL * np.linalg.norm(ref)
 
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("spec", [s for s in SCANS if s.kind == ci.PARALLEL_2D], ids=lambda s: s.name)
+def test_images_read_in_place_match_the_copies(ct, spec, dtype):
+    # ct_project_A_noalloc always makes copies; the operations are the same
+    g = ct.Geometry.from_spec(spec, vol_dtype=dtype)
+    x = torch.from_numpy(ci.random_vector(spec.n, seed=82).astype(np.float32).reshape(spec.vol_shape)).cuda()
+    y = torch.empty(spec.sino_shape, device="cuda")
+    ct.ct_project_A_noalloc(g, x, y)
+    assert torch.equal(ct.project_A(g, x), y)
