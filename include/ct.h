@@ -122,8 +122,9 @@ typedef struct {
 CT_API void ct_solve_opts_default(ct_solve_opts *opts);
 
 /* Creates a geometry handle on the current device: validates the
- * description (positive sizes, 2D needs nz = nv = 1, cone needs
- * sdd > sod > 0 and the volume inside the source circle) and
+ * description (positive sizes, lengths finite in single precision, 2D needs
+ * nz = nv = 1, cone needs sdd > sod > 0 and the volume inside the source
+ * circle) and
  * uploads per-view tables; storage dtypes CT_F32 or CT_BF16.  The library owns the handle; free it with
  * ct_geom_destroy.  Returns CT_EINVAL or CT_ECUDA on failure (*out = NULL). */
 CT_API ct_status ct_geom_create(const ct_geom_desc *desc, ct_geom **out);

@@ -206,6 +206,12 @@ ct_status ct_geom_create(const ct_geom_desc *d, ct_geom **out)
         return set_error(CT_EINVAL, "all grid, detector and view counts must be positive");
     if (!(d->voxel_mm > 0) || !(d->du_mm > 0) || !(d->dv_mm > 0))
         return set_error(CT_EINVAL, "voxel and pixel sizes must be positive");
+    // the kernels compute in FP32 (2D scans use neither dv nor the distances)
+    const bool has_depth = d->kind == CT_CONE_3D;
+    for (double len : {d->voxel_mm, d->du_mm, has_depth ? d->dv_mm : 1.0, has_depth ? d->sod_mm : 1.0,
+                       has_depth ? d->sdd_mm : 1.0})
+        if (!std::isfinite(float(len)))
+            return set_error(CT_EINVAL, "lengths must be finite in single precision (got %g mm)", len);
     if (!std::isfinite(d->angle_start_rad) || !std::isfinite(d->angle_span_rad))
         return set_error(CT_EINVAL, "view angles must be finite");
     if (d->projector != CT_PROJ_JOSEPH && d->projector != CT_PROJ_SIDDON)
@@ -234,6 +240,8 @@ ct_status ct_geom_create(const ct_geom_desc *d, ct_geom **out)
         const int nz_run = d->nz == 1 ? 1 : (d->nz + B_ZC_RUN_MAX - 1) / B_ZC_RUN_MAX * B_ZC_RUN_MAX;
         const double zslices = std::max(0.5 * (d->nz - 1), nz_run - 1 - 0.5 * (d->nz - 1));
         const double over = zslices * vx * mmax / d->dv_mm - 0.5 * (d->nv - 1);
+        if (!(over < 1e9))   // (past what an int holds)
+            return set_error(CT_EINVAL, "problem too large for 32-bit element indexing");
         padv = std::max(PAD_V, int(std::ceil(std::max(over, 0.0))) + PAD_V);
     }
 #ifdef CT_CHECK_BOUNDS
@@ -305,10 +313,14 @@ ct_status ct_geom_create(const ct_geom_desc *d, ct_geom **out)
     //   a_zsafe:  |z| stays within the grid plus one voxel, so no clamp is needed;
     //             checked over the rows the threads compute, which run up to
     //             the next multiple of the rays per thread past nv.
+    // Neither is set where an extreme is not a number, or where the walk's own
+    // FP32 coordinates can leave FP32's range: the unclamped walk takes its row
+    // from the bits of z, so a NaN would address outside the copies, while the
+    // clamped one carries it to the result.
     k.a_window = 0;
     k.a_zsafe = 1;
     if (cone) {
-        double smin = 1e300, smax = -1e300;
+        bool window = true;
         const int nv_run = (d->nv + A_VR - 1) / A_VR * A_VR;
         const double vmax = std::max(0.5 * (d->nv - 1), nv_run - 1 - 0.5 * (d->nv - 1)) * d->dv_mm;
         for (int s = 0; s < d->n_views; ++s) {
@@ -324,13 +336,20 @@ ct_status ct_geom_create(const ct_geom_desc *d, ct_geom **out)
                     double cp = (e ? 0.5 : -0.5) * (Na - 1) * vox;
                     double ratio = (cp - Sa) / da;
                     double sig = d->dv_mm * ratio / vox;
-                    smin = std::min(smin, sig);
-                    smax = std::max(smax, sig);
-                    if (vmax * std::fabs(ratio) / vox > 0.5 * (d->nz - 1) + 1.0) k.a_zsafe = 0;
+                    window = window && sig >= 0.0 && sig <= 0.98;
+                    if (!(vmax * std::fabs(ratio) / vox <= 0.5 * (d->nz - 1) + 1.0)) k.a_zsafe = 0;
                 }
             }
         }
-        k.a_window = (smin >= 0.0 && smax <= 0.98) ? 1 : 0;
+        // u, and the extreme of z = (row) (dv / d_a) (plane - S_a / vox): |d_a| >= sdd / sqrt(2)
+        const float u_max = k.du * float(d->nu);
+        const float z_max = k.dv / (0.5f * k.sdd) * float(nv_run) *
+                            (float(d->sod_mm) * k.inv_vox + float(std::max(d->nx, d->ny)));
+        if (!std::isfinite(u_max) || !std::isfinite(z_max)) {
+            window = false;
+            k.a_zsafe = 0;
+        }
+        k.a_window = window ? 1 : 0;
     }
 #ifdef CT_CHECK_BOUNDS
     // checked builds only: the projector may be told that no z clamp is
