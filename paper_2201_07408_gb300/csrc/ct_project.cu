@@ -316,27 +316,19 @@ __device__ __forceinline__ float row_lerp(const float *p, float wb)
     return fmaf(wb, v1 - v0, v0);
 }
 
-// One ray's sample on plane p from its plane row: z interpolated between two
-// rows of the copy, or (FLAT: a 2D scan, whose rays stay in its one slice) the
-// row itself.
-template <bool FLAT, bool BF>
-__device__ __forceinline__ float plane_sample(const GeomDev &g, const float *rowp, int zstride, float wb, float fz)
-{
-    if (FLAT) return row_lerp<BF>(rowp, wb);
-    const float z0f = floorf(fz);
-    const float *r = rowp + min(max(int(z0f), -PAD_A), g.nz) * zstride;
-    const float lo = row_lerp<BF>(r, wb), hi = row_lerp<BF>(r + zstride, wb);
-    return fmaf(fz - z0f, hi - lo, lo);
-}
-
 // The walk of detectors with one row (2D scans above all).  A scan has few
 // rays (8550 of them for 64 x 64 pixels and 90 views: two warps an SM), so
-// what bounds it is one ray's chain of loads: `split` (1, 2, 4 or 8) of a
-// block's 8 warps share the planes of a ray and add their sums.  One warp a
-// ray and two interpolated rows took 15.9 us for that scan, this 8.2 us; 256 x
-// 256 with 360 views 69.9 -> 57.7 us, 512 x 512 with 720 views 321 -> 227 us.
-// DIRECT: small images are read where they are (Xc is the volume; cells off the
-// grid read as zero, bf16 storage rounds what it reads), without copies.
+// what bounds it is one ray's chain of loads.  `split` (1, 2, 4 or 8) of a
+// block's 8 warps share the planes of a ray and add their sums, and a thread
+// fetches a batch of planes before it adds any: a loop that steps by `split`
+// is not unrolled into one by the compiler (1000 x 100 pixels with 90 views:
+// 196 us without batches, at any unroll factor).  FLAT: a 2D scan, whose rays
+// stay in its one slice.  DIRECT: small images are read where they are (Xc is
+// the volume; cells off the grid read as zero, bf16 storage rounds what it
+// reads), without copies.
+// Projections with their copies, two interpolated rows a plane and one warp a
+// ray against this: 64 x 64 with 90 views 18.7 -> 10.0 us, 512 x 512 with 720
+// views 325 -> 190 us, 1000 x 100 with 90 views 129 -> 41 us (bf16 84 -> 45 us).
 template <bool FLAT, bool BF, bool DIRECT>
 __global__ void __launch_bounds__(256) joseph_A_row_kernel(GeomDev g, const float *__restrict__ Xc,
                                                            const float *__restrict__ Yc, float *__restrict__ y,
@@ -344,6 +336,8 @@ __global__ void __launch_bounds__(256) joseph_A_row_kernel(GeomDev g, const floa
                                                            const int *__restrict__ stop)
 {
     if (stop && *stop) return;
+    // planes a batch (8 of bf16 pairs, whose one load a row is half as long a chain, are slower)
+    constexpr int BATCH = BF ? 4 : 8;
     __shared__ float part[8][32];
     const int w = threadIdx.y, wp = w % split;   // the warp's share of its rays' planes
     const int lane_u = (blockIdx.x * (8 / split) + w / split) * 32 + threadIdx.x;
@@ -354,26 +348,61 @@ __global__ void __launch_bounds__(256) joseph_A_row_kernel(GeomDev g, const floa
     const int zstride = c.Na * pitch;
     // (z = 0, plane 0, b = 0) in the padded copy
     const float *__restrict__ base = (c.xdom ? Xc : Yc) + PAD_A * zstride + PAD_A;
-    float acc = 0.0f;
-#pragma unroll 4
-    for (int p = c.p0 + wp; p <= c.p1; p += split) {
+    struct Sample {
+        float wb, wz;
+        float lo[2], hi[2];   // the two cells of the sample's row and of the row above (bf16 copies: a pair in the first)
+    };
+    auto fetch = [&](int p) {
+        Sample t;
         const float pm = float(p) - c.ca;
         const float fb = fmaf(pm, c.gb, c.fbc);
         const float b0f = floorf(fb);
         const int b0 = min(max(int(b0f), -PAD_A), c.Nb);
+        t.wb = fb - b0f;
         if (DIRECT) {
             const float *v = Xc + (c.xdom ? b0 * g.nx + p : p * g.nx + b0);
-            float v0 = b0 >= 0 && b0 < c.Nb ? __ldg(v) : 0.0f;
-            float v1 = b0 + 1 >= 0 && b0 + 1 < c.Nb ? __ldg(v + (c.xdom ? g.nx : 1)) : 0.0f;
-            if (BF) {
-                v0 = __bfloat162float(__float2bfloat16_rn(v0));
-                v1 = __bfloat162float(__float2bfloat16_rn(v1));
-            }
-            acc += fmaf(fb - b0f, v1 - v0, v0);
+            t.lo[0] = b0 >= 0 && b0 < c.Nb ? __ldg(v) : 0.0f;
+            t.lo[1] = b0 + 1 >= 0 && b0 + 1 < c.Nb ? __ldg(v + (c.xdom ? g.nx : 1)) : 0.0f;
         } else {
-            acc += plane_sample<FLAT, BF>(g, base + p * pitch + b0, zstride, fb - b0f, fmaf(c.gz0, pm - c.Sv, g.cz));
+            const float *r = base + p * pitch + b0;
+            if (!FLAT) {
+                const float fz = fmaf(c.gz0, pm - c.Sv, g.cz);
+                const float z0f = floorf(fz);
+                t.wz = fz - z0f;
+                r += min(max(int(z0f), -PAD_A), g.nz) * zstride;
+                t.hi[0] = __ldg(r + zstride);
+                if (!BF) t.hi[1] = __ldg(r + zstride + 1);
+            }
+            t.lo[0] = __ldg(r);
+            if (!BF) t.lo[1] = __ldg(r + 1);
         }
+        return t;
+    };
+    auto lerp = [&](const float (&v)[2], float wb) {   // (1 - wb) V[b0] + wb V[b0 + 1]
+        float v0 = v[0], v1 = v[1];
+        if (BF && DIRECT) {
+            v0 = __bfloat162float(__float2bfloat16_rn(v0));
+            v1 = __bfloat162float(__float2bfloat16_rn(v1));
+        } else if (BF) {
+            v0 = bf16_lo(__float_as_uint(v[0]));
+            v1 = bf16_hi(__float_as_uint(v[0]));
+        }
+        return fmaf(wb, v1 - v0, v0);
+    };
+    auto value = [&](const Sample &t) {
+        const float lo = lerp(t.lo, t.wb);
+        return FLAT ? lo : fmaf(t.wz, lerp(t.hi, t.wb) - lo, lo);
+    };
+    float acc = 0.0f;
+    int p = c.p0 + wp;
+    for (; p + (BATCH - 1) * split <= c.p1; p += BATCH * split) {
+        Sample t[BATCH];
+#pragma unroll
+        for (int k = 0; k < BATCH; ++k) t[k] = fetch(p + k * split);
+#pragma unroll
+        for (int k = 0; k < BATCH; ++k) acc += value(t[k]);
     }
+    for (; p <= c.p1; p += split) acc += value(fetch(p));
     part[w][threadIdx.x] = acc;
     __syncthreads();
     if (wp > 0 || !live) return;
@@ -552,10 +581,14 @@ template <bool FLAT, bool BF, bool DIRECT>
 static void launch_joseph_A_row(const GeomDev &g, const float *Xc, const float *Yc, float *y, SinoLayout lay,
                                 const int *stop, cudaStream_t st)
 {
-    // warps a ray: as many (up to 8) as keep the grid within 32 warps an SM
+    // warps a ray: as many (up to 8) as keep the grid within 96 warps an SM, about two
+    // waves; rays leave the image after different numbers of planes, so more and
+    // shorter shares even out (32 warps an SM: 9 x 1000 pixels, 90 views 114 us
+    // against 36 us, 300 x 300, 180 views 50 against 31 us)
     const int tiles = (g.nu + 31) / 32;
+    const size_t most = size_t(num_sms()) * 96;
     int split = 1;
-    while (split < 8 && size_t(tiles) * g.n_views * split * 2 <= size_t(num_sms()) * 32) split *= 2;
+    while (split < 8 && size_t(tiles) * g.n_views * split * 2 <= most) split *= 2;
     const dim3 block(32, 8), grid((tiles * split + 7) / 8, 1, g.n_views);
     joseph_A_row_kernel<FLAT, BF, DIRECT><<<grid, block, 0, st>>>(g, Xc, Yc, y, lay, split, stop);
 }
