@@ -398,28 +398,17 @@ __device__ __forceinline__ float4 load_quad(const void *base, size_t e)
     return __ldg(static_cast<const float4 *>(base) + e);
 }
 
-// A row's interpolation along u from one half of a quad entry: the row's
-// value and step (DIFF) or its two values.
-template <bool BF, bool DIFF>
-__device__ __forceinline__ float row_value(const char *half, float wu)
-{
-    float2 e;
-    if (BF) {
-        const uint32_t w = __ldg(reinterpret_cast<const uint32_t *>(half));
-        e = make_float2(bf16_lo(w), bf16_hi(w));
-    } else {
-        e = __ldg(reinterpret_cast<const float2 *>(half));
-    }
-    return fmaf(wu, DIFF ? e.y : e.y - e.x, e.x);
-}
-
 // Small volumes: a run of ZC slices a thread, and `split` (1, 2, 4 or 8) of a
 // block's 8 warps share the views of their 32 columns and add their sums.  A
 // 64 x 64 slice has 4096 voxels, less than one warp an SM, and a voxel's views
-// are a chain of loads, which is what bounds it.  FLAT: 2D scans, whose one
-// detector row is half a quad.  Against one block for 32 x 32 voxels (2D) and
-// the slab kernel below (3D): 64 x 64 with 90 views 38 -> 11 us, 512 x 512 with
-// 720 views 384 -> 325 us; 32^3 47 -> 10 us, 64^3 92 -> 36 us, 96^3 138 -> 123 us.
+// are a chain of loads, which is what bounds it.  A single slice fetches a batch
+// of views before it adds any (the compiler does not make one of a loop that
+// steps by `split` and skips views).  FLAT: 2D scans, whose one detector row is
+// half a quad.  Against one block for 32 x 32 voxels (2D) and the slab kernel
+// below (3D), whole calls: 64 x 64 with 90 views 41 -> 11 us, 300 x 300 with 720
+// views 271 -> 145 us (319 us in a plain loop), 512 x 512 with 720 views 400 ->
+// 317 us, 672 x 888 with 400 views 429 -> 376 us; kernels alone 32^3 47 -> 10 us,
+// 64^3 92 -> 36 us, 96^3 138 -> 123 us.
 template <int ZC, bool FLAT, bool BF, bool DIFF>
 __global__ void __launch_bounds__(256) voxel_B_small_kernel(GeomDev g, const void *__restrict__ ypad,
                                                             float *__restrict__ x, int split,
@@ -434,32 +423,83 @@ __global__ void __launch_bounds__(256) voxel_B_small_kernel(GeomDev g, const voi
     const float xc = (float(min(ix, g.nx - 1)) - g.cx) * g.vox, yc = (float(min(iy, g.ny - 1)) - g.cy) * g.vox;
     const float zfirst = (float(iz0) - g.cz) * g.vox;
     const size_t view_stride = size_t(g.nvp) * g.pitchU;
+    // the entry of a column in the view's first detector row
+    auto entry = [&](const ColumnView &c, int s) {
+        int col = c.col;
+        if (!c.skip && !CT_IN_BOUNDS(g, unsigned(col) < unsigned(g.pitchU), BS_B_COL, s, col)) col = 0;
+        return static_cast<const char *>(ypad) + ENTRY * (s * view_stride + size_t(g.padv) * g.pitchU + col);
+    };
+    auto row_of = [&](float v0f, int s) {
+        int row = int(v0f);
+        if (!CT_IN_BOUNDS(g, unsigned(row + g.padv) < unsigned(g.nvp), BS_B_ROW, s, row + g.padv)) row = -g.padv;
+        return row;
+    };
     float acc[ZC];
 #pragma unroll
     for (int k = 0; k < ZC; ++k) acc[k] = 0.0f;
-#pragma unroll(ZC > 1 ? 2 : 4)
-    for (int s = share; s < g.n_views; s += split) {
-        const ColumnView c = column_view(g, s, xc, yc, zfirst);
-        if (c.skip) continue;
-        int col = c.col;
-        if (!CT_IN_BOUNDS(g, unsigned(col) < unsigned(g.pitchU), BS_B_COL, s, col)) col = 0;
-        const char *pv = static_cast<const char *>(ypad) + ENTRY * (s * view_stride + size_t(g.padv) * g.pitchU + col);
-#pragma unroll
-        for (int k = 0; k < ZC; ++k) {
-            const float fv = fmaf(float(k), c.gv, c.fv0);
-            const float v0f = FLAT ? 0.0f : floorf(fv);
-            int row = int(v0f);
-            if (!CT_IN_BOUNDS(g, unsigned(row + g.padv) < unsigned(g.nvp), BS_B_ROW, s, row + g.padv)) row = -g.padv;
-            const char *p = pv + ptrdiff_t(row) * (ENTRY * g.pitchU);
-            float r;
-            if (FLAT) {
-                r = row_value<BF, DIFF>(p, c.wu);
-            } else {
-                const float4 q = load_quad<BF>(p, 0);
-                r = fmaf(c.wu, DIFF ? q.y : q.y - q.x, q.x);
-                r = fmaf(fv - v0f, fmaf(c.wu, DIFF ? q.w : q.w - q.z, q.z) - r, r);
+    if constexpr (ZC == 1) {
+        constexpr int BATCH = 8;
+        struct Sample {
+            float w, wu, wv;
+            float lo[2], hi[2];   // rows v and v + 1 of the entry (bf16: each a pair in the first)
+        };
+        auto fetch = [&](int s) {
+            Sample t;
+            const ColumnView c = column_view(g, s, xc, yc, zfirst);
+            const float v0f = FLAT ? 0.0f : floorf(c.fv0);
+            const char *p = entry(c, s) + ptrdiff_t(row_of(v0f, s)) * (ENTRY * g.pitchU);
+            t.w = t.wu = t.wv = t.lo[0] = t.lo[1] = t.hi[0] = t.hi[1] = 0.0f;   // a skipped view adds zero
+            if (!c.skip) {
+                t.w = c.w;
+                t.wu = c.wu;
+                t.wv = c.fv0 - v0f;
+                if (BF) {
+                    t.lo[0] = __uint_as_float(__ldg(reinterpret_cast<const uint32_t *>(p)));
+                    if (!FLAT) t.hi[0] = __uint_as_float(__ldg(reinterpret_cast<const uint32_t *>(p) + 1));
+                } else if (FLAT) {
+                    const float2 q = __ldg(reinterpret_cast<const float2 *>(p));
+                    t.lo[0] = q.x, t.lo[1] = q.y;
+                } else {
+                    const float4 q = __ldg(reinterpret_cast<const float4 *>(p));
+                    t.lo[0] = q.x, t.lo[1] = q.y, t.hi[0] = q.z, t.hi[1] = q.w;
+                }
             }
-            acc[k] = fmaf(c.w, r, acc[k]);
+            return t;
+        };
+        auto lerp = [&](const float (&e)[2], float wu) {   // a row's value and step (DIFF) or its two values
+            const float e0 = BF ? bf16_lo(__float_as_uint(e[0])) : e[0];
+            const float e1 = BF ? bf16_hi(__float_as_uint(e[0])) : e[1];
+            return fmaf(wu, DIFF ? e1 : e1 - e0, e0);
+        };
+        auto add = [&](const Sample &t) {
+            float r = lerp(t.lo, t.wu);
+            if (!FLAT) r = fmaf(t.wv, lerp(t.hi, t.wu) - r, r);
+            acc[0] = fmaf(t.w, r, acc[0]);
+        };
+        int s = share;
+        for (; s + (BATCH - 1) * split < g.n_views; s += BATCH * split) {
+            Sample t[BATCH];
+#pragma unroll
+            for (int k = 0; k < BATCH; ++k) t[k] = fetch(s + k * split);
+#pragma unroll
+            for (int k = 0; k < BATCH; ++k) add(t[k]);
+        }
+        for (; s < g.n_views; s += split) add(fetch(s));
+    } else {
+#pragma unroll 2
+        for (int s = share; s < g.n_views; s += split) {
+            const ColumnView c = column_view(g, s, xc, yc, zfirst);
+            if (c.skip) continue;
+            const char *pv = entry(c, s);
+#pragma unroll
+            for (int k = 0; k < ZC; ++k) {
+                const float fv = fmaf(float(k), c.gv, c.fv0);
+                const float v0f = floorf(fv);
+                const float4 q = load_quad<BF>(pv + ptrdiff_t(row_of(v0f, s)) * (ENTRY * g.pitchU), 0);
+                float r = fmaf(c.wu, DIFF ? q.y : q.y - q.x, q.x);
+                r = fmaf(fv - v0f, fmaf(c.wu, DIFF ? q.w : q.w - q.z, q.z) - r, r);
+                acc[k] = fmaf(c.w, r, acc[k]);
+            }
         }
     }
 #pragma unroll
