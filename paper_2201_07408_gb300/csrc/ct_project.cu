@@ -814,12 +814,20 @@ cudaError_t launch_project_At(const GeomDev &g, const float *y, float *x, float 
 
 using namespace ct;
 
-// 2D images of at most this many pixels are projected without copies: one
-// launch instead of two, while a walk down the columns of the image still finds
-// its lines in L1.  Kernels of a call, with copies and without: 64 x 64 pixels,
-// 90 views 15.2 and 12.7 us; 96 x 96, 140 views 18.6 and 17.1 us; 128 x 128, 180
-// views 21.0 and 20.8 us.
-constexpr size_t kDirectPixels = 96 * 96;
+// 2D images that are projected without copies: one launch instead of two.  Small
+// ones (96 x 96 pixels), while a call is short: a sample costs more than one
+// from the copies, whose lanes always read along a row, and most where rows are
+// multiples of 64 bytes, since a column of the image then lies in few of L1's
+// sets.  Samples (rays times planes) at which the two cross: 64 x 64 4e6, 96 x 96
+// between 1.2e6 and 5e6, 128 x 72 between 2e6 and 7e6, against 72 x 128 over 3e7,
+// 60 x 150 over 4e7, 9 x 1000 1e8.  Direct and with copies: 64 x 64 pixels, 90
+// views 7.2 and 11.0 us; 96 x 96, 90 views 10.1 and 12.4; 96 x 96, 1500 views 82 and 36.
+static bool reads_in_place(const GeomDev &g)
+{
+    const double samples = double(g.n_views) * g.nu * std::max(g.nx, g.ny);
+    return g.kind == CT_PARALLEL_2D && !g.siddon && size_t(g.nx) * g.ny <= 96 * 96 &&
+           samples <= (g.nx % 16 ? 3e7 : 4e6);
+}
 
 extern "C" ct_status ct_project_A(const ct_geom *geom, const float *x_dev, float *y_dev, void *stream)
 {
@@ -827,7 +835,7 @@ extern "C" ct_status ct_project_A(const ct_geom *geom, const float *x_dev, float
     if (!geom || !x_dev || !y_dev) return set_error(CT_EINVAL, "ct_project_A: NULL argument");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const GeomDev &g = geom->g;
-    if (g.kind == CT_PARALLEL_2D && !g.siddon && geom->n <= kDirectPixels) {
+    if (reads_in_place(g)) {
         ProfScope prof(PK_JOSEPH_A, st);
         if (g.vol_bf16)
             launch_joseph_A_row<true, true, true>(g, x_dev, x_dev, y_dev, plain_layout(g), nullptr, st);
