@@ -672,13 +672,19 @@ __global__ void __launch_bounds__(32 * TY, MINB) voxel_B_slab_kernel(GeomDev g, 
     }
 }
 
+// views, the tile, and the views listed by orientation
+static size_t slab_smem(const GeomDev &g, int zc, int ty)
+{
+    return size_t(g.n_views) * 2 * sizeof(float4) + size_t(zc) * ty * (B_TILE + 1) * sizeof(float) +
+           size_t(g.n_views) * sizeof(short);
+}
+
 template <int ZC, int TY, int MINB, bool BF, bool DIFF>
 static cudaError_t launch_voxel_B_slab(const GeomDev &g, const float *ypad, float *x, const int *stop,
                                        cudaStream_t st)
 {
     dim3 block(32, TY);
-    const size_t smem = size_t(g.n_views) * 2 * sizeof(float4) + size_t(ZC) * TY * (B_TILE + 1) * sizeof(float) +
-                        size_t(g.n_views) * sizeof(short);
+    const size_t smem = slab_smem(g, ZC, TY);
     cudaError_t e = raise_dyn_smem(reinterpret_cast<const void *>(voxel_B_slab_kernel<ZC, TY, MINB, BF, DIFF>), smem);
     if (e != cudaSuccess) return e;
     dim3 grid((g.nx + 31) / 32, (g.ny + TY - 1) / TY, (g.nz + ZC - 1) / ZC);
@@ -686,29 +692,42 @@ static cudaError_t launch_voxel_B_slab(const GeomDev &g, const float *ypad, floa
     return cudaGetLastError();
 }
 
+// warps that share a run's views: as many (up to 8) as keep the grid within 32 warps an SM
+static int small_split(const GeomDev &g, int zc)
+{
+    const size_t warps = size_t((g.nx + 31) / 32) * g.ny * ((g.nz + zc - 1) / zc), most = size_t(num_sms()) * 32;
+    int split = 1;
+    while (split < 8 && warps * split * 2 <= most) split *= 2;
+    return split;
+}
+
+static dim3 small_grid(const GeomDev &g, int zc)
+{
+    return dim3((g.nx + 31) / 32 * ((g.ny * small_split(g, zc) + 7) / 8), (g.nz + zc - 1) / zc);
+}
+
 template <int ZC, bool FLAT, bool BF, bool DIFF>
 static cudaError_t launch_voxel_B_small(const GeomDev &g, const float *ypad, float *x, const int *stop,
                                         cudaStream_t st)
 {
-    // warps a run: as many (up to 8) as keep the grid within 32 warps an SM
-    const int tiles = (g.nx + 31) / 32, runs = (g.nz + ZC - 1) / ZC;
-    int split = 1;
-    while (split < 8 && size_t(tiles) * g.ny * runs * split * 2 <= size_t(num_sms()) * 32) split *= 2;
-    const dim3 block(32, 8), grid(tiles * ((g.ny * split + 7) / 8), runs);
-    voxel_B_small_kernel<ZC, FLAT, BF, DIFF><<<grid, block, 0, st>>>(g, ypad, x, split, stop);
+    voxel_B_small_kernel<ZC, FLAT, BF, DIFF>
+        <<<small_grid(g, ZC), dim3(32, 8), 0, st>>>(g, ypad, x, small_split(g, ZC), stop);
     return cudaGetLastError();
 }
 
-// Slab blocks of ZC slices, and the time of the waves they take: a block of 12
-// slices costs 0.83 of one of 16 (4.76 ms against 4.17 ms for 256^3).
-static size_t slab_blocks(const GeomDev &g, int zc)
+// The time that slab blocks of ZC slices take.  FP32 entries: waves of 4 blocks
+// an SM, a block of 12 slices 0.83 of one of 16 (4.76 ms against 4.17 ms for
+// 256^3).  bf16 entries are bound by issue slots, so by an SM's blocks (two at
+// least: fewer do not hide their loads), 0.79 of one of 16.  With the FP32 rule
+// bf16 volumes that do not fill the SMs took 12 slices where 16 are faster: 160 x
+// 160 x 48, 360 views, 421 us against 391; 81 x 117 x 138 579 against 553.
+static double slab_cost(const GeomDev &g, int zc, bool bf)
 {
-    return size_t((g.nx + 31) / 32) * ((g.ny + 7) / 8) * ((g.nz + zc - 1) / zc);
-}
-static double slab_cost(const GeomDev &g, int zc)
-{
-    const size_t slots = size_t(num_sms()) * 4;
-    return double((slab_blocks(g, zc) + slots - 1) / slots) * (zc + 7.5);
+    const size_t sms = num_sms(), waves = sms * 4;
+    const size_t blocks = size_t((g.nx + 31) / 32) * ((g.ny + 7) / 8) * ((g.nz + zc - 1) / zc);
+    if (!bf) return double((blocks + waves - 1) / waves) * (zc + 7.5);
+    const size_t rest = blocks % waves;
+    return double(blocks / waves * 4 + (rest ? std::max<size_t>(2, (rest + sms - 1) / sms) : 0)) * (zc + 3.0);
 }
 
 template <bool BF, bool DIFF>
@@ -716,14 +735,19 @@ static cudaError_t launch_voxel_B_t(const GeomDev &g, const float *ypad, float *
 {
     if (g.kind == CT_PARALLEL_2D) return launch_voxel_B_small<1, true, BF, DIFF>(g, ypad, x, stop, st);
     if (g.nz == 1) return launch_voxel_B_small<1, false, BF, DIFF>(g, ypad, x, stop, st);
-    // where the slab kernel's blocks do not fill the SMs (about 100^3; its
-    // samples cost half the small kernel's once they do)
-    if (slab_blocks(g, B_ZC_SLAB) < size_t(num_sms()) * (BF ? 1 : 2))
+    // where the small kernel's blocks are resident at once (about 100^3; its
+    // samples cost twice the slab kernel's, whose blocks are too few there): 6
+    // blocks an SM on FP32 entries, 4 on bf16.  Just past the line, 360 views, small
+    // kernel and slabs: 256 x 256 x 16 489 and 424 us, 128 x 128 x 64 628 and 540;
+    // before it, 112 x 112 x 64 374 and 510, 96^3 378 and 479; bf16 80^3 284 and 321.
+    // (And where the slab kernel's shared memory does not hold the views.)
+    const dim3 small = small_grid(g, 4);
+    if (size_t(small.x) * small.y <= size_t(num_sms()) * (BF ? 4 : 6) || slab_smem(g, B_ZC_SLAB, 8) > 226 * 1024)
         return launch_voxel_B_small<4, false, BF, DIFF>(g, ypad, x, stop, st);
     // runs of 12 where 16 leave a last wave nearly empty (160 x 152 x 100: 593 -> 496 us); the row margin
     // covers multiples of 16 past nz
     const bool covered = (g.nz + 11) / 12 * 12 <= (g.nz + B_ZC_SLAB - 1) / B_ZC_SLAB * B_ZC_SLAB;
-    if (covered && slab_cost(g, 12) < slab_cost(g, B_ZC_SLAB))
+    if (covered && slab_cost(g, 12, BF) < slab_cost(g, B_ZC_SLAB, BF))
         return launch_voxel_B_slab<12, 8, 4, BF, DIFF>(g, ypad, x, stop, st);
     return launch_voxel_B_slab<B_ZC_SLAB, 8, 4, BF, DIFF>(g, ypad, x, stop, st);
 }
