@@ -122,14 +122,6 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b)
 // r = 1, 2, k < N/3, follow.  Lanes with consecutive k read
 // consecutive entries (in the full-length table they are N/(4 Ns) entries
 // apart, all in one bank).
-__device__ __forceinline__ int fft_radix4_points(int N)
-{
-    const int P = N % 3 == 0 ? N / 3 : N;   // the power of two in N
-    int Ns = 1;
-    while (Ns * 4 <= P) Ns *= 4;
-    return Ns;
-}
-
 // Buffer element i lives at slot fsw(i): within each aligned block of 16
 // elements the low four bits are XORed with 5 ((i >> 4) mod 4).  The
 // radix-4 stages after 1 and 4 combined points write elements 4t + r and
@@ -141,10 +133,12 @@ __device__ __forceinline__ int fsw(int i) { return i ^ (5 * ((i >> 4) & 3)); }
 
 // One FFT of length N (= 4 T) by the T threads of a group; a holds the input
 // and receives the output, b is scratch.  Every thread of the block calls it
-// (it synchronises the block).
+// (it synchronises the block).  R3: N is three times a power of two (a kernel of
+// its own: short rows took 5 % longer in one that asks).
+template <bool R3>
 __device__ __forceinline__ void fft_group(float2 *&a, float2 *&b, const float2 *__restrict__ stw, int N, int t)
 {
-    const int T = N >> 2, P = N % 3 == 0 ? N / 3 : N;
+    const int T = N >> 2, P = R3 ? N / 3 : N;
     int Ns = 1;
     for (; Ns * 4 <= P; Ns *= 4) {
         const int k = t & (Ns - 1);
@@ -185,7 +179,7 @@ __device__ __forceinline__ void fft_group(float2 *&a, float2 *&b, const float2 *
         w += Ns;
         Ns *= 2;
     }
-    if (P < N) {   // a last radix-3 stage, Ns = N / 3: one butterfly a thread and a third one for every third
+    if (R3) {   // a last radix-3 stage, Ns = N / 3: one butterfly a thread and a third one for every third
         for (int j = t; j < Ns; j += T) {
             const float2 v0 = a[fsw(j)], v1 = cmul(a[fsw(j + Ns)], w[j]), v2 = cmul(a[fsw(j + 2 * Ns)], w[Ns + j]);
             const float2 s = make_float2(v1.x + v2.x, v1.y + v2.y);
@@ -221,6 +215,7 @@ static FftShape fft_shape(int N)
     return f;
 }
 
+template <bool R3>
 __global__ void ramp_fft_kernel(GeomDev g, const float *__restrict__ src, float *__restrict__ dst, SinoLayout lay,
                                 int transpose, const int *__restrict__ stop)
 {
@@ -236,8 +231,8 @@ __global__ void ramp_fft_kernel(GeomDev g, const float *__restrict__ src, float 
     for (int i = threadIdx.x; i < N; i += blockDim.x) H[i] = g.fft_h[i];
     {
         int Ns = 1;
-        const int P = N % 3 == 0 ? N / 3 : N, N4 = fft_radix4_points(N);
-        for (; Ns < N4; Ns *= 4)   // radix-4 entries (Ns - 1) + (r - 1) Ns + k = tw[r k N / (4 Ns)]
+        const int P = R3 ? N / 3 : N;   // the power of two in N
+        for (; Ns * 4 <= P; Ns *= 4)   // radix-4 entries (Ns - 1) + (r - 1) Ns + k = tw[r k N / (4 Ns)]
             for (int i = threadIdx.x; i < 3 * Ns; i += blockDim.x) {
                 const int r = i / Ns + 1, k = i - (r - 1) * Ns;
                 stw[(Ns - 1) + i] = g.fft_tw[r * k * (N / (4 * Ns))];
@@ -247,7 +242,7 @@ __global__ void ramp_fft_kernel(GeomDev g, const float *__restrict__ src, float 
             for (int i = threadIdx.x; i < Ns; i += blockDim.x) w[i] = g.fft_tw[i * (N / (2 * Ns))];
             w += Ns;
         }
-        if (P < N)      // and a radix-3 stage: tw[r k], k < N / 3
+        if (R3)         // and a radix-3 stage: tw[r k], k < N / 3
             for (int i = threadIdx.x; i < 2 * P; i += blockDim.x) w[i] = g.fft_tw[i < P ? i : 2 * (i - P)];
     }
     const int nu = g.nu;
@@ -274,13 +269,13 @@ __global__ void ramp_fft_kernel(GeomDev g, const float *__restrict__ src, float 
             a[fsw(u)] = z;
         }
         __syncthreads();
-        fft_group(a, b, stw, N, t);
+        fft_group<R3>(a, b, stw, N, t);
         for (int k = t; k < N; k += T) {   // conj(Z) H / N
             const float2 z = a[fsw(k)];
             a[fsw(k)] = make_float2(z.x * H[k], -z.y * H[k]);
         }
         __syncthreads();
-        fft_group(a, b, stw, N, t);
+        fft_group<R3>(a, b, stw, N, t);
         // conj of the transform: row 0 in .x, row 1 in -.y
         if (live && lay.quads) {
             // horizontal pairs (u, u+1) for u = -1 .. nu-1, two 8-byte stores each
@@ -309,16 +304,17 @@ __global__ void ramp_fft_kernel(GeomDev g, const float *__restrict__ src, float 
     }
 }
 
+template <bool R3>
 static cudaError_t launch_ramp_fft(const GeomDev &g, const float *src, float *dst, SinoLayout lay, bool transpose,
                                    const int *stop, cudaStream_t st)
 {
     const FftShape fs = fft_shape(g.fft_n);
     if (fs.smem > 48 * 1024) {
-        cudaError_t e = raise_dyn_smem(reinterpret_cast<const void *>(ramp_fft_kernel), fs.smem);
+        cudaError_t e = raise_dyn_smem(reinterpret_cast<const void *>(ramp_fft_kernel<R3>), fs.smem);
         if (e != cudaSuccess) return e;
     }
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ramp_fft_kernel, fs.threads, fs.smem) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ramp_fft_kernel<R3>, fs.threads, fs.smem) != cudaSuccess ||
         per_sm < 1) {
         cudaGetLastError();
         per_sm = 1;
@@ -327,14 +323,15 @@ static cudaError_t launch_ramp_fft(const GeomDev &g, const float *src, float *ds
     const int want = (npairs + fs.groups - 1) / fs.groups;
     const unsigned blocks = unsigned(std::max(1, std::min(want, num_sms() * per_sm)));
     ProfScope prof(PK_RAMP, st);
-    ramp_fft_kernel<<<blocks, fs.threads, fs.smem, st>>>(g, src, dst, lay, transpose ? 1 : 0, stop);
+    ramp_fft_kernel<R3><<<blocks, fs.threads, fs.smem, st>>>(g, src, dst, lay, transpose ? 1 : 0, stop);
     return cudaGetLastError();
 }
 
 cudaError_t launch_ramp(const GeomDev &g, const float *src, float *dst, SinoLayout lay, bool transpose,
                         const int *stop, cudaStream_t st)
 {
-    return launch_ramp_fft(g, src, dst, lay, transpose, stop, st);
+    return g.fft_n % 3 == 0 ? launch_ramp_fft<true>(g, src, dst, lay, transpose, stop, st)
+                            : launch_ramp_fft<false>(g, src, dst, lay, transpose, stop, st);
 }
 
 // ---------------------------------------------------------------------------
