@@ -326,11 +326,13 @@ __device__ __forceinline__ float row_lerp(const float *p, float wb)
 // stay in its one slice.  DIRECT: small images are read where they are (Xc is
 // the volume; cells off the grid read as zero, bf16 storage rounds what it
 // reads), without copies.
-// Projections with their copies, two interpolated rows a plane and one warp a
-// ray against this: 64 x 64 with 90 views 18.7 -> 10.0 us, 512 x 512 with 720
-// views 325 -> 190 us, 1000 x 100 with 90 views 129 -> 41 us (bf16 84 -> 45 us).
+// Registers for 4 blocks an SM: ptxas then keeps a batch's loads together (512 x
+// 512, 720 views 190 us without a bound, 162 us for 2 to 4 blocks, 175 for 6).
+// Calls with copies, two interpolated rows a plane and one warp a ray against
+// this: 512 x 512 with 720 views 325 -> 162 us, 1024 x 1024 with 360 views 622 ->
+// 310 us, 1000 x 100 with 90 views 129 -> 28 us (bf16 84 -> 29 us).
 template <bool FLAT, bool BF, bool DIRECT>
-__global__ void __launch_bounds__(256) joseph_A_row_kernel(GeomDev g, const float *__restrict__ Xc,
+__global__ void __launch_bounds__(256, 4) joseph_A_row_kernel(GeomDev g, const float *__restrict__ Xc,
                                                            const float *__restrict__ Yc, float *__restrict__ y,
                                                            SinoLayout lay, int split,
                                                            const int *__restrict__ stop)
@@ -577,18 +579,27 @@ __global__ void __launch_bounds__(A_BLOCK, kAMinBlocks)
     }
 }
 
+// Warps that share the planes of a one-row detector's rays: as many as keep the
+// grid within 32 warps an SM, and on to 128, about four waves, while a share is 32
+// planes or more: rays leave the image after different numbers of planes, and more
+// and shorter shares even out (9 x 1000 pixels, 90 views: 114 us with 32 warps an
+// SM, 36 us with 96; 512 x 512, 360 views 99 us with 96, 90 us with 128; the
+// transpose of 1024 x 1024, 90 views 320 us with 32, 232 us with 96).
+static int row_split(const GeomDev &g, int limit)
+{
+    const size_t warps = size_t((g.nu + 31) / 32) * g.n_views, sms = num_sms();
+    int split = 1;
+    while (split < limit && (warps * split * 2 <= sms * 32 ||
+                             (warps * split * 2 <= sms * 128 && std::max(g.nx, g.ny) >= split * 2 * 32)))
+        split *= 2;
+    return split;
+}
+
 template <bool FLAT, bool BF, bool DIRECT>
 static void launch_joseph_A_row(const GeomDev &g, const float *Xc, const float *Yc, float *y, SinoLayout lay,
                                 const int *stop, cudaStream_t st)
 {
-    // warps a ray: as many (up to 8) as keep the grid within 96 warps an SM, about two
-    // waves; rays leave the image after different numbers of planes, so more and
-    // shorter shares even out (32 warps an SM: 9 x 1000 pixels, 90 views 114 us
-    // against 36 us, 300 x 300, 180 views 50 against 31 us)
-    const int tiles = (g.nu + 31) / 32;
-    const size_t most = size_t(num_sms()) * 96;
-    int split = 1;
-    while (split < 8 && size_t(tiles) * g.n_views * split * 2 <= most) split *= 2;
+    const int tiles = (g.nu + 31) / 32, split = row_split(g, 8);
     const dim3 block(32, 8), grid((tiles * split + 7) / 8, 1, g.n_views);
     joseph_A_row_kernel<FLAT, BF, DIRECT><<<grid, block, 0, st>>>(g, Xc, Yc, y, lay, split, stop);
 }
