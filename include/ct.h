@@ -162,7 +162,9 @@ CT_API ct_status ct_adjoint_At(const ct_geom *geom, const float *y_dev, float *x
 
 /* y = B^T x: exact transpose of ct_backproject_B for b_kind CT_B_UN
  * (voxel splatting with the same bilinear weights) and CT_B_FBP
- * (F^T B_un^T); CT_B_AT gives A x.  FP32 atomics.  x: n, y: m (overwritten). */
+ * (F^T B_un^T); CT_B_AT gives A x.  FP32 atomics.  x: n, y: m (overwritten).
+ * CT_B_UN needs no scratch memory: where its accumulators cannot be had it
+ * adds straight into y. */
 CT_API ct_status ct_adjoint_Bt(const ct_geom *geom, const float *x_dev, float *y_dev, int b_kind,
                         void *stream);
 

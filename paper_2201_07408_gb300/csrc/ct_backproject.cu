@@ -694,7 +694,7 @@ static int small_split(const GeomDev &g, int zc)
 {
     const size_t warps = size_t((g.nx + 31) / 32) * g.ny * ((g.nz + zc - 1) / zc), most = size_t(num_sms()) * 32;
     int split = 1;
-    while (split < 8 && warps * split * 2 <= most) split *= 2;
+    while (split < 8 && split * 2 <= g.n_views && warps * split * 2 <= most) split *= 2;
     return split;
 }
 
@@ -759,23 +759,46 @@ cudaError_t launch_voxel_B(const GeomDev &g, const float *ypad, float *x, const 
 }
 
 // ---------------------------------------------------------------------------
-// y = B_un^T x: voxel splatting with the same weights.  FP32 reductions into an
-// accumulator with a border column on both sides, Y[view][v][u + 1], kept twice
-// so that the two pixels of a row go as one request (add_pair); a last pass adds
-// the two up.
+// y = B_un^T x: voxel splatting with the same weights, by FP32 reductions: a
+// request a pixel straight into y, or (PAIRS) into an accumulator with a border
+// column on both sides, Y[view][v][u + 1], kept twice so that the two pixels of a
+// row go as one request (add_pair); a last pass adds the two up.
 // ---------------------------------------------------------------------------
 static size_t bt_floats(const GeomDev &g) { return pair_acc_floats(size_t(g.n_views) * g.nv * (g.nu + 2)); }
-size_t bt_scratch_floats(const GeomDev &g) { return 2 * bt_floats(g); }
+size_t bt_scratch_floats(const GeomDev &g, Scatter how) { return how == SCATTER_PAIRS ? 2 * bt_floats(g) : 0; }
 
-// the pair (u0, u0 + 1), u0 in [-1, nu - 1], of detector row v; rows off the detector are not entries of B
+// Pairs halve the requests, for a pass that zeroes the accumulators and one that
+// adds them up.  Samples (voxels times views) at which they begin to win, straight
+// into y and in pairs: about 1.2e6 for the slab kernel (16^3, 30 views 9 and 15
+// us; 50 x 56 x 51, 57 views 55 and 49 us; 256^3, 358 views 13.4 and 12.2 ms), 5e5
+// for thin slabs, and 6e4 in 2D (64 x 64, 10 views 12 and 15 us; 136 x 309, 2 views
+// 25 and 19 us; 1024 x 1024, 512 views 2.1 and 1.5 ms), but no image of under 2000
+// pixels (16 x 16, 600 views 14 and 18 us) and no single view of a small one (512
+// x 512 17 and 18 us).
+Scatter bt_scatter(const GeomDev &g)
+{
+    const double voxels = double(g.nx) * g.ny * g.nz, samples = voxels * g.n_views;
+    const double least = g.nz >= B_ZC ? 1.2e6 : g.nz > 1 ? 5e5 : 6e4;
+    return samples >= least && (g.n_views > 1 || samples >= 1e6) && voxels >= 2000.0 ? SCATTER_PAIRS : SCATTER_DIRECT;
+}
+
+// the pair (u0, u0 + 1), u0 in [-1, nu - 1], of detector row v; what lies off the detector is not an entry of B
+template <bool PAIRS>
 __device__ __forceinline__ void splat(const GeomDev &g, float *acc, size_t odd, int s, int u0, int v, float lo,
                                       float hi)
 {
     if (v < 0 || v >= g.nv) return;
-    add_pair(acc, odd, (size_t(s) * g.nv + v) * (g.nu + 2) + u0 + 1, lo, hi);
+    if (PAIRS) {
+        add_pair(acc, odd, (size_t(s) * g.nv + v) * (g.nu + 2) + u0 + 1, lo, hi);
+    } else {
+        float *p = acc + ((size_t(s) * g.nv + v) * g.nu + u0);
+        if (u0 >= 0 && lo != 0.0f) atomicAdd(p, lo);
+        if (u0 + 1 < g.nu && hi != 0.0f) atomicAdd(p + 1, hi);
+    }
 }
 
 // `split` blocks share the views of a voxel
+template <bool PAIRS>
 __global__ void __launch_bounds__(B_BX *B_BY) voxel_Bt_kernel(GeomDev g, const float *__restrict__ x,
                                                               float *__restrict__ acc, size_t odd, int split,
                                                               const int *__restrict__ stop)
@@ -800,8 +823,8 @@ __global__ void __launch_bounds__(B_BX *B_BY) voxel_Bt_kernel(GeomDev g, const f
         if (v0f < -1.0f || v0f > float(g.nv - 1)) continue;
         const int v0 = int(v0f), u0 = c.col - PAD_U;
         const float lo = xv * (1.0f - wv), hi = xv * wv;
-        if (lo != 0.0f) splat(g, acc, odd, s, u0, v0, lo * c.a0, lo * c.a1);
-        if (hi != 0.0f) splat(g, acc, odd, s, u0, v0 + 1, hi * c.a0, hi * c.a1);
+        if (lo != 0.0f) splat<PAIRS>(g, acc, odd, s, u0, v0, lo * c.a0, lo * c.a1);
+        if (hi != 0.0f) splat<PAIRS>(g, acc, odd, s, u0, v0 + 1, hi * c.a0, hi * c.a1);
     }
 }
 
@@ -816,10 +839,9 @@ __global__ void __launch_bounds__(B_BX *B_BY) voxel_Bt_kernel(GeomDev g, const f
 // copy of the reductions.  One launch per lane orientation, in 256-thread
 // blocks (MINB resident per SM): XL takes the views whose lanes run along x
 // on 32 x 8 column tiles, !XL those along y on 8 x 32 tiles.  `split` blocks
-// share a run's views (small volumes).  Dense data, 256^3: 16.5 ms with a
-// request a pixel, 12.2 ms with one a pair (runs of 16 slices 11.7 ms, but 10 %
-// slower at 128^3: 0.66 -> 0.73 ms); 44^3 0.129 -> 0.043 ms.
-template <int ZC, bool XL, int MINB>
+// share a run's views (small volumes).  Pairs in runs of 16
+// slices: 256^3 11.7 ms against 12.2, but 128^3 0.73 against 0.66 ms.
+template <int ZC, bool XL, int MINB, bool PAIRS>
 __global__ void __launch_bounds__(256, MINB) voxel_Bt_slab_kernel(GeomDev g, const float *__restrict__ x,
                                                                   float *__restrict__ acc, size_t odd, int split,
                                                                   const int *__restrict__ stop)
@@ -854,7 +876,7 @@ __global__ void __launch_bounds__(256, MINB) voxel_Bt_slab_kernel(GeomDev g, con
         const int u0 = c.col - PAD_U;
         auto flush = [&](int v, float r) {
             if (r == 0.0f) return;
-            splat(g, acc, odd, s, u0, v, r * c.a0, r * c.a1);
+            splat<PAIRS>(g, acc, odd, s, u0, v, r * c.a0, r * c.a1);
         };
         int vc = 0;
         float acc_lo = 0.0f, acc_hi = 0.0f;
@@ -897,47 +919,57 @@ __global__ void __launch_bounds__(256) unpair_sino_kernel(const float *__restric
         }
 }
 
-template <int ZC, int MINB>
+template <int ZC, int MINB, bool PAIRS>
 static cudaError_t launch_voxel_Bt_slab(const GeomDev &g, const float *x, float *acc, size_t odd, const int *stop,
                                         cudaStream_t st)
 {
+    auto *along_x = voxel_Bt_slab_kernel<ZC, true, MINB, PAIRS>, *along_y = voxel_Bt_slab_kernel<ZC, false, MINB, PAIRS>;
     const size_t smem = size_t(g.n_views) * 2 * sizeof(float4);
-    cudaError_t e = raise_dyn_smem(reinterpret_cast<const void *>(voxel_Bt_slab_kernel<ZC, true, MINB>), smem);
-    if (e == cudaSuccess)
-        e = raise_dyn_smem(reinterpret_cast<const void *>(voxel_Bt_slab_kernel<ZC, false, MINB>), smem);
+    cudaError_t e = raise_dyn_smem(reinterpret_cast<const void *>(along_x), smem);
+    if (e == cudaSuccess) e = raise_dyn_smem(reinterpret_cast<const void *>(along_y), smem);
     if (e != cudaSuccess) return e;
     const int runs = (g.nz + ZC - 1) / ZC;
     dim3 block(32, 8);
     dim3 gx((g.nx + 31) / 32, (g.ny + 7) / 8, runs);
     dim3 gy((g.nx + 7) / 8, (g.ny + 31) / 32, runs);
     // small volumes: blocks share a run's views until the grid has 4 blocks an SM
+    const size_t most = size_t(num_sms()) * 4;
     int split = 1;
-    while (split < 16 && size_t(gx.x) * gx.y * runs * split * 2 <= size_t(num_sms()) * 4) split *= 2;
+    while (split < 16 && size_t(gx.x) * gx.y * runs * split * 2 <= most) split *= 2;
     gx.z *= split;
     gy.z *= split;
-    voxel_Bt_slab_kernel<ZC, true, MINB><<<gx, block, smem, st>>>(g, x, acc, odd, split, stop);
-    voxel_Bt_slab_kernel<ZC, false, MINB><<<gy, block, smem, st>>>(g, x, acc, odd, split, stop);
+    along_x<<<gx, block, smem, st>>>(g, x, acc, odd, split, stop);
+    along_y<<<gy, block, smem, st>>>(g, x, acc, odd, split, stop);
     return cudaGetLastError();
 }
 
-cudaError_t launch_voxel_Bt(const GeomDev &g, const float *x, float *y, float *acc, const int *stop,
+template <bool PAIRS>
+static cudaError_t launch_voxel_Bt_t(const GeomDev &g, const float *x, float *acc, size_t odd, const int *stop,
+                                     cudaStream_t st)
+{
+    if (g.nz >= B_ZC) return launch_voxel_Bt_slab<B_ZC, 4, PAIRS>(g, x, acc, odd, stop, st);
+    // 2D, or a slab thinner than a z run: one voxel per thread
+    dim3 block(B_BX, B_BY);
+    dim3 grid((g.nx + B_BX - 1) / B_BX, (g.ny + B_BY - 1) / B_BY, g.nz);
+    const size_t most = size_t(num_sms()) * 8;
+    int split = 1;
+    while (split < 32 && split * 2 <= g.n_views && size_t(grid.x) * grid.y * g.nz * split * 2 <= most) split *= 2;
+    grid.z *= split;
+    voxel_Bt_kernel<PAIRS><<<grid, block, 0, st>>>(g, x, acc, odd, split, stop);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_voxel_Bt(const GeomDev &g, Scatter how, const float *x, float *y, float *acc, const int *stop,
                             cudaStream_t st)
 {
     ProfScope prof(PK_VOXEL_BT, st);
     const size_t odd = bt_floats(g), rows = size_t(g.n_views) * g.nv;
-    cudaError_t e = cudaMemsetAsync(acc, 0, 2 * odd * sizeof(float), st);
-    if (e != cudaSuccess) return e;
-    if (g.nz < B_ZC) {   // 2D, or a slab thinner than a z run: one voxel per thread
-        dim3 block(B_BX, B_BY);
-        dim3 grid((g.nx + B_BX - 1) / B_BX, (g.ny + B_BY - 1) / B_BY, g.nz);
-        int split = 1;
-        while (split < 32 && size_t(grid.x) * grid.y * g.nz * split * 2 <= size_t(num_sms()) * 8) split *= 2;
-        grid.z *= split;
-        voxel_Bt_kernel<<<grid, block, 0, st>>>(g, x, acc, odd, split, stop);
-        e = cudaGetLastError();
-    } else {
-        e = launch_voxel_Bt_slab<B_ZC, 4>(g, x, acc, odd, stop, st);
+    if (how != SCATTER_PAIRS) {
+        cudaError_t e = cudaMemsetAsync(y, 0, rows * g.nu * sizeof(float), st);
+        return e == cudaSuccess ? launch_voxel_Bt_t<false>(g, x, y, 0, stop, st) : e;
     }
+    cudaError_t e = cudaMemsetAsync(acc, 0, 2 * odd * sizeof(float), st);
+    if (e == cudaSuccess) e = launch_voxel_Bt_t<true>(g, x, acc, odd, stop, st);
     if (e != cudaSuccess) return e;
     const unsigned blocks = unsigned(std::min<size_t>((rows + 7) / 8, size_t(num_sms()) * 16));
     unpair_sino_kernel<<<blocks, dim3(32, 8), 0, st>>>(acc, odd, g.nu, rows, y, stop);
@@ -998,13 +1030,18 @@ extern "C" ct_status ct_adjoint_Bt(const ct_geom *geom, const float *x_dev, floa
         return set_error(CT_EINVAL, "ct_adjoint_Bt: unknown b_kind %d", b_kind);
     const GeomDev &g = geom->g;
     const bool fbp = b_kind == CT_B_FBP;
-    const size_t acc_bytes = Arena::align(bt_scratch_floats(g) * sizeof(float));
+    const size_t dst_bytes = fbp ? Arena::align(geom->m * sizeof(float)) : 0;
+    Scatter how = bt_scatter(g);
     Arena ar;
-    ct_status rc = arena_open(ar, acc_bytes + (fbp ? Arena::align(geom->m * sizeof(float)) : 0), nullptr, 0, st);
+    ct_status rc = arena_open(ar, Arena::align(bt_scratch_floats(g, how) * sizeof(float)) + dst_bytes, nullptr, 0, st);
+    if (rc == CT_ENOMEM && how != SCATTER_DIRECT) {   // short of memory: the way that takes none
+        how = SCATTER_DIRECT;
+        rc = arena_open(ar, dst_bytes, nullptr, 0, st);
+    }
     if (rc != CT_OK) return rc;
-    float *acc = ar.take<float>(bt_scratch_floats(g));
+    float *acc = ar.take<float>(bt_scratch_floats(g, how));
     float *dst = fbp ? ar.take<float>(geom->m) : y_dev;
-    cudaError_t e = launch_voxel_Bt(g, x_dev, dst, acc, nullptr, st);
+    cudaError_t e = launch_voxel_Bt(g, how, x_dev, dst, acc, nullptr, st);
     if (e == cudaSuccess && fbp) e = launch_ramp(g, dst, y_dev, plain_layout(g), true, nullptr, st);
     arena_close(ar);
     if (e != cudaSuccess) return cuda_error(e, "ct_adjoint_Bt launch");

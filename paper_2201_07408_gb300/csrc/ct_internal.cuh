@@ -290,13 +290,20 @@ cudaError_t launch_plane_copies(const GeomDev &g, const float *vol, const double
 // y = A x from the plane copies, written in `lay`.
 cudaError_t launch_project_A(const GeomDev &g, const float *Xc, const float *Yc, float *y,
                             SinoLayout lay, const int *stop, cudaStream_t st);
-// x = A^T y (overwritten); y in plain layout.  acc: at_scratch_floats(g) floats,
-// 256-byte aligned, contents overwritten.
-size_t at_scratch_floats(const GeomDev &g);
-cudaError_t launch_project_At(const GeomDev &g, const float *y, float *x, float *acc, const int *stop,
+// How a transpose (A^T, B_un^T) scatters: straight into its output, into
+// accumulators, or into accumulators kept twice (add_pair).
+enum Scatter { SCATTER_DIRECT, SCATTER_SINGLE, SCATTER_PAIRS };
+// x = A^T y (overwritten); y in plain layout.  acc: at_scratch_floats(g, how)
+// floats, 256-byte aligned, contents overwritten.  at_scatter: the fastest way
+// on this geometry; at_scatter_lean: the one that takes the least memory.
+Scatter at_scatter(const GeomDev &g);
+Scatter at_scatter_lean(const GeomDev &g);
+size_t at_scratch_floats(const GeomDev &g, Scatter how);
+cudaError_t launch_project_At(const GeomDev &g, Scatter how, const float *y, float *x, float *acc, const int *stop,
                              cudaStream_t st);
 // the line-intersection projector and its transpose (ct_siddon.cu); the
-// transpose adds to the zeroed accumulators Xa, Ya, laid out like the copies
+// transpose adds to the zeroed accumulators Xa, Ya, laid out like the copies, or
+// (Ya null) to the zeroed volume Xa
 cudaError_t launch_siddon_A(const GeomDev &g, const float *Xc, const float *Yc, float *y, SinoLayout lay,
                             const int *stop, cudaStream_t st);
 cudaError_t launch_siddon_At(const GeomDev &g, const float *y, float *Xa, float *Ya, const int *stop,
@@ -318,14 +325,16 @@ enum QuadForm { QUAD_ROWDIFF, QUAD_CORNERS };
 // launch_ramp, QUAD_CORNERS after a projector wrote it with store_sino.
 cudaError_t launch_voxel_B(const GeomDev &g, const float *ypad, float *x, const int *stop,
                            cudaStream_t st, QuadForm form);
-// y = B_un^T x (y plain).  acc: bt_scratch_floats(g) floats, 256-byte aligned,
-// contents overwritten.
-size_t bt_scratch_floats(const GeomDev &g);
-cudaError_t launch_voxel_Bt(const GeomDev &g, const float *x, float *y, float *acc, const int *stop,
+// y = B_un^T x (y plain).  acc: bt_scratch_floats(g, how) floats, 256-byte
+// aligned, contents overwritten (none for SCATTER_DIRECT, the lean way).
+Scatter bt_scatter(const GeomDev &g);
+size_t bt_scratch_floats(const GeomDev &g, Scatter how);
+cudaError_t launch_voxel_Bt(const GeomDev &g, Scatter how, const float *x, float *y, float *acc, const int *stop,
                             cudaStream_t st);
 
-// The scatters (A^T, B_un^T) are bound by the rate of reduction requests, about
-// 2.8e10 warp requests a second whatever each carries.  Their contributions
+// While what they add to stays in L2, the scatters (A^T, B_un^T) are bound by the
+// rate of reduction requests, about 2.8e10 warp requests a second whatever each
+// carries.  Their contributions
 // come in pairs of neighbouring elements, so an accumulator is kept twice, the
 // second copy shifted by one element: every pair is 8-byte aligned in one of
 // them and goes as one request.  Element e is acc[e] + acc[odd + e + 1].

@@ -965,7 +965,7 @@ static void take_op_bufs(Arena &ar, const GeomDev &g, OpBufs &b, bool need_t, bo
     b.Yc = ar.take<float>(size_t(g.nzp) * g.ny * g.pitchY);
     b.ypad = ar.take<float>(padded_sino_floats(g));
     b.t = need_t ? ar.take<float>(size_t(g.n_views) * g.nv * g.nu) : nullptr;
-    b.acc = need_acc ? ar.take<float>(at_scratch_floats(g)) : nullptr;
+    b.acc = need_acc ? ar.take<float>(at_scratch_floats(g, at_scatter(g))) : nullptr;
 }
 
 // out_vol = B sino.  `sino` is a plain sinogram, scaled by (*scale) first when
@@ -991,7 +991,7 @@ static cudaError_t apply_B(const GeomDev &g, int b_kind, float *sino, const doub
         if (e == cudaSuccess) e = launch_voxel_B(g, b.ypad, out_vol, stop, st, QUAD_ROWDIFF);
         return e;
     }
-    return launch_project_At(g, sino, out_vol, b.acc, stop, st);   // exact transpose A^T
+    return launch_project_At(g, at_scatter(g), sino, out_vol, b.acc, stop, st);   // exact transpose A^T
 }
 
 static ct_status check_common(const ct_geom *geom, const float *b, int k, const float *x,
@@ -1546,8 +1546,8 @@ static void carve_vjp(Arena &ar, const GeomDev &g, int k, int b_kind, VjpWs &w)
     w.gm.V = ar.take<float>(w.gm.ldv * size_t(k + 1));
     w.t = ar.take<float>(m);
     w.tf = b_kind == CT_B_FBP ? ar.take<float>(m) : nullptr;
-    w.acc = ar.take<float>(at_scratch_floats(g));
-    w.bt_acc = ar.take<float>(bt_scratch_floats(g));
+    w.acc = ar.take<float>(at_scratch_floats(g, at_scatter(g)));
+    w.bt_acc = ar.take<float>(bt_scratch_floats(g, bt_scatter(g)));
     const size_t ld = size_t(k) + 1;
     w.gm.H = ar.take<double>(ld * k);
     w.gm.H2 = ar.take<double>(ld);
@@ -1584,7 +1584,7 @@ __global__ void scale_vec_kernel(float *__restrict__ v, size_t len, const double
 static cudaError_t apply_Bt(const GeomDev &g, int b_kind, const float *vol, float *t, float *tf, float *bt_acc,
                             float *out, const int *stop, cudaStream_t s)
 {
-    cudaError_t e = launch_voxel_Bt(g, vol, b_kind == CT_B_FBP ? t : out, bt_acc, stop, s);
+    cudaError_t e = launch_voxel_Bt(g, bt_scatter(g), vol, b_kind == CT_B_FBP ? t : out, bt_acc, stop, s);
     if (e == cudaSuccess && b_kind == CT_B_FBP) e = launch_ramp(g, t, out, plain_layout(g), true, stop, s);
     (void)tf;
     return e;
@@ -1626,7 +1626,7 @@ static ct_status bagmres_vjp(const ct_geom *geom, const float *gx, int k, float 
             e = cudaGetLastError();
         }
         if (e == cudaSuccess) e = apply_Bt(g, o.b_kind, vj, w.t, w.tf, w.bt_acc, sino, stop, s);
-        if (e == cudaSuccess) e = launch_project_At(g, sino, q, w.acc, stop, s);
+        if (e == cudaSuccess) e = launch_project_At(g, at_scatter(g), sino, q, w.acc, stop, s);
         if (e == cudaSuccess) e = arnoldi_orthogonalise(gm, q, j, k, n, o, s);
     }
     if (e == cudaSuccess) e = backsolve(gm.R, gm.g, gm.y, &gm.st->iters, k, s);

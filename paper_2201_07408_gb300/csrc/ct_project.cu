@@ -649,27 +649,53 @@ cudaError_t launch_project_A(const GeomDev &g, const float *Xc, const float *Yc,
 // projector reads one: contributions to the same row are summed in
 // registers and a row is flushed when the window moves past it.
 //
-// A flush adds to two neighbouring cells, b0 and b0 + 1, as one request to one
-// of an orientation's two accumulators (add_pair).  Samples on the zero border
+// A flush adds to two neighbouring cells, b0 and b0 + 1: as two requests, or
+// (PAIRS) as one to one of an orientation's two accumulators (add_pair; the
+// rule and both sides' times stand at at_scatter).  Samples on the zero border
 // add to the border or are skipped (they are zero entries of A); a last pass
-// adds the four accumulators up.  Dense data, 256^3: 13.9 ms with a request a
-// cell, 12.1 ms so (128^3 1.01 -> 0.63 ms); what binds then is the rate at which
-// L2 adds words, about 1.5e12 a second (32 and 48 rays a thread, 11.9 and 12.3
-// ms).  Small scans were bound by a warp's chain of planes: 44^3 0.121 -> 0.039
-// ms, 64 x 64 30 -> 19 us.
+// adds the accumulators up.  Small scans were bound by a warp's chain of planes,
+// which `p_split` warps share: 44^3 0.121 -> 0.039 ms, 64 x 64 30 -> 19 us.
 // ---------------------------------------------------------------------------
 static size_t at_floats(const GeomDev &g, bool x)
 {
     return pair_acc_floats(size_t(g.nzp) * (x ? size_t(g.nx) * g.pitchX : size_t(g.ny) * g.pitchY));
 }
 
-// Joseph's transpose keeps each accumulator twice, the line-intersection one's once
-size_t at_scratch_floats(const GeomDev &g)
+size_t at_scratch_floats(const GeomDev &g, Scatter how)
 {
-    return (g.siddon ? 1 : 2) * (at_floats(g, true) + at_floats(g, false));
+    return how == SCATTER_DIRECT ? 0 : (how == SCATTER_PAIRS ? 2 : 1) * (at_floats(g, true) + at_floats(g, false));
 }
 
-template <int VR, bool WINDOW, bool ZCLAMP>
+Scatter at_scatter_lean(const GeomDev &g) { return g.siddon ? SCATTER_DIRECT : SCATTER_SINGLE; }
+
+// What each way costs beside its scattered adds: zeroing the accumulators and
+// adding them up.  Measured (dense data; one way and the other):
+// - Pairs halve the requests and double what the adds touch.  While the four
+//   accumulators fit L2 (129 MB), they win: 128^3, 128 views 0.89 against 1.10 ms,
+//   192^3 3.4 against 4.0 ms.  Past it single accumulators do: 256^3, 358 views
+//   11.7 against 12.2 ms, 320^3 28 against 51 ms, 512^3, 64 views 25 against 40 ms.
+// - Nor do they win where few rays cross a voxel (100^3 with one view 31 against
+//   33 us), or on large one-row scans (1024 x 1024, 128 views or more, 1 % either
+//   way, but 10 views 47 against 52 us).
+// - The line-intersection transpose straight into the volume saves two launches
+//   (16^3 9 against 15 us; not where hundreds of rays cross each voxel: 21 x 46 x
+//   3, 180 views 43 against 29 us), wins where few rays cross a voxel of a tall
+//   volume (214 x 131 x 296, 3 views, 82 against 105 us), and where dozens of
+//   columns fall on a voxel (44^3, 1320 columns 18 against 21 ms).
+Scatter at_scatter(const GeomDev &g)
+{
+    const double planes = double(g.n_views) * g.nu * g.nv * std::max(g.nx, g.ny);   // of all rays
+    const double per_voxel = planes / (double(g.nx) * g.ny * g.nz);
+    if (g.siddon)
+        return (planes < 2.5e6 && per_voxel < 200.0) || (planes < 6e6 && per_voxel < 25.0) ||
+                       (per_voxel < 10.0 && g.nv < g.nz) || g.nu > 20 * std::max(g.nx, g.ny)
+                   ? SCATTER_DIRECT : SCATTER_SINGLE;
+    const double bytes = 4.0 * at_scratch_floats(g, SCATTER_PAIRS);
+    if (g.nv == 1) return bytes <= 50e6 ? SCATTER_PAIRS : SCATTER_SINGLE;
+    return bytes <= 128e6 && (per_voxel >= 10.0 || bytes <= 12e6) ? SCATTER_PAIRS : SCATTER_SINGLE;
+}
+
+template <int VR, bool WINDOW, bool ZCLAMP, bool PAIRS>
 __global__ void __launch_bounds__(A_BLOCK) joseph_At_kernel(GeomDev g, const float *__restrict__ y,
                                                             float *__restrict__ X, size_t x_odd,
                                                             float *__restrict__ Y, size_t y_odd, int v_tiles,
@@ -721,7 +747,13 @@ __global__ void __launch_bounds__(A_BLOCK) joseph_At_kernel(GeomDev g, const flo
         // adds a row's summed contribution r to cells b0, b0 + 1 of grid row z
         auto flush = [&](int z, float r) {
             if (r == 0.0f || z < 0 || z >= zmax) return;
-            add_pair(base, odd, row0 + unsigned(z) * zstride, r * (1.0f - wb), r * wb);
+            const unsigned e = row0 + unsigned(z) * zstride;
+            if (PAIRS) {
+                add_pair(base, odd, e, r * (1.0f - wb), r * wb);
+            } else {
+                if (b0 >= 0) atomicAdd(base + e, r * (1.0f - wb));
+                if (b0 + 1 < c.Nb) atomicAdd(base + e + 1, r * wb);
+            }
         };
         int zc = 0;
         float acc_lo = 0.0f, acc_hi = 0.0f;   // rows zc and zc + 1
@@ -786,38 +818,51 @@ __global__ void __launch_bounds__(256) unplane_kernel(GeomDev g, const float *__
     }
 }
 
-cudaError_t launch_project_At(const GeomDev &g, const float *y, float *x, float *acc, const int *stop,
-                             cudaStream_t st)
+template <bool PAIRS>
+static void launch_joseph_At(const GeomDev &g, const float *y, float *X, size_t x_odd, float *Y, size_t y_odd,
+                             const int *stop, cudaStream_t st)
 {
-    ProfScope prof(PK_JOSEPH_AT, st);
-    const size_t x_odd = at_floats(g, true), y_odd = at_floats(g, false);
-    float *X = acc, *Y = acc + (g.siddon ? 1 : 2) * x_odd;
-    cudaError_t e = cudaMemsetAsync(acc, 0, sizeof(float) * at_scratch_floats(g), st);
-    if (e != cudaSuccess) return e;
-    const dim3 ublock(32, 8), ugrid((g.nx + 31) / 32, (g.ny + 31) / 32, std::min(g.nz, 65535));
-    if (g.siddon) {
-        e = launch_siddon_At(g, y, X, Y, stop, st);
-        if (e != cudaSuccess) return e;
-        unplane_kernel<false><<<ugrid, ublock, 0, st>>>(g, X, x_odd, Y, y_odd, x, stop);
-        return cudaGetLastError();
-    }
     constexpr int WPB = A_BLOCK / 32;
     const int u_tiles = (g.nu + 31) / 32, v_tiles = g.nv == 1 ? 1 : (g.nv + A_VR - 1) / A_VR;
     // small scans: warps share a tile's planes until the grid has 32 warps an SM
+    const size_t most = size_t(num_sms()) * 32;
     int split = 1;
-    while (split < 16 && size_t(u_tiles) * v_tiles * g.n_views * split * 2 <= size_t(num_sms()) * 32) split *= 2;
+    while (split < 16 && size_t(u_tiles) * v_tiles * g.n_views * split * 2 <= most) split *= 2;
+    if (g.nv == 1) split = row_split(g, 16);
     const dim3 grid(u_tiles, (v_tiles * split + WPB - 1) / WPB, g.n_views);
     if (g.nv == 1)
-        joseph_At_kernel<1, false, true><<<grid, A_BLOCK, 0, st>>>(g, y, X, x_odd, Y, y_odd, v_tiles, split, stop);
+        joseph_At_kernel<1, false, true, PAIRS><<<grid, A_BLOCK, 0, st>>>(g, y, X, x_odd, Y, y_odd, v_tiles, split, stop);
     else if (g.a_window && g.a_zsafe)
-        joseph_At_kernel<A_VR, true, false><<<grid, A_BLOCK, 0, st>>>(g, y, X, x_odd, Y, y_odd, v_tiles, split, stop);
+        joseph_At_kernel<A_VR, true, false, PAIRS><<<grid, A_BLOCK, 0, st>>>(g, y, X, x_odd, Y, y_odd, v_tiles, split, stop);
     else if (g.a_window)
-        joseph_At_kernel<A_VR, true, true><<<grid, A_BLOCK, 0, st>>>(g, y, X, x_odd, Y, y_odd, v_tiles, split, stop);
+        joseph_At_kernel<A_VR, true, true, PAIRS><<<grid, A_BLOCK, 0, st>>>(g, y, X, x_odd, Y, y_odd, v_tiles, split, stop);
     else
-        joseph_At_kernel<A_VR, false, true><<<grid, A_BLOCK, 0, st>>>(g, y, X, x_odd, Y, y_odd, v_tiles, split, stop);
-    e = cudaGetLastError();
+        joseph_At_kernel<A_VR, false, true, PAIRS><<<grid, A_BLOCK, 0, st>>>(g, y, X, x_odd, Y, y_odd, v_tiles, split, stop);
+}
+
+cudaError_t launch_project_At(const GeomDev &g, Scatter how, const float *y, float *x, float *acc, const int *stop,
+                             cudaStream_t st)
+{
+    ProfScope prof(PK_JOSEPH_AT, st);
+    const bool direct = how == SCATTER_DIRECT, pairs = how == SCATTER_PAIRS;
+    const size_t x_odd = at_floats(g, true), y_odd = at_floats(g, false);
+    float *X = direct ? x : acc, *Y = direct ? nullptr : acc + (pairs ? 2 : 1) * x_odd;
+    const size_t zeroed = direct ? size_t(g.nx) * g.ny * g.nz : at_scratch_floats(g, how);
+    cudaError_t e = cudaMemsetAsync(X, 0, sizeof(float) * zeroed, st);
     if (e != cudaSuccess) return e;
-    unplane_kernel<true><<<ugrid, ublock, 0, st>>>(g, X, x_odd, Y, y_odd, x, stop);
+    if (g.siddon)
+        e = launch_siddon_At(g, y, X, Y, stop, st);
+    else if (pairs)
+        launch_joseph_At<true>(g, y, X, x_odd, Y, y_odd, stop, st);
+    else
+        launch_joseph_At<false>(g, y, X, x_odd, Y, y_odd, stop, st);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e != cudaSuccess || direct) return e;
+    const dim3 ublock(32, 8), ugrid((g.nx + 31) / 32, (g.ny + 31) / 32, std::min(g.nz, 65535));
+    if (pairs)
+        unplane_kernel<true><<<ugrid, ublock, 0, st>>>(g, X, x_odd, Y, y_odd, x, stop);
+    else
+        unplane_kernel<false><<<ugrid, ublock, 0, st>>>(g, X, x_odd, Y, y_odd, x, stop);
     return cudaGetLastError();
 }
 
@@ -874,10 +919,14 @@ extern "C" ct_status ct_adjoint_At(const ct_geom *geom, const float *y_dev, floa
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const GeomDev &g = geom->g;
     Arena ar;
-    const size_t floats = at_scratch_floats(g);
-    ct_status rc = arena_open(ar, Arena::align(floats * sizeof(float)), nullptr, 0, st);
+    Scatter how = at_scatter(g);
+    ct_status rc = arena_open(ar, Arena::align(at_scratch_floats(g, how) * sizeof(float)), nullptr, 0, st);
+    if (rc == CT_ENOMEM && how != at_scatter_lean(g)) {   // short of memory: the way that takes less
+        how = at_scatter_lean(g);
+        rc = arena_open(ar, Arena::align(at_scratch_floats(g, how) * sizeof(float)), nullptr, 0, st);
+    }
     if (rc != CT_OK) return rc;
-    cudaError_t e = launch_project_At(g, y_dev, x_dev, ar.take<float>(floats), nullptr, st);
+    cudaError_t e = launch_project_At(g, how, y_dev, x_dev, ar.take<float>(at_scratch_floats(g, how)), nullptr, st);
     arena_close(ar);
     if (e != cudaSuccess) return cuda_error(e, "ct_adjoint_At launch");
     return CT_OK;

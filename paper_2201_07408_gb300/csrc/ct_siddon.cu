@@ -21,7 +21,7 @@
 // round, so that the lanes of a warp, neighbouring rays at about the same place
 // along their axis, read neighbouring words.  The transpose adds with FP32
 // atomics into two accumulators laid out the same way, and a last pass adds
-// those up.  With one layout for all rays (x fastest), rays along x touched a
+// those up, or (SCATTER_DIRECT) straight into the volume.  With one layout for all rays (x fastest), rays along x touched a
 // line a lane: A_S^T on dense data 1.33 -> 1.00 ms at 128^3 and 26.7 -> 20.0 ms
 // at 256^3, A_S 0.64 -> 0.61 and 12.6 -> 12.2 ms.  A walk of a detector column's
 // rays together (they share their line in the x-y plane; z fastest, lanes along
@@ -181,6 +181,8 @@ __global__ void __launch_bounds__(256) siddon_A_kernel(GeomDev g, const float *_
     store_sino(y, lay, s, iv, iu, acc * g.vox);
 }
 
+// DIRECT: into the volume Xa itself
+template <bool DIRECT>
 __global__ void __launch_bounds__(256) siddon_At_kernel(GeomDev g, const float *__restrict__ y,
                                                        float *__restrict__ Xa, float *__restrict__ Ya,
                                                        const int *__restrict__ stop)
@@ -198,7 +200,7 @@ __global__ void __launch_bounds__(256) siddon_At_kernel(GeomDev g, const float *
     if (!ray_walk(g, s, iv, iu, w)) return;
     // lengths come in voxel units: the ray's value carries the voxel size
     const float yv = yr * g.vox;
-    const RayLayout l = ray_layout(g, w);
+    const RayLayout l = DIRECT ? RayLayout{true, 0, 1, g.nx, g.nx * g.ny} : ray_layout(g, w);
     float *__restrict__ acc = l.xdom ? Xa : Ya;
     walk(g, w, l, [&](int e, float len) {
         if (len > 0.0f) atomicAdd(acc + e, yv * len);
@@ -224,7 +226,10 @@ cudaError_t launch_siddon_At(const GeomDev &g, const float *y, float *Xa, float 
 {
     const long long m = (long long)g.nu * g.nv * g.n_views;
     const unsigned blocks = unsigned((m + 255) / 256);
-    siddon_At_kernel<<<blocks, 256, 0, st>>>(g, y, Xa, Ya, stop);
+    if (Ya)
+        siddon_At_kernel<false><<<blocks, 256, 0, st>>>(g, y, Xa, Ya, stop);
+    else
+        siddon_At_kernel<true><<<blocks, 256, 0, st>>>(g, y, Xa, Ya, stop);
     return cudaGetLastError();
 }
 
