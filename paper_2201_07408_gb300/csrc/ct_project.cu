@@ -473,10 +473,14 @@ constexpr unsigned FLOOR_MAGIC_BITS = 0x4b400000u;
 // 256^3 4.32 ms (bf16 copies 4.41 ms); unrolled by 2, 4.38 ms (4.57 ms); 5
 // blocks unrolled by 2, 4.42 ms; 6 and 8 blocks, 4.80 and 5.51 ms (ptxas then
 // keeps fewer row loads in flight); 8 rays a thread, 4.65-4.74 ms.  The plain
-// walk over a two-row window took 5.04 ms (bf16 5.41 ms).  Left after it:
+// walk over a two-row window took 5.04 ms (bf16 5.41 ms).  On bf16 copies with the
+// clamp (a detector taller than the slices) 4 planes at a time need more registers
+// than there are: 74 x 143 x 24, 21 views 93 us against 83 by 3 (plain walk 82), 31 x
+// 68 x 42, 18 views 52 against 45 (47); by 2, 5 % slower on few views.  Left after it:
 // 12.1 instructions a sample (16.8 before), the FMA pipe 53 % and issue 56 %
 // busy, the rest latency of the row loads (a third of them miss L1).
 constexpr int kAPlaneUnroll = 4;
+constexpr int kAPlaneUnrollClampedBF = 3;
 constexpr int kAMinBlocks = 4;
 
 template <int VR, bool WINDOW, bool ZCLAMP, bool BF>
@@ -504,7 +508,7 @@ __global__ void __launch_bounds__(A_BLOCK, kAMinBlocks)
     for (int i = 0; i < VR / 2; ++i) acc[i] = pack2(0.0f, 0.0f);
     const f32x2 magic = pack2(FLOOR_MAGIC, FLOOR_MAGIC);
 
-#pragma unroll kAPlaneUnroll
+#pragma unroll (BF && ZCLAMP ? kAPlaneUnrollClampedBF : kAPlaneUnroll)
     for (int p = c.p0; p <= c.p1; ++p) {
         const float pm = float(p) - c.ca;
         const float fb = fmaf(pm, c.gb, c.fbc);
