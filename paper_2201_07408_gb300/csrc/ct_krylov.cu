@@ -470,10 +470,28 @@ static cudaError_t mgs_pass_t(float *q, const TB *vprev, const double *hprev, co
                               const int *stop, const int *skip, cudaStream_t st)
 {
     constexpr size_t G = 16 / sizeof(TB);   // elements of a 16-byte group of the basis
-    const int vec = (len % G == 0) && (reinterpret_cast<uintptr_t>(q) % 16 == 0) &&
+    // in groups where the vectors are aligned (a solve's always are, whatever their length); the elements past
+    // the last group, and vectors that are not aligned, one by one
+    const int vec = (reinterpret_cast<uintptr_t>(q) % 16 == 0) &&
                     (!vprev || reinterpret_cast<uintptr_t>(vprev) % 16 == 0) &&
                     (!vcur || reinterpret_cast<uintptr_t>(vcur) % 16 == 0);
     ProfScope prof(PK_MGS, st);
+    // past one block, single elements take all the threads that are resident at once (a sweep of 16.8 M elements, j =
+    // 4: 511 us with 4 blocks an SM, 471 so; 100001 elements 61 us with 16 elements a thread, 45 so)
+    if (!vec && len > 16 * SWEEP_NT) {
+        int per_sm = 8;
+        if (len > size_t(num_sms()) * 8 * RED_BLOCK * 4 &&
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mgs_pass_kernel<MODE, TB, RED_BLOCK>, RED_BLOCK, 0) !=
+                cudaSuccess) {
+            cudaGetLastError();
+            per_sm = 4;
+        }
+        const size_t most = size_t(num_sms()) * std::min(std::max(per_sm, 1), 8);
+        const unsigned blocks = unsigned(std::max<size_t>(1, std::min((len / 4 + RED_BLOCK - 1) / RED_BLOCK, most)));
+        mgs_pass_kernel<MODE, TB, RED_BLOCK><<<blocks, RED_BLOCK, 0, st>>>(
+            q, vprev, hprev, vcur, len, vec, partials, counter, out_dot, out_sumsq, stop, skip);
+        return cudaGetLastError();
+    }
     if (len <= sweep_max()) {
         mgs_pass_kernel<MODE, TB, SWEEP_NT><<<sweep_blocks(len), SWEEP_NT, 0, st>>>(
             q, vprev, hprev, vcur, len, vec, partials, counter, out_dot, out_sumsq, stop, skip);
