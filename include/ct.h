@@ -194,9 +194,8 @@ CT_API ct_status ct_bagmres_solve(const ct_geom *geom, const float *b_dev, int k
 /* ct_bagmres_solve with the data and the image in HOST memory: b_host (m
  * floats) is copied to the device, the solve runs as ct_bagmres_solve, and
  * x_k is copied back into x_out_host (n floats) before the call returns.
- * The two device vectors are taken from the stream-ordered allocator
- * (cudaMallocAsync) on `stream` and freed before return; the workspace is
- * as for ct_bagmres_solve.  Page-locked host buffers give asynchronous
+ * The two device vectors are scratch memory (see above), freed before
+ * return; the workspace is as for ct_bagmres_solve.  Page-locked host buffers give asynchronous
  * copies; pageable ones work too.  Synchronous: on return x_out_host and
  * resid_hist hold the result.  Returns CT_ENOMEM when the device vectors
  * cannot be allocated; other codes as ct_bagmres_solve. */
@@ -228,9 +227,9 @@ CT_API ct_status ct_bagmres_solve_err(const ct_geom *geom, const float *b_dev, i
  *               -1 after the last iteration done.  May be NULL.
  *   iters_done: total iterations over all cycles.
  * opts->tol stops a cycle at tol times that cycle's starting residual and
- * stops the solve when the residual reaches tol times resid[0].  Scratch
- * (the projector's copies, two sinograms and one volume) comes from the
- * stream-ordered allocator; the workspace, when given, is as for
+ * stops the solve when the residual reaches tol times resid[0].  The
+ * projector's copies, two sinograms and one volume are scratch memory (see
+ * above); the workspace, when given, is as for
  * ct_bagmres_solve with k = m.  Synchronous.  Return codes as
  * ct_bagmres_solve; CT_EINVAL for cycles < 1. */
 CT_API ct_status ct_bagmres_restarted(const ct_geom *geom, const float *b_dev, int m, int cycles,

@@ -2008,8 +2008,8 @@ ct_status ct_bagmres_solve_host(const ct_geom *geom, const float *b_host, int k,
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const size_t mb = geom->m * sizeof(float), nb = geom->n * sizeof(float);
     void *bd = nullptr, *xd = nullptr;
-    cudaError_t e = cudaMallocAsync(&bd, mb, s);
-    if (e == cudaSuccess) e = cudaMallocAsync(&xd, nb, s);
+    cudaError_t e = scratch_alloc(&bd, mb, s);
+    if (e == cudaSuccess) e = scratch_alloc(&xd, nb, s);
     if (e != cudaSuccess) {
         if (bd) cudaFreeAsync(bd, s);
         cudaGetLastError();
