@@ -169,7 +169,9 @@ CT_API ct_status ct_adjoint_Bt(const ct_geom *geom, const float *x_dev, float *y
                         void *stream);
 
 /* yf = F y (transpose = 0) or yf = F^T y (transpose = 1): the ramp filter
- * of B_FBP = B_un F (Sec. III) on its own.  y, yf: m floats, distinct. */
+ * of B_FBP = B_un F (Sec. III) on its own.  y, yf: m floats, distinct.
+ * Detector rows of at most 2048 columns: CT_EINVAL past that, here and from
+ * every call with b_kind CT_B_FBP. */
 CT_API ct_status ct_ramp_F(const ct_geom *geom, const float *y_dev, float *yf_dev, int transpose,
                     void *stream);
 

@@ -327,6 +327,13 @@ static cudaError_t launch_ramp_fft(const GeomDev &g, const float *src, float *ds
     return cudaGetLastError();
 }
 
+// A row's transform takes fft_n / 4 threads of one block.
+ct_status check_ramp(const GeomDev &g, const char *who)
+{
+    if (g.fft_n <= 4096) return CT_OK;
+    return set_error(CT_EINVAL, "%s: the ramp filter takes detector rows of at most 2048 columns (got %d)", who, g.nu);
+}
+
 cudaError_t launch_ramp(const GeomDev &g, const float *src, float *dst, SinoLayout lay, bool transpose,
                         const int *stop, cudaStream_t st)
 {
@@ -986,6 +993,8 @@ extern "C" ct_status ct_ramp_F(const ct_geom *geom, const float *y_dev, float *y
     NvtxRange call_range("ct_ramp_F");
     if (!geom || !y_dev || !yf_dev) return set_error(CT_EINVAL, "ct_ramp_F: NULL argument");
     if (y_dev == yf_dev) return set_error(CT_EINVAL, "ct_ramp_F: input and output must differ");
+    ct_status rc = check_ramp(geom->g, "ct_ramp_F");
+    if (rc != CT_OK) return rc;
     cudaError_t e = launch_ramp(geom->g, y_dev, yf_dev, plain_layout(geom->g), transpose != 0, nullptr,
                                 static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return cuda_error(e, "ct_ramp_F launch");
@@ -1002,8 +1011,10 @@ extern "C" ct_status ct_backproject_B(const ct_geom *geom, const float *y_dev, f
     if (b_kind != CT_B_UN && b_kind != CT_B_FBP)
         return set_error(CT_EINVAL, "ct_backproject_B: unknown b_kind %d", b_kind);
     const GeomDev &g = geom->g;
+    ct_status rc = b_kind == CT_B_FBP ? check_ramp(g, "ct_backproject_B") : CT_OK;
+    if (rc != CT_OK) return rc;
     Arena ar;
-    ct_status rc = arena_open(ar, padded_sino_bytes(g), nullptr, 0, st);
+    rc = arena_open(ar, padded_sino_bytes(g), nullptr, 0, st);
     if (rc != CT_OK) return rc;
     float *ypad = ar.take<float>(padded_sino_floats(g));
     cudaError_t e;
@@ -1031,9 +1042,11 @@ extern "C" ct_status ct_adjoint_Bt(const ct_geom *geom, const float *x_dev, floa
     const GeomDev &g = geom->g;
     const bool fbp = b_kind == CT_B_FBP;
     const size_t dst_bytes = fbp ? Arena::align(geom->m * sizeof(float)) : 0;
+    ct_status rc = fbp ? check_ramp(g, "ct_adjoint_Bt") : CT_OK;
+    if (rc != CT_OK) return rc;
     Scatter how = bt_scatter(g);
     Arena ar;
-    ct_status rc = arena_open(ar, Arena::align(bt_scratch_floats(g, how) * sizeof(float)) + dst_bytes, nullptr, 0, st);
+    rc = arena_open(ar, Arena::align(bt_scratch_floats(g, how) * sizeof(float)) + dst_bytes, nullptr, 0, st);
     if (rc == CT_ENOMEM && how != SCATTER_DIRECT) {   // short of memory: the way that takes none
         how = SCATTER_DIRECT;
         rc = arena_open(ar, dst_bytes, nullptr, 0, st);

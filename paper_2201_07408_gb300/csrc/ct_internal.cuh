@@ -315,6 +315,8 @@ cudaError_t launch_siddon_At(const GeomDev &g, const float *y, float *Xa, float 
 cudaError_t launch_pad_sino(const GeomDev &g, float *src, const double *scale,
                             bool normalize_inplace, float *dst, const int *stop,
                             cudaStream_t st);
+// CT_EINVAL with a message where a row is longer than the filter's transform takes.
+ct_status check_ramp(const GeomDev &g, const char *who);
 // dst = F src (or F^T src) from a plain sinogram into layout `lay`.
 cudaError_t launch_ramp(const GeomDev &g, const float *src, float *dst, SinoLayout lay,
                         bool transpose, const int *stop, cudaStream_t st);

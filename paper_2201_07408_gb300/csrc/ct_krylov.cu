@@ -1023,7 +1023,7 @@ static ct_status check_common(const ct_geom *geom, const float *b, int k, const 
     if (o->dot_mode != 0 && o->dot_mode != 1)
         return set_error(CT_EINVAL, "solver: dot_mode must be 0 or 1");
     if (!(o->tol >= 0.0)) return set_error(CT_EINVAL, "solver: tol must be >= 0");
-    return CT_OK;
+    return o->b_kind == CT_B_FBP ? check_ramp(geom->g, "solver") : CT_OK;
 }
 
 static size_t round_ld(size_t len) { return (len + 63) & ~size_t(63); }
@@ -1615,8 +1615,10 @@ static ct_status bagmres_vjp(const ct_geom *geom, const float *gx, int k, float 
         return set_error(CT_EINVAL, "ct_bagmres_vjp: b_kind must be CT_B_UN or CT_B_FBP");
     const GeomDev &g = geom->g;
     const size_t n = geom->n;
+    ct_status rc = o.b_kind == CT_B_FBP ? check_ramp(g, "ct_bagmres_vjp") : CT_OK;
+    if (rc != CT_OK) return rc;
     Arena ar;
-    ct_status rc = open_ws(ar, vjp_bytes(g, k, o.b_kind), o, s);
+    rc = open_ws(ar, vjp_bytes(g, k, o.b_kind), o, s);
     if (rc != CT_OK) return rc;
     VjpWs w;
     carve_vjp(ar, g, k, o.b_kind, w);
@@ -2128,6 +2130,7 @@ ct_status ct_bagmres_state_start(ct_gmres_state *state, const float *b_dev, void
     NvtxRange call_range("ct_bagmres_state_start");
     if (!state || !b_dev) return set_error(CT_EINVAL, "ct_bagmres_state_start: NULL argument");
     ct_status rc = state_check_device(state->geom, "ct_bagmres_state_start");
+    if (rc == CT_OK && state->o.b_kind == CT_B_FBP) rc = check_ramp(state->geom->g, "ct_bagmres_state_start");
     if (rc != CT_OK) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     cudaError_t e = ba_start(state->geom->g, state->w, b_dev, state->kmax, state->geom->n, state->o, s);
