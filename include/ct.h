@@ -411,6 +411,15 @@ CT_API ct_status ct_measure_gather_peak(int repeats, double *gbs_out, void *stre
  *   "oom"            every later request to the stream-ordered allocator is
  *                    refused as if it had failed (CT_ENOMEM); calls given a
  *                    workspace, and ct_project_A_noalloc, still run;
+ *   "sweep_stall:N"  in every later solve, the one-launch Gram-Schmidt sweep of
+ *                    iteration N >= 1, where it runs over several blocks, has
+ *                    one block keep its sum to itself and the others give up
+ *                    waiting after about a millisecond, so the solve returns
+ *                    CT_ETIMEOUT with iters_done = N - 1 and its history as
+ *                    above;
+ *   "sweep_refused"  the sweep's cooperative launch is refused, as where its
+ *                    blocks cannot all be resident, and a launch a pass takes
+ *                    its place (the same bits);
  *   "none" or ""     (or spec NULL) clears the injection.
  * The environment variable CT_FAULT, read once when the library is loaded,
  * sets the initial spec (a malformed value is reported on stderr and

@@ -7,8 +7,15 @@
 //                  solve stops with CT_ENONFINITE after N - 1 iterations;
 //   oom            allocations from the stream-ordered allocator are refused
 //                  as if it had failed (CT_ENOMEM); caller workspaces still work.
-// The NaN is an ordinary value written by a one-thread kernel; nothing
-// faults, traps or waits.
+//   sweep_stall:N  in iteration N's one-launch sweep over several blocks the
+//                  last one does not publish its sum and the others give up
+//                  after a few thousand reads (about a millisecond), so the
+//                  solve stops with CT_ETIMEOUT after N - 1 iterations;
+//   sweep_refused  the sweep's cooperative launch is refused, as where its
+//                  blocks cannot all be resident: single passes take its place.
+// The NaN is an ordinary value written by a one-thread kernel, and the silent
+// block returns like the others; nothing faults or traps, and no wait is longer
+// than usual.
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -40,25 +47,32 @@ bool parse_fault(const char *text, FaultSpec &out, std::string &canon, std::stri
             if (end == s.size()) break;
             continue;
         }
+        const size_t colon = item.find(':');
+        const std::string name = item.substr(0, colon);
         if (item == "oom") {
             out.oom = 1;
-        } else if (item.compare(0, 12, "nan_at_iter:") == 0) {
-            const char *num = item.c_str() + 12;
+        } else if (item == "sweep_refused") {
+            out.sweep_refused = 1;
+        } else if (colon != std::string::npos && (name == "nan_at_iter" || name == "sweep_stall")) {
+            const char *num = item.c_str() + colon + 1;
             char *stop = nullptr;
             const long v = std::strtol(num, &stop, 10);
             if (!*num || *stop || v < 1 || v > 1000000) {
-                err = "nan_at_iter needs an iteration number >= 1: '" + item + "'";
+                err = name + " needs an iteration number >= 1: '" + item + "'";
                 return false;
             }
-            out.nan_at_iter = int(v);
+            (name == "nan_at_iter" ? out.nan_at_iter : out.sweep_stall) = int(v);
         } else {
-            err = "unknown fault '" + item + "' (known: nan_at_iter:N, oom, none)";
+            err = "unknown fault '" + item + "' (known: nan_at_iter:N, oom, sweep_stall:N, sweep_refused, none)";
             return false;
         }
         if (end == s.size()) break;
     }
     if (out.nan_at_iter) canon = "nan_at_iter:" + std::to_string(out.nan_at_iter);
-    if (out.oom) canon += std::string(canon.empty() ? "" : ",") + "oom";
+    auto add = [&](const std::string &item) { canon += (canon.empty() ? "" : ",") + item; };
+    if (out.oom) add("oom");
+    if (out.sweep_stall) add("sweep_stall:" + std::to_string(out.sweep_stall));
+    if (out.sweep_refused) add("sweep_refused");
     return true;
 }
 

@@ -360,6 +360,8 @@ cudaError_t raise_dyn_smem(const void *func, size_t bytes);
 struct FaultSpec {
     int nan_at_iter = 0;   // iteration (>= 1) whose new vector gets a NaN; 0 = off
     int oom = 0;           // refuse stream-ordered allocations
+    int sweep_stall = 0;   // iteration (>= 1) in whose one-launch sweep a block stays silent; 0 = off
+    int sweep_refused = 0; // cooperative launches are refused
 };
 FaultSpec fault_spec();
 // Writes a NaN into v[0] when the spec names this iteration (1-based).

@@ -174,12 +174,12 @@ __device__ __forceinline__ void block_total2(const Acc<MODE> &a, const Acc<MODE>
 
 // The sums of n partials in a fixed order, valid in thread 0 afterwards (every
 // thread of the block calls it).  load(i, a, b) reads partial i and says
-// whether it is there yet; a partial that stays away for SLOT_POLLS reads ends
+// whether it is there yet; a partial that stays away for max_polls reads ends
 // the wait (false, in every thread).  Four warps add: few FP64 additions in
 // all, and a lane's reads go out together.
-constexpr int SLOT_POLLS = 1 << 22;
 template <typename F>
-__device__ __forceinline__ bool sum_partials(F load, int n, bool want_a, bool want_b, double &ta, double &tb)
+__device__ __forceinline__ bool sum_partials(F load, int n, bool want_a, bool want_b, double &ta, double &tb,
+                                             int max_polls = 1)
 {
     __shared__ double sum[2][4];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -197,7 +197,7 @@ __device__ __forceinline__ bool sum_partials(F load, int n, bool want_a, bool wa
                     a[k] = b[k] = 0.0;
                     if (i0 + 128 * k < n) all = load(i0 + 128 * k, a[k], b[k]) && all;
                 }
-            } while (!all && ++polls < SLOT_POLLS);
+            } while (!all && ++polls < max_polls);
             ok = ok && all;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -673,6 +673,12 @@ __global__ void givens_kernel(GivensArgs A)
 // resident); a wait that runs out marks the solve and ends the kernel.
 // ---------------------------------------------------------------------------
 constexpr unsigned long long SLOT_EMPTY = ~0ull;
+// How long a block waits for another's sum, in reads (2^22: a few seconds, against microseconds that
+// any wait takes between resident blocks), and a block that publishes none (-1; fault injection).
+struct SweepWait {
+    int max_polls = 1 << 22;
+    int silent = -1;
+};
 
 __device__ __forceinline__ bool slot_get(const unsigned long long *p, double &v)
 {
@@ -699,7 +705,7 @@ template <int MODE, typename TB, int ELEMS>
 __global__ void __launch_bounds__(SWEEP_NT)
     mgs_sweep_kernel(float *q, const TB *V, size_t ldv, int j, size_t len, double *h, double *first_ss,
                      double *last_ss, unsigned long long *slots, int set, const int *stop, const int *skip,
-                     SolverState *st, GivensArgs giv)
+                     SolverState *st, GivensArgs giv, SweepWait wait)
 {
     constexpr int G = 16 / sizeof(TB), NG = ELEMS / G;
     const int nb = gridDim.x;
@@ -767,7 +773,7 @@ __global__ void __launch_bounds__(SWEEP_NT)
         block_total2<SWEEP_NT, MODE>(dot, ss, want_dot, want_ss, ta, tb);
         if (nb > 1) {
             unsigned long long *out = mine + (i % 3) * 2 * nb;
-            if (threadIdx.x == 0) {
+            if (threadIdx.x == 0 && int(blockIdx.x) != wait.silent) {
                 if (want_dot) slot_put(out, ta);
                 if (want_ss) slot_put(out + nb, tb);
             }
@@ -784,7 +790,7 @@ __global__ void __launch_bounds__(SWEEP_NT)
             const bool ok = sum_partials([&](int b, double &va, double &vb) {
                 const bool ga = !want_dot || slot_get(in + b, va), gb = !want_ss || slot_get(in + nb + b, vb);
                 return ga && gb;
-            }, nb, want_dot, want_ss, ta, tb);
+            }, nb, want_dot, want_ss, ta, tb, wait.max_polls);
             if (!ok) {
                 if (threadIdx.x == 0) st->status = ST_TIMEOUT;
                 return;
@@ -1198,14 +1204,22 @@ static cudaError_t launch_sweep(GmresWs &w, float *q, int j, double *hcol, size_
     const TB *V = static_cast<const TB *>(w.V);
     GivensArgs g{};
     if (giv) g = *giv;
-    void *args[] = {&q, &V, &w.ldv, &j, &len, &hcol, &first_ss, &last_ss, &w.slots, &set, &stop, &skip, &w.st, &g};
+    SweepWait wait;
+    void *args[] = {&q,    &V,   &w.ldv, &j,    &len,  &hcol, &first_ss, &last_ss, &w.slots,
+                    &set, &stop, &skip,  &w.st, &g,    &wait};
     ProfScope prof(PK_MGS, s);
     const unsigned blocks = sweep_blocks(len);
     if (blocks == 1) {   // nobody to wait for
         auto *kernel = len <= SWEEP_NT * 8 ? mgs_sweep_kernel<MODE, TB, 8> : mgs_sweep_kernel<MODE, TB, 16>;
-        kernel<<<1, SWEEP_NT, 0, s>>>(q, V, w.ldv, j, len, hcol, first_ss, last_ss, w.slots, set,
-                                                              stop, skip, w.st, g);
+        kernel<<<1, SWEEP_NT, 0, s>>>(q, V, w.ldv, j, len, hcol, first_ss, last_ss, w.slots, set, stop, skip, w.st, g,
+                                      wait);
         return cudaGetLastError();
+    }
+    const FaultSpec fault = fault_spec();
+    if (fault.sweep_refused) return cudaErrorCooperativeLaunchTooLarge;
+    if (fault.sweep_stall == j + 1) {
+        wait.max_polls = 1 << 12;
+        wait.silent = int(blocks) - 1;
     }
     const void *kernel = len <= size_t(blocks) * SWEEP_NT * 16
                              ? reinterpret_cast<const void *>(mgs_sweep_kernel<MODE, TB, 16>)
@@ -1235,6 +1249,9 @@ static cudaError_t device_sweep(GmresWs &w, int mode, float *q, int j, double *h
             e != cudaErrorNotSupported)
             return e;
         cudaGetLastError();
+        // the launch that was to empty the other set's slots did not run: a later one must not find them full
+        e = cudaMemsetAsync(w.slots, 0xff, slots_count() * sizeof(unsigned long long), s);
+        if (e != cudaSuccess) return e;
     }
     cudaError_t e = cudaSuccess;
     for (int i = 0; i <= j + 1 && e == cudaSuccess; ++i)
