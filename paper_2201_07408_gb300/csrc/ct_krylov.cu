@@ -995,10 +995,8 @@ static void take_op_bufs(Arena &ar, const GeomDev &g, OpBufs &b, bool need_t, bo
 // out_vol = B sino.  `sino` is a plain sinogram, scaled by (*scale) first when
 // given (and normalised in place when `normalize`).
 static cudaError_t apply_B(const GeomDev &g, int b_kind, float *sino, const double *scale, bool normalize,
-                           OpBufs &b, float *out_vol, const int *stop, cudaStream_t st,
-                           float *scratch_vec /* n floats for A^T zeroing, unused otherwise */)
+                           OpBufs &b, float *out_vol, const int *stop, cudaStream_t st)
 {
-    (void)scratch_vec;
     cudaError_t e = cudaSuccess;
     if (b_kind == CT_B_UN) {
         e = launch_pad_sino(g, sino, scale, normalize, b.ypad, stop, st);
@@ -1340,7 +1338,7 @@ static cudaError_t ba_start(const GeomDev &g, GmresWs &w, const float *b, int km
     if (e == cudaSuccess)
         e = cudaMemsetAsync(w.ob.ypad, 0, padded_sino_floats(g) * sizeof(float), s);
     if (e == cudaSuccess)
-        e = apply_B(g, o.b_kind, const_cast<float *>(b), nullptr, false, w.ob, w.q, nullptr, s, nullptr);
+        e = apply_B(g, o.b_kind, const_cast<float *>(b), nullptr, false, w.ob, w.q, nullptr, s);
     if (e == cudaSuccess)
         e = mgs_pass(o.dot_mode, w.q, nullptr, nullptr, nullptr, n, w.partials, &w.st->counter, nullptr,
                      &w.st->sumsq, nullptr, nullptr, s);
@@ -1377,7 +1375,7 @@ static cudaError_t ba_iteration(const GeomDev &g, GmresWs &w, int j, int kmax, s
         if (e == cudaSuccess) e = launch_voxel_B(g, w.ob.ypad, w.q, stop, s, QUAD_CORNERS);
     } else {
         e = launch_project_A(g, w.ob.Xc, w.ob.Yc, w.ob.t, plain_layout(g), stop, s);
-        if (e == cudaSuccess) e = apply_B(g, o.b_kind, w.ob.t, nullptr, false, w.ob, w.q, stop, s, nullptr);
+        if (e == cudaSuccess) e = apply_B(g, o.b_kind, w.ob.t, nullptr, false, w.ob, w.q, stop, s);
     }
     if (e == cudaSuccess) e = arnoldi_orthogonalise(w, w.q, j, kmax, n, o, s, sg);
     return e;
@@ -1540,7 +1538,7 @@ static ct_status abgmres(const ct_geom *geom, const float *b, int k, float *x, d
         NvtxRange iter_range("AB-GMRES iteration");
         float *vj = Vf + size_t(j) * w.ldv;
         float *q = Vf + size_t(j + 1) * w.ldv;
-        e = apply_B(g, o.b_kind, vj, &w.st->inv_norm, true, w.ob, w.tvol, stop, s, nullptr);
+        e = apply_B(g, o.b_kind, vj, &w.st->inv_norm, true, w.ob, w.tvol, stop, s);
         if (e == cudaSuccess) e = launch_plane_copies(g, w.tvol, nullptr, nullptr, w.ob.Xc, w.ob.Yc, stop, s);
         if (e == cudaSuccess) e = launch_project_A(g, w.ob.Xc, w.ob.Yc, q, plain_layout(g), stop, s);
         if (e == cudaSuccess) e = arnoldi_orthogonalise(w, q, j, k, m, o, s);
@@ -1549,7 +1547,7 @@ static ct_status abgmres(const ct_geom *geom, const float *b, int k, float *x, d
     // u = V y (data space) into the last basis slot, then x = B u
     float *u = Vf + size_t(k) * w.ldv;
     if (e == cudaSuccess) e = combine(Vf, w.ldv, k, m, w.y, &w.st->iters, u, s);
-    if (e == cudaSuccess) e = apply_B(g, o.b_kind, u, nullptr, false, w.ob, x, nullptr, s, nullptr);
+    if (e == cudaSuccess) e = apply_B(g, o.b_kind, u, nullptr, false, w.ob, x, nullptr, s);
     if (e != cudaSuccess) {
         arena_close(ar);
         return cuda_error(e, "ct_abgmres_solve launch");
@@ -1616,12 +1614,11 @@ __global__ void scale_vec_kernel(float *__restrict__ v, size_t len, const double
 }
 
 // out_sino = B^T vol (plain layout); b_kind B_UN or B_FBP
-static cudaError_t apply_Bt(const GeomDev &g, int b_kind, const float *vol, float *t, float *tf, float *bt_acc,
-                            float *out, const int *stop, cudaStream_t s)
+static cudaError_t apply_Bt(const GeomDev &g, int b_kind, const float *vol, float *t, float *bt_acc, float *out,
+                            const int *stop, cudaStream_t s)
 {
     cudaError_t e = launch_voxel_Bt(g, bt_scatter(g), vol, b_kind == CT_B_FBP ? t : out, bt_acc, stop, s);
     if (e == cudaSuccess && b_kind == CT_B_FBP) e = launch_ramp(g, t, out, plain_layout(g), true, stop, s);
-    (void)tf;
     return e;
 }
 
@@ -1662,14 +1659,14 @@ static ct_status bagmres_vjp(const ct_geom *geom, const float *gx, int k, float 
             scale_vec_kernel<<<vb, RED_BLOCK, 0, s>>>(vj, n, &gm.st->inv_norm, stop);
             e = cudaGetLastError();
         }
-        if (e == cudaSuccess) e = apply_Bt(g, o.b_kind, vj, w.t, w.tf, w.bt_acc, sino, stop, s);
+        if (e == cudaSuccess) e = apply_Bt(g, o.b_kind, vj, w.t, w.bt_acc, sino, stop, s);
         if (e == cudaSuccess) e = launch_project_At(g, at_scatter(g), sino, q, w.acc, stop, s);
         if (e == cudaSuccess) e = arnoldi_orthogonalise(gm, q, j, k, n, o, s);
     }
     if (e == cudaSuccess) e = backsolve(gm.R, gm.g, gm.y, &gm.st->iters, k, s);
     float *z = Vf + size_t(k) * gm.ldv;
     if (e == cudaSuccess) e = combine(Vf, gm.ldv, k, n, gm.y, &gm.st->iters, z, s);
-    if (e == cudaSuccess) e = apply_Bt(g, o.b_kind, z, w.t, w.tf, w.bt_acc, gb, nullptr, s);
+    if (e == cudaSuccess) e = apply_Bt(g, o.b_kind, z, w.t, w.bt_acc, gb, nullptr, s);
     if (e != cudaSuccess) {
         arena_close(ar);
         return cuda_error(e, "ct_bagmres_vjp launch");
@@ -1735,7 +1732,7 @@ static ct_status cgls(const ct_geom *geom, const float *b, int k, float *x, doub
     // rr = ||r||^2, s = B r, gamma = ||s||^2, p = s
     if (e == cudaSuccess)
         e = mgs_pass(1, w.r, nullptr, nullptr, nullptr, m, w.partials, ctr, nullptr, &st->rr, nullptr, nullptr, s);
-    if (e == cudaSuccess) e = apply_B(g, o.b_kind, w.r, nullptr, false, w.ob, w.s, nullptr, s, nullptr);
+    if (e == cudaSuccess) e = apply_B(g, o.b_kind, w.r, nullptr, false, w.ob, w.s, nullptr, s);
     if (e == cudaSuccess)
         e = mgs_pass(1, w.s, nullptr, nullptr, nullptr, n, w.partials, ctr, nullptr, &st->gamma, nullptr, nullptr, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(w.p, w.s, n * sizeof(float), cudaMemcpyDeviceToDevice, s);
@@ -1773,7 +1770,7 @@ static ct_status cgls(const ct_geom *geom, const float *b, int k, float *x, doub
             }
         }
         // s = B r ; gamma_new = ||s||^2 ; p = s + (gamma_new/gamma) p ; gamma = gamma_new
-        if (e == cudaSuccess) e = apply_B(g, o.b_kind, w.r, nullptr, false, w.ob, w.s, stop, s, nullptr);
+        if (e == cudaSuccess) e = apply_B(g, o.b_kind, w.r, nullptr, false, w.ob, w.s, stop, s);
         if (e == cudaSuccess)
             e = mgs_pass(1, w.s, nullptr, nullptr, nullptr, n, w.partials, ctr, nullptr, &st->gamma_new, stop,
                          nullptr, s);

@@ -28,15 +28,6 @@
 
 namespace ct {
 
-struct RaySetup {
-    int xdom;      // 1: planes along x
-    int p0, p1;    // inclusive plane range that can hold nonzero samples
-    float ca;      // (N_a - 1)/2
-    float fbc, gb; // in-plane fractional index at the central plane, slope per plane
-    float fzc, gz; // z fractional index at the central plane, slope per plane
-    float weight;  // vox |d| / |d_a|
-};
-
 // Narrows [p0, p1] to the planes whose f(p) = fc + (p - ca) g lies in
 // [lo - 0.5, hi + 0.5].  Every sample with f in [lo, hi) stays inside; every
 // kept sample has floor(f) in [lo - 1, hi], inside the zero border.
@@ -97,41 +88,6 @@ __device__ __forceinline__ void clip_planes_run(float fc_f, float g_f, float fc_
     hull(a0, a1, b0, b1, w0, w1);
     p0 = max(p0, max(u0, w0));
     p1 = min(p1, min(u1, w1));
-}
-
-__device__ __forceinline__ RaySetup ray_setup(const GeomDev &g, int s, int iv, int iu)
-{
-    const float4 *vp = reinterpret_cast<const float4 *>(g.viewA + s);
-    const float4 a = __ldg(vp), b = __ldg(vp + 1);
-    // a = (dx0, dxu, dy0, dyu), b = (dzv, crossu, sx, sy)
-    const float u = (float(iu) - g.cu) * g.du;
-    const float v = (float(iv) - g.cv) * g.dv;
-    const float dx = fmaf(u, a.y, a.x);
-    const float dy = fmaf(u, a.w, a.z);
-    const float dz = v * b.x;
-    const float cross = u * b.y;
-    RaySetup r;
-    r.xdom = fabsf(dx) >= fabsf(dy);
-    const float da = r.xdom ? dx : dy;
-    const float db = r.xdom ? dy : dx;
-    const float Sa = r.xdom ? b.z : b.w;
-    const int Na = r.xdom ? g.nx : g.ny;
-    const int Nb = r.xdom ? g.ny : g.nx;
-    const float cb = r.xdom ? g.cy : g.cx;
-    r.ca = r.xdom ? g.cx : g.cy;
-    const float inv_da = 1.0f / da;
-    r.gb = db * inv_da;
-    // x-dominant: y(c) = (c d_y - cross)/d_x ; y-dominant: x(c) = (c d_x + cross)/d_y
-    const float cterm = cross * inv_da * g.inv_vox;
-    r.fbc = r.xdom ? cb - cterm : cb + cterm;
-    r.gz = dz * inv_da;
-    r.fzc = fmaf(-Sa * g.inv_vox, r.gz, g.cz);
-    r.weight = g.vox * sqrtf(fmaf(dx, dx, fmaf(dy, dy, dz * dz))) * fabsf(inv_da);
-    r.p0 = 0;
-    r.p1 = Na - 1;
-    clip_planes(r.fbc, r.gb, -1.0f, float(Nb), r.ca, Na, r.p0, r.p1);
-    clip_planes(r.fzc, r.gz, -1.0f, float(g.nz), r.ca, Na, r.p0, r.p1);
-    return r;
 }
 
 // ---------------------------------------------------------------------------
