@@ -219,10 +219,10 @@ def aggregate_over_ranks(elapsed_s, iters, world, device=None):
 NCU_TRAFFIC = {
     # (kernel, storage, workload): (bytes per launch, source file,
     # source_code_sha of that file and ct_internal.cuh at capture time)
-    ("voxel_B", "f32", "cone_256"): (1211157504 + 80132096, "ct_backproject.cu",
-                                     "80ea43cf7db79703c3a6cf2f4ea2502d846665209df26d7877f6efafcc9137c5"),
-    ("joseph_A", "f32", "cone_256"): (412163840 + 137549056, "ct_project.cu",
-                                      "1433cf8b9c78380fe3e9b597dceeb3620d93fa4165fee657d0563f2d51c29e79"),
+    ("voxel_B", "f32", "cone_256"): (1214532000 + 79516672, "ct_backproject.cu",
+                                     "475d1138d9d6eb87c9690b9ea19e4ce0fe0dbddb70fe9eb945ed42b233cfd96d"),
+    ("joseph_A", "f32", "cone_256"): (420552704 + 137946368, "ct_project.cu",
+                                      "df6f51d1c6cb16f86ff583c136b41a38048844981f7817959e41bf34b73256cc"),
 }
 
 
@@ -232,9 +232,9 @@ NCU_TRAFFIC = {
 # at least 4 for B's 128-bit warp loads, 1 for A's 32-bit ones).  Keyed like NCU_TRAFFIC.
 NCU_L1 = {
     ("voxel_B", "f32", "cone_256"): ({"data_pipe_frac": 0.797, "passes_per_request": 5.34}, "ct_backproject.cu",
-                                     "80ea43cf7db79703c3a6cf2f4ea2502d846665209df26d7877f6efafcc9137c5"),
-    ("joseph_A", "f32", "cone_256"): ({"data_pipe_frac": 0.452, "passes_per_request": 1.39}, "ct_project.cu",
-                                      "1433cf8b9c78380fe3e9b597dceeb3620d93fa4165fee657d0563f2d51c29e79"),
+                                     "475d1138d9d6eb87c9690b9ea19e4ce0fe0dbddb70fe9eb945ed42b233cfd96d"),
+    ("joseph_A", "f32", "cone_256"): ({"data_pipe_frac": 0.520, "passes_per_request": 1.38}, "ct_project.cu",
+                                      "df6f51d1c6cb16f86ff583c136b41a38048844981f7817959e41bf34b73256cc"),
 }
 
 

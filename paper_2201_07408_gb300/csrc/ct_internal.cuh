@@ -334,9 +334,8 @@ size_t bt_scratch_floats(const GeomDev &g, Scatter how);
 cudaError_t launch_voxel_Bt(const GeomDev &g, Scatter how, const float *x, float *y, float *acc, const int *stop,
                             cudaStream_t st);
 
-// While what they add to stays in L2, the scatters (A^T, B_un^T) are bound by the
-// rate of reduction requests, about 2.8e10 warp requests a second whatever each
-// carries.  Their contributions
+// The scatters (A^T, B_un^T) wait for L2 to take their reductions, and while what
+// they add to stays in L2, fewer requests are faster.  Their contributions
 // come in pairs of neighbouring elements, so an accumulator is kept twice, the
 // second copy shifted by one element: every pair is 8-byte aligned in one of
 // them and goes as one request.  Element e is acc[e] + acc[odd + e + 1].

@@ -433,8 +433,8 @@ constexpr unsigned FLOOR_MAGIC_BITS = 0x4b400000u;
 // clamp (a detector taller than the slices) 4 planes at a time need more registers
 // than there are: 74 x 143 x 24, 21 views 93 us against 83 by 3 (plain walk 82), 31 x
 // 68 x 42, 18 views 52 against 45 (47); by 2, 5 % slower on few views.  Left after it:
-// 12.1 instructions a sample (16.8 before), the FMA pipe 53 % and issue 56 %
-// busy, the rest latency of the row loads (a third of them miss L1).
+// 11.9 instructions a sample (16.8 before), the FMA pipe 52-55 % and issue 55-58
+// % busy, the rest latency of the row loads (a third of them miss L1).
 constexpr int kAPlaneUnroll = 4;
 constexpr int kAPlaneUnrollClampedBF = 3;
 constexpr int kAMinBlocks = 4;
