@@ -498,8 +498,12 @@ static cudaError_t mgs_pass_t(float *q, const TB *vprev, const double *hprev, co
         return cudaGetLastError();
     }
     // a thread's two groups a step put six 16-byte loads in flight, and 4 blocks an SM of them cover the memory's
-    // latency (256^3: 32.8 us a pass; 2, 6 and 8 blocks 38.3, 39.2, 35.8)
-    const unsigned blocks = unsigned(std::min((len / G + RED_BLOCK - 1) / RED_BLOCK, size_t(num_sms()) * 4));
+    // latency (256^3, compensated: 34.4 us a pass; 5, 6 and 8 blocks 42.3, 39.2, 37.9); a bf16 basis moves half the
+    // bytes at as many operations, and the compensated sums of 8 elements a group then take 6 (36.0, 32.7, 31.4,
+    // 35.0 us with 4, 5, 6, 8; plain sums 28.7 with 4); plain sums over FP32, 5 (37.4, 35.7, 43.9, 40.1)
+    constexpr int BLOCKS_PER_SM = MODE == 0 ? (G == 8 ? 6 : 4) : (G == 8 ? 4 : 5);
+    const unsigned blocks = unsigned(std::min((len / G + RED_BLOCK - 1) / RED_BLOCK,
+                                              size_t(num_sms()) * BLOCKS_PER_SM));
     mgs_pass_kernel<MODE, TB, RED_BLOCK><<<blocks, RED_BLOCK, 0, st>>>(q, vprev, hprev, vcur, len, vec, partials,
                                                                        counter, out_dot, out_sumsq, stop, skip);
     return cudaGetLastError();

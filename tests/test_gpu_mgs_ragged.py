@@ -55,6 +55,24 @@ def test_sweep_coefficients(ct, n, offset, mode, tol):
     assert np.isnan(rest).all()   # nothing written past q
 
 
+@pytest.mark.parametrize("mode", [0, 1])
+@pytest.mark.parametrize("vol", ["f32", "bf16"])
+def test_long_vectors_on_a_device_and_a_host_basis(ct, vol, mode):
+    """Vectors past the one-launch sweep, ragged: both bases take the same passes, bit for bit."""
+    spec = ci._cone("cone_143x139x131", 0, 0.9, 3, 40, 20, 7.0, nxyz=(143, 139, 131))
+    g = ct.Geometry.from_spec(spec, vol_dtype=vol)
+    b = torch.from_numpy(ci.random_vector(spec.m, seed=84).astype(np.float32)).cuda()
+    out = []
+    for basis in ("device", "host"):
+        st = ct.GmresState(g, 3, basis, ct.make_opts(b_kind="un", dot_mode=mode))
+        st.start(b)
+        x = torch.empty(spec.vol_shape, device="cuda")
+        out.append((st.extend(3, x).resid.copy(), x))
+        st.close()
+    assert np.array_equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+    assert np.all(np.diff(out[0][0]) <= 1e-12 * out[0][0][0])
+
+
 @pytest.mark.parametrize("vol", ["f32", "bf16"])
 @pytest.mark.parametrize("nxyz", [(15, 13, 11), (23, 18, 7), (14, 15, 9)], ids=str)
 def test_ragged_solve(ct, nxyz, vol):
