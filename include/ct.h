@@ -109,8 +109,9 @@ typedef struct {
     int b_kind;              /* ct_b_kind; default CT_B_UN */
     double tol;              /* stop when resid[j] <= tol*resid[0]; 0 = run all k */
     int dot_mode;            /* Arnoldi inner products: 0 = compensated FP32 accumulation (FMA
-                                two-product + two-sum) then FP64 reduction (default),
-                                1 = plain FP32 FMA accumulation then FP64 reduction */
+                                two-product + two-sum; default), 1 = plain FP32 FMA accumulation;
+                                either is summed in FP32 triples that keep the rounding errors
+                                within a block, and in FP64 between blocks */
     int reorth;              /* 0 = one MGS sweep (default), 1 = a second sweep when the
                                 norm drops below 1/sqrt(2) of its value before the sweep */
     int record_data_resid;   /* CGLS only: resid holds the recomputed ||b - A x_j|| */
